@@ -364,7 +364,8 @@ vrt_status vrt_set_stream(vrt_grid g, void* cuda_stream);
 /* Stage durations of the last frame in milliseconds (waits), measured with
  * CUDA events on the grid's stream while VRT_OPT_STAGE_TIMING is on. Order:
  * 0 ingest, 1 voxelize pass 1, 2 mips, 3 cull marks, 4 scan, 5 voxelize
- * pass 2, 6 trace, 7 repair rounds (list + re-trace), 8 voxel-space shading.
+ * pass 2, 6 trace, 7 repair rounds (list + re-trace), 8 voxel-space shading or
+ * the per-hit AO of an opaque trace.
  * Stages that did not run since the last vrt_voxelize read -1. Writes
  * min(n, 9) entries. */
 #define VRT_N_STAGES 9

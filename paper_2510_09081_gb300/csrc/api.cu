@@ -862,6 +862,11 @@ vrt_status vrt_trace(vrt_grid g, const vrt_camera* cam, const vrt_render_params*
     }
     stage_mark(g, ST_REPAIR, 1);
   }
+  if (K == 1 && a.ao == 1) {
+    stage_mark(g, ST_SHADE, 0);
+    g->launches += launch_shade_hits(a, g->stream);
+    stage_mark(g, ST_SHADE, 1);
+  }
   if (g->trace_counters) {
     VRT_CUDA(g, cudaMemsetAsync((char*)g->st + offsetof(DevStatus, tr_u_entries), 0,
                                 3 * sizeof(unsigned long long), g->stream));

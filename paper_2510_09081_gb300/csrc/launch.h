@@ -120,6 +120,9 @@ int launch_cull(const GridDev& g, const HostCamera& cam, float alpha, uint8_t* e
                 uint8_t* btmp, uint8_t* cdist, float* emean, float depth_max, uint32_t* occq,
                 unsigned long long occq_cap, cudaStream_t s);
 int launch_trace(const TraceArgs& a, int K, cudaStream_t s);
+// Cone AO of the hits an opaque trace (K = 1, a.ao = 1) and its repair rounds
+// left in a.rgba.
+int launch_shade_hits(const TraceArgs& a, cudaStream_t s);
 // Instrumented trace: the set bits of the three touch bitmaps into
 // st->tr_u_entries, tr_u_vertices, tr_u_voxels (which the caller cleared).
 int launch_touch_count(const uint32_t* list_bits, size_t list_words, const uint32_t* vert_bits,

@@ -30,9 +30,9 @@
 //    C += T alpha c, T *= 1 - alpha, until T < 1e-4 (ground-truth order).
 // Shading: colour = |unit tangent| per component times either cone-traced
 // ambient occlusion per hit when enabled (six cones over the occupancy
-// pyramid; a cone's occlusion is 1 - prod(1 - s_k) over its samples, so the
-// samples of one hit can be taken by different lanes), or one trilinear sample
-// of the voxel-space shading field at the hit (Sec. 3.4, built by shade.cu).
+// pyramid; the hits of an opaque trace are shaded by a kernel of their own at
+// the end), or one trilinear sample of the voxel-space shading field at the hit
+// (Sec. 3.4, built by shade.cu).
 //
 // Culling validation: a ray that reaches a voxel holding segments but no list
 // queues the voxel (deduplicated by a bitmap), marches on as if the voxel were
@@ -106,9 +106,15 @@ __device__ __forceinline__ float shade_at(const TraceArgs& A, float3 P) {
   return acc;
 }
 
-// Per-hit shading factor: A.ao = 1 cone AO at P, 2 the voxel-space field.
-__device__ __noinline__ float hit_shade(const TraceArgs& A, float3 P) {
-  return A.ao == 2 ? shade_at(A, P) : ao_lane(A, P);
+// Shading factor of a transparent hit at P. The trace kernels are instantiated
+// with AO for cone AO per hit and without it for no shading or the voxel-space
+// field: a call to the AO code anywhere in a kernel costs all its rays
+// registers (bundles at alpha 0.3 without AO 1% slower, small random walks 3%).
+__device__ __noinline__ float field_shade(const TraceArgs& A, float3 P) { return shade_at(A, P); }
+template <bool AO>
+__device__ __forceinline__ float hit_shade(const TraceArgs& A, float3 P) {
+  if constexpr (AO) return ao_lane(A, P);
+  else return field_shade(A, P);
 }
 
 __device__ __forceinline__ float3 tangent_colour(const TraceArgs& A, uint32_t id) {
@@ -314,17 +320,21 @@ __device__ int advance(const TraceArgs& A, Ray& R, int budget) {
   return -1;  // budget used up, ray still on its way
 }
 
-__device__ void init_ray(const TraceArgs& A, Ray& R, int px, int py, bool valid) {
-  const CamDev& c = A.cam;
+// Origin and unit direction of pixel (px, py)'s ray.
+__device__ __forceinline__ void pixel_ray(const CamDev& c, int px, int py, float3& o, float3& d) {
   const float fx = (float)px + 0.5f, fy = (float)py + 0.5f;
   if (c.ortho) {
-    R.o = c.o0 + fx * c.ox + fy * c.oy;
-    R.d = c.d0;
+    o = c.o0 + fx * c.ox + fy * c.oy;
+    d = c.d0;
   } else {
-    R.o = c.o0;
-    const float3 d = c.d0 + fx * c.dx + fy * c.dy;
-    R.d = (1.0f / sqrtf(dot3(d, d))) * d;
+    o = c.o0;
+    const float3 v = c.d0 + fx * c.dx + fy * c.dy;
+    d = (1.0f / sqrtf(dot3(v, v))) * v;
   }
+}
+
+__device__ void init_ray(const TraceArgs& A, Ray& R, int px, int py, bool valid) {
+  pixel_ray(A.cam, px, py, R.o, R.d);
   R.C[0] = R.C[1] = R.C[2] = 0.0f;
   R.T = 1.0f;
   R.first_id = -1;
@@ -380,8 +390,26 @@ __device__ void resume_ray(const TraceArgs& A, Ray& R) {
   R.tcur = s1.w;
 }
 
+// An opaque ray ends at its nearest hit. With cone AO its pixel carries the hit
+// (segment id and depth) to k_shade_hits, which writes the colour; otherwise it
+// is shaded here.
+__device__ __forceinline__ void opaque_hit(const TraceArgs& A, Ray& R, uint32_t id, float t) {
+  if (A.ao == 1) {
+    R.C[0] = __uint_as_float(id);
+    R.C[1] = t;
+  } else {
+    float3 c = tangent_colour(A, id);
+    if (A.ao) c = shade_at(A, R.o + t * R.d) * c;
+    R.C[0] = A.alpha * c.x; R.C[1] = A.alpha * c.y; R.C[2] = A.alpha * c.z;
+  }
+  R.T *= (1.0f - A.alpha);
+  R.first_id = (int)id;
+  R.first_t = t;
+  R.active = false;
+}
+
 // The warp processes the pending voxel of lane `L`.
-template <bool OPAQUE, bool COUNT, bool KEY16>
+template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
 __device__ void process_voxel(const TraceArgs& A, Ray& R, int L) {
   const int lane = threadIdx.x & 31;
   const float3 o = shfl3(R.o, L), d = shfl3(R.d, L);
@@ -411,15 +439,7 @@ __device__ void process_voxel(const TraceArgs& A, Ray& R, int L) {
     if (best != ~0ull) {
       const uint32_t id = (uint32_t)(best & 0xffffffffu);
       const float t = hit_depth<KEY16>(A, best, o, d);
-      float3 c = tangent_colour(A, id);
-      if (A.ao) c = (A.ao == 2 ? shade_at(A, o + t * d) : ao_warp(A, o + t * d)) * c;
-      if (lane == L) {
-        R.C[0] = A.alpha * c.x; R.C[1] = A.alpha * c.y; R.C[2] = A.alpha * c.z;
-        R.T *= (1.0f - A.alpha);
-        R.first_id = (int)id;
-        R.first_t = t;
-        R.active = false;
-      }
+      if (lane == L) opaque_hit(A, R, id, t);
     }
     return;
   }
@@ -483,7 +503,7 @@ __device__ void process_voxel(const TraceArgs& A, Ray& R, int L) {
         const uint32_t id = (uint32_t)(mine & 0xffffffffu);
         tq = hit_depth<KEY16>(A, mine, o, d);
         c = tangent_colour(A, id);
-        if (A.ao) c = hit_shade(A, o + tq * d) * c;
+        if (A.ao) c = hit_shade<AO>(A, o + tq * d) * c;
       }
       // accumulate in key order
       for (int q = 0; q < n_out; ++q) {
@@ -532,7 +552,7 @@ __device__ void process_voxel(const TraceArgs& A, Ray& R, int L) {
 // ray, sorted and composited by the ray's own lane afterwards). A transparent
 // ray with more hits in the voxel keeps its voxel pending for the whole-warp
 // path, which starts it again from scratch.
-template <bool OPAQUE, bool COUNT, bool KEY16>
+template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
 __device__ void process_flat(const TraceArgs& A, Ray& R) {
   extern __shared__ unsigned long long s_key[];  // [kRayKeys][kTraceThreads]
   __shared__ float4 s_ray[2][kTraceThreads];      // (o, t_enter), (d, t_exit)
@@ -712,14 +732,7 @@ __device__ void process_flat(const TraceArgs& A, Ray& R) {
     const unsigned long long best = s_best[tid];
     if (best != ~0ull) {
       const uint32_t id = (uint32_t)(best & 0xffffffffu);
-      const float t = hit_depth<KEY16>(A, best, R.o, R.d);
-      float3 c = tangent_colour(A, id);
-      if (A.ao) c = hit_shade(A, R.o + t * R.d) * c;
-      R.C[0] = A.alpha * c.x; R.C[1] = A.alpha * c.y; R.C[2] = A.alpha * c.z;
-      R.T *= (1.0f - A.alpha);
-      R.first_id = (int)id;
-      R.first_t = t;
-      R.active = false;
+      opaque_hit(A, R, id, hit_depth<KEY16>(A, best, R.o, R.d));
     }
     R.pending = false;
     if (R.t1 < 0.0f) R.active = false;
@@ -747,7 +760,7 @@ __device__ void process_flat(const TraceArgs& A, Ray& R) {
     const uint32_t id = (uint32_t)(kq & 0xffffffffu);
     const float t = hit_depth<KEY16>(A, kq, R.o, R.d);
     float3 c = tangent_colour(A, id);
-    if (A.ao) c = hit_shade(A, R.o + t * R.d) * c;
+    if (A.ao) c = hit_shade<AO>(A, R.o + t * R.d) * c;
     const float w = R.T * A.alpha;
     R.C[0] = fmaf(w, c.x, R.C[0]);
     R.C[1] = fmaf(w, c.y, R.C[1]);
@@ -772,7 +785,7 @@ __device__ __forceinline__ void lap(unsigned long long& c, long long& t) {
   }
 }
 
-template <bool OPAQUE, bool COUNT, bool KEY16>
+template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
 __device__ void trace_warp(const TraceArgs& A, Ray& R) {
   const int lane = threadIdx.x & 31;
   long long t = COUNT ? clock64() : 0;
@@ -793,14 +806,14 @@ __device__ void trace_warp(const TraceArgs& A, Ray& R) {
     if (!pend && !walk) break;
     if (walk && 4 * __popc(pend) < __popc(pend | walk)) continue;
     lap<COUNT>(R.cyc[0], t);
-    process_flat<OPAQUE, COUNT, KEY16>(A, R);
+    process_flat<OPAQUE, COUNT, KEY16, AO>(A, R);
     lap<COUNT>(R.cyc[1], t);
     // long lists: the whole warp on one list at a time
     unsigned pm = __ballot_sync(FULL, R.pending);
     while (pm) {
       const int L = __ffs(pm) - 1;
       pm &= pm - 1;
-      process_voxel<OPAQUE, COUNT, KEY16>(A, R, L);
+      process_voxel<OPAQUE, COUNT, KEY16, AO>(A, R, L);
       if (lane == L) {
         R.pending = false;
         if (R.t1 < 0.0f) R.active = false;
@@ -857,8 +870,8 @@ __device__ __forceinline__ void finish(const TraceArgs& A, const Ray& R, bool va
 // together at the end. Measured faster than persistent refilling here, since
 // the tile's rays share lists. The tile shape is a tuned parameter (default
 // 4 x 8, measured slightly faster than 8 x 4 or 16 x 2 on the bundles frame).
-template <bool OPAQUE, bool COUNT, bool KEY16, int TW>
-__global__ void __launch_bounds__(kTraceThreads) k_trace_tile(TraceArgs A) {
+template <bool OPAQUE, bool COUNT, bool KEY16, bool AO, int TW>
+__global__ void __launch_bounds__(kTraceThreads, COUNT ? 1 : 4) k_trace_tile(TraceArgs A) {
   constexpr int TH = 32 / TW;
   const int lane = threadIdx.x & 31;
   const int warp = threadIdx.x >> 5;
@@ -869,7 +882,7 @@ __global__ void __launch_bounds__(kTraceThreads) k_trace_tile(TraceArgs A) {
   R.cyc[0] = R.cyc[1] = R.cyc[2] = R.cyc[3] = 0;
   R.pix = valid ? (uint32_t)(py * A.cam.width + px) : 0u;
   init_ray(A, R, px, py, valid);
-  trace_warp<OPAQUE, COUNT, KEY16>(A, R);
+  trace_warp<OPAQUE, COUNT, KEY16, AO>(A, R);
   finish<COUNT>(A, R, valid);
 }
 
@@ -891,8 +904,8 @@ __device__ __forceinline__ void write_pixel(const TraceArgs& A, const Ray& R) {
 // atomic per refill). Work item w of the image is pixel (w mod 32) of the
 // (w / 32)-th 8x4 tile, so a full refill is a coherent tile; in the repair
 // re-trace, item w is the w-th queued pixel.
-template <bool OPAQUE, bool COUNT, bool KEY16>
-__global__ void __launch_bounds__(kTraceThreads) k_trace(TraceArgs A) {
+template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
+__global__ void __launch_bounds__(kTraceThreads, COUNT ? 1 : (OPAQUE ? 5 : 4)) k_trace(TraceArgs A) {
   const int lane = threadIdx.x & 31;
   const uint32_t W = (uint32_t)A.cam.width, H = (uint32_t)A.cam.height;
   const uint32_t tiles_x = (W + 7) / 8;
@@ -956,14 +969,14 @@ __global__ void __launch_bounds__(kTraceThreads) k_trace(TraceArgs A) {
       if (!R.pending) R.active = false;
     }
     lap<COUNT>(R.cyc[0], tclk);
-    process_flat<OPAQUE, COUNT, KEY16>(A, R);
+    process_flat<OPAQUE, COUNT, KEY16, AO>(A, R);
     lap<COUNT>(R.cyc[1], tclk);
     // long lists: the whole warp on one list at a time
     unsigned pm = __ballot_sync(FULL, R.pending);
     while (pm) {
       const int L = __ffs(pm) - 1;
       pm &= pm - 1;
-      process_voxel<OPAQUE, COUNT, KEY16>(A, R, L);
+      process_voxel<OPAQUE, COUNT, KEY16, AO>(A, R, L);
       if (lane == L) {
         R.pending = false;
         if (R.t1 < 0.0f) R.active = false;
@@ -1004,43 +1017,46 @@ __global__ void __launch_bounds__(kTraceThreads) k_trace(TraceArgs A) {
 }
 
 // Persistent grid: as many blocks as can be resident at once.
-template <bool OPAQUE, bool COUNT, bool KEY16>
+template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
 int persistent_blocks(size_t smem) {
   static int blocks = 0;  // per instantiation; the device does not change under a grid
   if (!blocks) {
     int dev = 0, sms = 0, per_sm = 0;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace<OPAQUE, COUNT, KEY16>, kTraceThreads, smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace<OPAQUE, COUNT, KEY16, AO>, kTraceThreads, smem);
     blocks = max(1, sms) * max(1, per_sm);
   }
   return blocks;
 }
 
-template <bool OPAQUE, bool COUNT, bool KEY16>
+template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
 void launch_one(const TraceArgs& a, size_t smem, cudaStream_t s) {
-  if (!OPAQUE && !a.pix_list) {
-    // the instrumented and 16+16-key traces use the default tile
-    const int tw = (COUNT || KEY16) ? 4 : a.tile_w;
-    const int th = 32 / tw;
-    const dim3 grid((a.cam.width + 2 * tw - 1) / (2 * tw), (a.cam.height + 2 * th - 1) / (2 * th));
-    if constexpr (COUNT || KEY16) {
-      k_trace_tile<OPAQUE, COUNT, KEY16, 4><<<grid, kTraceThreads, smem, s>>>(a);
-    } else {
-      if (tw == 2) k_trace_tile<OPAQUE, COUNT, KEY16, 2><<<grid, kTraceThreads, smem, s>>>(a);
-      else if (tw == 8) k_trace_tile<OPAQUE, COUNT, KEY16, 8><<<grid, kTraceThreads, smem, s>>>(a);
-      else if (tw == 16) k_trace_tile<OPAQUE, COUNT, KEY16, 16><<<grid, kTraceThreads, smem, s>>>(a);
-      else k_trace_tile<OPAQUE, COUNT, KEY16, 4><<<grid, kTraceThreads, smem, s>>>(a);
+  if constexpr (!OPAQUE) {
+    if (!a.pix_list) {
+      // the instrumented and 16+16-key traces use the default tile
+      const int tw = (COUNT || KEY16) ? 4 : a.tile_w;
+      const int th = 32 / tw;
+      const dim3 grid((a.cam.width + 2 * tw - 1) / (2 * tw), (a.cam.height + 2 * th - 1) / (2 * th));
+      if constexpr (COUNT || KEY16) {
+        k_trace_tile<OPAQUE, COUNT, KEY16, AO, 4><<<grid, kTraceThreads, smem, s>>>(a);
+      } else {
+        if (tw == 2) k_trace_tile<OPAQUE, COUNT, KEY16, AO, 2><<<grid, kTraceThreads, smem, s>>>(a);
+        else if (tw == 8) k_trace_tile<OPAQUE, COUNT, KEY16, AO, 8><<<grid, kTraceThreads, smem, s>>>(a);
+        else if (tw == 16) k_trace_tile<OPAQUE, COUNT, KEY16, AO, 16><<<grid, kTraceThreads, smem, s>>>(a);
+        else k_trace_tile<OPAQUE, COUNT, KEY16, AO, 4><<<grid, kTraceThreads, smem, s>>>(a);
+      }
+      return;
     }
-  } else {
-    k_trace<OPAQUE, COUNT, KEY16><<<persistent_blocks<OPAQUE, COUNT, KEY16>(smem), kTraceThreads, smem, s>>>(a);
   }
+  k_trace<OPAQUE, COUNT, KEY16, AO><<<persistent_blocks<OPAQUE, COUNT, KEY16, AO>(smem), kTraceThreads, smem, s>>>(a);
 }
 
 template <bool COUNT, bool KEY16>
 void launch_mode(const TraceArgs& a, int K, size_t smem, cudaStream_t s) {
-  if (K == 1) launch_one<true, COUNT, KEY16>(a, smem, s);
-  else launch_one<false, COUNT, KEY16>(a, smem, s);
+  if (K == 1) launch_one<true, COUNT, KEY16, false>(a, smem, s);  // AO: k_shade_hits
+  else if (a.ao == 1) launch_one<false, COUNT, KEY16, true>(a, smem, s);
+  else launch_one<false, COUNT, KEY16, false>(a, smem, s);
 }
 
 int launch_trace(const TraceArgs& a, int K, cudaStream_t s) {
@@ -1052,6 +1068,35 @@ int launch_trace(const TraceArgs& a, int K, cudaStream_t s) {
     if (a.key16) launch_mode<false, true>(a, K, smem, s);
     else launch_mode<false, false>(a, K, smem, s);
   }
+  return 1;
+}
+
+// Cone AO of an opaque trace: the pixels hold their hits (opaque_hit), and one
+// thread per pixel, 8x4 tiles to a warp, shades them after the last repair
+// round. Inside the trace the rays of a warp find their hits in different
+// rounds, so few of its lanes shaded at a time, at the trace's occupancy
+// (95% of the trace's cycles on the 1080p ABC view); here every lane has a hit
+// and neighbours share texels.
+__global__ void __launch_bounds__(kTraceThreads) k_shade_hits(TraceArgs A) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int px = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
+  const int py = blockIdx.y * 8 + (warp >> 1) * 4 + (lane >> 3);
+  if (px >= A.cam.width || py >= A.cam.height) return;
+  float4* out = &A.rgba[(size_t)py * A.cam.width + px];
+  const float4 v = *out;
+  if (v.w == 0.0f) return;  // no hit: transparent black
+  const uint32_t id = __float_as_uint(v.x);
+  // a pixel the repair left unfinished (vrt_sync reports it) holds no hit
+  if (id >= A.n_vert || id + 1 >= A.n_vert) return;
+  float3 o, d;
+  pixel_ray(A.cam, px, py, o, d);
+  const float3 c = ao_lane(A, o + v.y * d) * tangent_colour(A, id);
+  *out = make_float4(A.alpha * c.x, A.alpha * c.y, A.alpha * c.z, v.w);
+}
+
+int launch_shade_hits(const TraceArgs& a, cudaStream_t s) {
+  const dim3 grid((a.cam.width + 15) / 16, (a.cam.height + 7) / 8);
+  k_shade_hits<<<grid, kTraceThreads, 0, s>>>(a);
   return 1;
 }
 
