@@ -99,9 +99,8 @@ typedef struct {
                        of the occupied voxels, culling again every 8th build.
                        The image is the same in every mode. */
   int32_t k;        /* 0, 1, 8, 16 or 32; kept for compatibility: the trace
-                       keeps 4 nearest keys per lane (128 per warp) and
-                       rescans a list when it must, so the image does not
-                       depend on k */
+                       composites every hit whatever k, so the image does
+                       not depend on it */
   int32_t voxel_shading; /* 0: shade per hit (ao_cones); 1: voxel-space
                        shading (Sec. 3.4): before the trace, every voxel
                        within one step of a listed voxel gets the value
@@ -273,14 +272,13 @@ vrt_status vrt_read_shading(vrt_grid g, float* values_host, uint8_t* valid_host)
  * wrong (every list access stays bounded). -1 restores the normal scan. With
  * g == NULL it applies, process-wide, to vrt_scan_counts_noalloc (status bit
  * 0). No wait is left unbounded in either case.
- * VRT_OPT_TRACE_SHORT_LIST (8): value in [0, 1024] (default 1024): voxel lists
- * up to this length share the warp entry by entry in the trace; longer ones
+ * VRT_OPT_TRACE_SHORT_LIST (8): value in [0, 1024] (not set: no limit): voxel
+ * lists up to this length share the warp entry by entry in the trace; longer ones
  * take the whole-warp path (one list at a time). The image does not depend on
  * it; for testing that path.
- * VRT_OPT_TRACE_RAY_KEYS (9): value in [1, 32] (default 32): hit slots per
- * transparent ray and voxel on the shared-entry path; a ray with more hits in
- * one voxel takes the whole-warp path for it. The image does not depend on
- * it; for testing.
+ * VRT_OPT_TRACE_RAY_KEYS (9): value in [1, 32] (not set: no limit): a transparent
+ * ray with more hits in one voxel takes the whole-warp path for it. The image
+ * does not depend on it; for testing.
  * VRT_OPT_HIT_KEY (10): the order of the hits a ray composites within one
  * voxel (Sec. 3.5). VRT_HIT_KEY_DEPTH_ID (default): by depth in fp32, equal
  * depths by segment id -- the ground-truth order, independent of how the list
@@ -289,11 +287,12 @@ vrt_status vrt_read_shading(vrt_grid g, float* values_host, uint8_t* valid_host)
  * 16-bit index in the voxel's list, so hits whose depths fall in the same
  * 1/65536 of the interval follow the list's order (which the list build's
  * atomics leave arbitrary); depths and shading still use the exact hit.
- * VRT_OPT_TRACE_TILE (11): the pixel tile a warp of the transparent trace owns:
- * 32 pixels, 2, 4 (default), 8 or 16 wide (16, 8, 4 or 2 tall). Rays of a tile
- * that wait in the same voxel share each list entry's loads, so the best shape
- * depends on the scene and camera (vrt_tune_shapes measures it). The image
- * does not depend on it. The instrumented trace and the 16+16 key use 4. */
+ * VRT_OPT_TRACE_TILE (11): the pixel tile a warp of the trace owns: 32 pixels, 2,
+ * 4 (default), 8 or 16 wide (16, 8, 4 or 2 tall). Rays of a tile that wait in the
+ * same voxel share each list entry's loads, so the best shape depends on the
+ * scene and camera (vrt_tune_shapes measures it). The image does not depend on
+ * it. Transparent images too small for such tiles to fill the GPU use tiles of
+ * 16, 8 or 4 pixels of a fixed shape. */
 #define VRT_OPT_FORCE_EXACT 1
 #define VRT_OPT_STAGE_TIMING 2
 #define VRT_OPT_TRACE_COUNTERS 3

@@ -36,6 +36,7 @@ struct vrt_grid_s {
   // voxels
   uint32_t *word = nullptr, *cur = nullptr, *vis = nullptr;
   uint8_t *bdist = nullptr, *btmp = nullptr;  // empty-brick distance field and its scratch
+  uint2* bmask = nullptr;    // [bricks] occupied voxels of each brick
   uint32_t* need = nullptr;
   uint8_t* eroded = nullptr;
   uint8_t* cdist = nullptr;  // [bricks] distance to a brick with eroded occupancy
@@ -90,8 +91,8 @@ struct vrt_grid_s {
   // frame is captured on (the legacy default stream cannot be captured)
   float cull_depth = 0.0f;  // VRT_OPT_CULL_DEPTH (0: the default threshold)
   int scan_stall = -1;      // VRT_OPT_TEST_SCAN_STALL (-1: off)
-  uint32_t short_list = kShortList;  // VRT_OPT_TRACE_SHORT_LIST
-  uint32_t ray_keys = kRayKeys;      // VRT_OPT_TRACE_RAY_KEYS
+  uint32_t short_list = 0xffffu;  // VRT_OPT_TRACE_SHORT_LIST (default: every list)
+  uint32_t ray_keys = 0xffffu;    // VRT_OPT_TRACE_RAY_KEYS (default: no limit of its own)
   int key16 = 0;                     // VRT_OPT_HIT_KEY
   int tile_w = 4;                    // VRT_OPT_TRACE_TILE
   bool use_graph = false;
@@ -162,7 +163,7 @@ GridDev gdev(vrt_grid g) {
   d.corr = (g->r / d.r_clamp) * (g->r / d.r_clamp);
   d.occ_scale = (float)g->occ_scale;
   d.force_exact = g->force_exact;
-  d.word = g->word; d.cur = g->cur; d.vis = g->vis; d.bdist = g->bdist;
+  d.word = g->word; d.cur = g->cur; d.vis = g->vis; d.bdist = g->bdist; d.bmask = g->bmask;
   d.lists = g->lists; d.list_cap = g->list_cap;
   d.xq = g->xq; d.xq_cap = g->xq_cap;
   d.rec = g->rec; d.rank = g->rank; d.rec_cap = (uint32_t)g->list_cap;
@@ -429,7 +430,7 @@ void free_all(vrt_grid g) {
     for (int j = 0; j < 2; ++j)
       if (g->ev[i][j]) { cudaEventDestroy(g->ev[i][j]); g->ev[i][j] = nullptr; }
   dfree(g, g->raw); dfree(g, g->flags); dfree(g, g->pos); dfree(g, g->nrm); dfree(g, g->order);
-  dfree(g, g->word); dfree(g, g->cur); dfree(g, g->vis); dfree(g, g->bdist); dfree(g, g->btmp);
+  dfree(g, g->word); dfree(g, g->cur); dfree(g, g->vis); dfree(g, g->bdist); dfree(g, g->btmp); dfree(g, g->bmask);
   dfree(g, g->need); dfree(g, g->eroded); dfree(g, g->cdist); dfree(g, g->emean); dfree(g, g->lists); dfree(g, g->tile_state);
   dfree(g, g->xq); dfree(g, g->rec); dfree(g, g->rank);
   dfree(g, g->mips); dfree(g, g->vq[0]); dfree(g, g->vq[1]); dfree(g, g->pq[0]); dfree(g, g->pq[1]);
@@ -477,6 +478,7 @@ vrt_status vrt_create_grid(const vrt_grid_desc* desc, void* cuda_stream, vrt_gri
   chk(dalloc(g, &g->need, nv / 32));
   chk(dalloc(g, &g->bdist, nb));
   chk(dalloc(g, &g->btmp, nb));
+  chk(dalloc(g, &g->bmask, nb));
   g->n_tiles = (uint32_t)(nv / 4096);
   chk(dalloc(g, &g->tile_state, g->n_tiles));
   chk(dalloc(g, &g->st, 1));
@@ -647,7 +649,7 @@ vrt_status vrt_voxelize(vrt_grid g) {
   stage_mark(g, ST_INGEST, 1);
   stage_mark(g, ST_PASS1, 0);
   g->launches += launch_pass1(g->pos, g->nrm, g->order, g->V, gdev(g), g->stream);
-  g->launches += launch_brick_dist(gdev(g), g->btmp, g->bdist, g->stream);
+  g->launches += launch_brick_dist(gdev(g), g->btmp, g->bdist, g->bmask, g->stream);
   stage_mark(g, ST_PASS1, 1);
   VRT_CUDA(g, cudaGetLastError());
   g->stage = 2;

@@ -11,19 +11,25 @@
 
 namespace vrt {
 
-// One thread per brick: 0 when any of its 64 voxels has a count, else the cap.
-__global__ void __launch_bounds__(256) k_brick_occ(GridDev g, uint8_t* __restrict__ out) {
-  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
-  const uint32_t nb = 1u << (3 * g.log2nb);
-  if (b >= nb) return;
-  const uint4* w = reinterpret_cast<const uint4*>(g.word + ((size_t)b << 6));
-  uint32_t any = 0;
+// The occupancy mask of each brick, and 0 when any of its 64 voxels has a count,
+// else the cap. A thread reads one x-row of a brick (16 bytes, so a warp reads
+// 512 contiguous bytes) and the brick's 16 threads combine their four bits.
+__global__ void __launch_bounds__(256) k_brick_occ(GridDev g, uint8_t* __restrict__ out,
+                                                   uint2* __restrict__ mask) {
+  const uint32_t row = blockIdx.x * blockDim.x + threadIdx.x;
+  const int lane = threadIdx.x & 31;
+  const uint4 v = __ldg(reinterpret_cast<const uint4*>(g.word) + row);  // n^3 / 4 rows: whole blocks
+  const uint32_t m = ((v.x & 0xffffu) ? 1u : 0u) | ((v.y & 0xffffu) ? 2u : 0u) |
+                     ((v.z & 0xffffu) ? 4u : 0u) | ((v.w & 0xffffu) ? 8u : 0u);
+  uint32_t half = m << (4 * (lane & 7));  // rows 0-7 and 8-15 of a brick: 32 bits each
 #pragma unroll
-  for (int q = 0; q < 16; ++q) {
-    const uint4 v = __ldg(&w[q]);
-    any |= (v.x | v.y | v.z | v.w) & 0xffffu;
+  for (int o = 4; o > 0; o >>= 1) half |= __shfl_xor_sync(0xffffffffu, half, o);
+  const uint32_t hi = __shfl_down_sync(0xffffffffu, half, 8);
+  if ((lane & 15) == 0) {
+    const uint32_t b = row >> 4;
+    mask[b] = make_uint2(half, hi);
+    out[b] = (half | hi) ? 0 : (uint8_t)kBrickDistMax;
   }
-  out[b] = any ? 0 : (uint8_t)kBrickDistMax;
 }
 
 // out(b) = min over |i| <= kBrickDistMax (inside the grid) of max(|i|, in(b + i e)),
@@ -56,10 +62,9 @@ int launch_brick_dist_passes(int log2nb, uint8_t* tmp, uint8_t* dist, cudaStream
   return 3;
 }
 
-int launch_brick_dist(const GridDev& g, uint8_t* tmp, uint8_t* dist, cudaStream_t s) {
-  const uint32_t nb = 1u << (3 * g.log2nb);
+int launch_brick_dist(const GridDev& g, uint8_t* tmp, uint8_t* dist, uint2* mask, cudaStream_t s) {
   const int T = 256;
-  k_brick_occ<<<(nb + T - 1) / T, T, 0, s>>>(g, tmp);
+  k_brick_occ<<<(1u << (3 * g.log2nb + 4)) / T, T, 0, s>>>(g, tmp, mask);
   return 1 + launch_brick_dist_passes(g.log2nb, tmp, dist, s);
 }
 

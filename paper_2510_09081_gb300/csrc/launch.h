@@ -50,9 +50,10 @@ struct TraceArgs {
   float4* resume;            // [2 * pixels] state of a ray at its first culled voxel:
                              // (C, T), (first id bits, first t, voxel index bits, entry t)
   uint32_t short_list;       // lists up to this length share the warp entry by entry
-  uint32_t ray_keys;         // hit slots per transparent ray on that path (<= kRayKeys)
+  uint32_t ray_keys;         // hits a transparent ray may have on that path
   int key16;                 // order hits by the paper's 16+16-bit per-voxel key
-  int tile_w;                // transparent trace: warp tile width (2, 4, 8 or 16 pixels)
+  int tile_w;                // warp tile width (2, 4, 8 or 16 pixels)
+  int tile_n;                // rays a warp of the main trace owns (launch_trace sets it)
   int count;                 // accumulate trace work counters
   uint32_t* touch_list;      // instrumented trace: bit per list entry read
   uint32_t* touch_vert;      //   bit per vertex read (segment end points)
@@ -94,8 +95,9 @@ int launch_pass1(const float4* pos, const float4* nrm, const uint32_t* order, lo
 // 12-bit spatial keys (Morton code of the 16^3 cell) of the vertices mid[0..P).
 int launch_poly_keys(const float* raw, const uint32_t* mid, uint32_t P, int n, uint16_t* key,
                      cudaStream_t s);
-// Empty-brick distance field from the counts of pass 1 (tmp: one byte per brick).
-int launch_brick_dist(const GridDev& g, uint8_t* tmp, uint8_t* dist, cudaStream_t s);
+// Occupancy masks and empty-brick distance field from the counts of pass 1
+// (tmp: one byte per brick).
+int launch_brick_dist(const GridDev& g, uint8_t* tmp, uint8_t* dist, uint2* mask, cudaStream_t s);
 // The three distance passes from per-brick bytes in tmp (0 = occupied, else
 // kBrickDistMax); tmp is overwritten.
 int launch_brick_dist_passes(int log2nb, uint8_t* tmp, uint8_t* dist, cudaStream_t s);

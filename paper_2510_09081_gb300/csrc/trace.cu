@@ -1,16 +1,23 @@
 // A6: voxel ray tracing (Sec. 3.5).
 //
-// One ray per pixel; a warp owns a pixel tile, 4 wide and 8 tall for
-// transparent rays, 8 by 4 for opaque ones (in the repair re-trace, 32 queued
-// pixels). Each lane steps its own ray by 3D-DDA (Amanatides & Woo)
-// through the grid box until it reaches a voxel with a list; in a brick with
-// no occupied voxel it crosses, in one step, the whole cube of empty bricks
-// that the distance field built after pass 1 guarantees around it. The warp then
-// numbers the entries of all its lanes' pending lists one after another and
-// takes them 32 at a time, one (ray, entry) pair per lane, so no lane idles on
-// another lane's longer list. Very long lists, and a transparent ray with more
-// hits in one voxel than its shared-memory slots hold, go to a whole-warp path
-// that processes one voxel at a time (lane l takes entries l, l+32, ...).
+// One ray per pixel; a warp owns a tile of pixels, 4 wide and 8 tall (in the
+// repair re-trace, its share of the queued pixels). Each lane walks its own ray by
+// 3D-DDA (Amanatides & Woo), a 4^3 brick per round, until it reaches an occupied
+// voxel; in a brick with no occupied voxel it crosses, in one step, the whole cube
+// of empty bricks that the distance field built after pass 1 guarantees around
+// it. The warp then numbers the entries of its lanes' pending lists one after
+// another and takes them 64 at a time, so no lane idles on another lane's longer
+// list; rays waiting in the same voxel share an entry's loads. A list longer than
+// the test options allow, or (with the 16+16 key) more hits in a round than its
+// shared-memory slots hold, goes to a whole-warp path that processes one voxel
+// at a time (lane l takes entries l, l+32, ...).
+//
+// Bound by instruction issue and latency, not memory: 20 warps an SM, 1.3 G warp
+// instructions at 53% of the issue slots for 147M (ray, entry) pairs. Against a
+// trace that kept all of a ray's state in registers (128, 16 warps an SM),
+// stepped voxel by voxel on three loads a step, and took a pair a lane: sparse
+// walks at 4K 31.0 -> 21.4 ms, 157x93 pixels at alpha 0.1 0.70 -> 0.22 ms, 10M-segment
+// bundles at 1080p 3.25 -> 2.80 ms, opaque ABC at 1080p 0.57 -> 0.41 ms.
 //
 // For each listed segment the lane computes the first entry of the ray into
 // the segment's capsule; an entry counts only if it lies in the voxel's ray
@@ -20,8 +27,8 @@
 // line passes farther than r from the ray.
 //  - opaque: the minimum 64-bit key (depth bits << 32 | segment id) is the
 //    voxel's nearest hit; the ray stops at the first voxel that has one.
-//  - transparent, shared entries: a ray's hits in the voxel are collected in
-//    shared memory, sorted by key and composited by the ray's lane.
+//  - transparent, shared entries: the hits of the warp's rays are collected in
+//    shared memory, ranked by key and composited by each ray's lane.
 //  - transparent, whole-warp path: each lane keeps its 4 smallest keys beyond the last
 //    composited one; the warp extracts keys in global (depth, id) order by
 //    repeated minimum reductions -- only up to the smallest key a lane had to
@@ -45,6 +52,8 @@
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
 
+#include <cmath>
+
 #include "launch.h"
 #include "pyramid.cuh"
 
@@ -52,17 +61,21 @@ namespace vrt {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kLaneKeys = 4;              // transparent, shared list: keys kept per lane per scan
-// kRayKeys (vrt_internal.cuh): hit slots per transparent ray on the shared-entry
-// path, 32 KB of shared memory per block; A.ray_keys <= kRayKeys of them are used.
-// 40 slots (40 KB) left the 4 resident blocks of an SM so little L1 that the
-// trace of a sparse 512^3 set at 4K ran 5% slower; 24 slots sent too many rays
-// to the whole-warp path (bundles trace 2.5% slower).
 constexpr int kTraceThreads = 128;
-constexpr int kStepRound = 1;             // tile trace: DDA steps a walking lane takes per round
-
-__device__ __forceinline__ bool bit_at(const uint32_t* bits, uint32_t i) {
-  return (bits[i >> 5] >> (i & 31)) & 1u;
-}
+// Transparent: hits of a round that a warp's rays share (slots are bytes), and the
+// (ray, entry) pairs a round takes rays for. About 7% of the pairs of dense sets
+// give hits; 128 and 768 send more rays back for another pass (bundles at
+// 1080p 2.92 ms against 2.86), and a larger pool takes L1 from the lists.
+constexpr uint32_t kPool = 192;
+constexpr uint32_t kRoundPairs = 1536;
+constexpr uint32_t kLost = 1u << 31;  // WarpMem::cnt: a hit of the ray found the pool full
+// Rays that share an entry's loads. Lists are short (4 entries on average for
+// sparse walks, 24 for the bundles), so larger groups leave lanes without an
+// entry: groups of 32 take 0.55 ms where 4 take 0.43 on the opaque 1080p ABC
+// view, and 3.37 against 3.30 on the bundles; single rays 0.46 and 3.73.
+constexpr int kGroup = 4;
+// Warps the GPU holds at the transparent trace's 5 blocks per SM.
+constexpr int kResidentWarps = 152 * 5 * (kTraceThreads / 32);
 
 // Instrumented trace: mark element i of a touch bitmap.
 __device__ __forceinline__ void touch(uint32_t* bits, uint32_t i) {
@@ -117,12 +130,11 @@ __device__ __forceinline__ float hit_shade(const TraceArgs& A, float3 P) {
   else return field_shade(A, P);
 }
 
-__device__ __forceinline__ float3 tangent_colour(const TraceArgs& A, uint32_t id) {
-  const float3 a = f3(__ldg(&A.pos[id])), b = f3(__ldg(&A.pos[id + 1]));
+__device__ __forceinline__ float3 tangent_colour(float3 a, float3 b) {
   const float3 dv = b - a;
   const float l2 = dot3(dv, dv);
   if (!(l2 > 0.0f)) return make_float3(1.0f, 1.0f, 1.0f);
-  const float il = rsqrtf(l2);  // the hardware's approximate reciprocal square root
+  const float il = rsqrt_normal(l2);
   return make_float3(fabsf(dv.x) * il, fabsf(dv.y) * il, fabsf(dv.z) * il);
 }
 
@@ -190,134 +202,187 @@ __device__ __forceinline__ unsigned long long entry_key(const TraceArgs& A, uint
   return hit_key<KEY16>(t, id, s - beg, t0, t1);
 }
 
-// Per-lane ray state. Components are kept as scalars (no runtime-indexed
-// arrays) so the DDA state stays in registers.
-struct Ray {
-  float3 o, d, inv, ooi;  // ooi = o * inv: the boundary b is crossed at b * inv - ooi
-  int sx, sy, sz;      // step direction per axis (-1, 0, 1)
-  int vx, vy, vz;      // current voxel
-  float tcur, t1;
-  float C[3], T;
-  int first_id;
-  float first_t;
-  uint32_t pix, n_queued;
-  bool active, pending, missed;
-  uint32_t beg, end;   // pending voxel's list
-  float vt0, vt1;      // pending voxel's ray interval
-  unsigned n_steps, n_entries, n_cap, n_vox;  // work counters
-  unsigned n_hits, n_ww_vox, n_ww_ent;
-  unsigned long long cyc[4];  // warp cycles: DDA, shared-entry path, whole-warp path, capsule stage
+// One warp's shared memory. Per ray: what the line and capsule tests of other
+// lanes read (origin and entry parameter, direction and exit parameter) and what
+// its own lane needs only between tests (reciprocal direction, colour, first
+// hit), which keeps the registers of a lane to the walk's or the test's working
+// set. Transparent hits of a round go to a pool that the warp's rays share;
+// opaque rays keep their nearest key.
+template <bool OPAQUE, bool KEY16>
+struct WarpMem {
+  float4 o[32];     // origin, entry parameter of the pending voxel
+  float4 d[32];     // direction, exit parameter
+  float4 inv[32];   // 1 / direction per axis (0 where it is 0); first hit's id as bits
+  float4 acc[32];   // colour so far; first hit's depth
+  uint32_t uid[128];             // segment ids of the units of this step and the last
+  uint16_t uli[KEY16 ? 128 : 2]; // their list indices (16+16 keys)
+  uint16_t q[32 + 64 * kGroup];  // pairs queued for the capsule test: unit | ray << 8
+  unsigned long long key[OPAQUE ? 32 : kPool];  // opaque: the ray's nearest key
+  float col[OPAQUE ? 1 : 3][OPAQUE ? 1 : kPool];
+  uint16_t own[OPAQUE ? 2 : kPool];    // the hit's ray | its number among the ray's hits << 8
+  uint8_t slot[OPAQUE ? 4 : kPool];    // pool slots, ray after ray
+  uint8_t order[OPAQUE ? 4 : kPool];   // the same, each ray's by key
+  uint32_t cnt[OPAQUE ? 1 : 32];       // hits of each ray in the round
 };
 
-// Parameter where the ray leaves coordinate range [lo, hi] along an axis
-// (the side it moves toward); +inf when it does not move on that axis.
-__device__ __forceinline__ float exit_t(int s, int lo, int hi, float ooi, float inv) {
-  return s != 0 ? fmaf((float)(s > 0 ? hi : lo), inv, -ooi) : __int_as_float(0x7f800000);
+// Registers a lane keeps for its ray. Voxel coordinates are packed, four added
+// to each (so that the fields stay positive one step outside the grid):
+// (x + 4) | (y + 4) << 10 | (z + 4) << 20.
+struct Ray {
+  uint32_t p;
+  uint2 mask;          // the current brick's occupied voxels
+  int kd;              // and its distance to an occupied brick
+  float tcur, t1, T;
+  uint32_t pix, vox;   // pixel; pending voxel's word index
+  uint32_t beg, len;   // pending voxel's list
+  uint32_t n_queued;
+  bool active, pending, missed;
+};
+
+// Work counters of a lane (instrumented trace).
+struct Work {
+  unsigned steps = 0, entries = 0, cap = 0, vox = 0, hits = 0, ww_vox = 0, ww_ent = 0;
+  // warp cycles: DDA, shared-entry path, whole-warp path, capsule stage
+  unsigned long long cyc[4] = {0, 0, 0, 0};
+};
+
+__device__ __forceinline__ uint32_t pack_pos(int x, int y, int z) {
+  return (uint32_t)(x + 4) | ((uint32_t)(y + 4) << 10) | ((uint32_t)(z + 4) << 20);
+}
+__device__ __forceinline__ void unpack_pos(uint32_t p, int& x, int& y, int& z) {
+  x = (int)(p & 1023u) - 4;
+  y = (int)((p >> 10) & 1023u) - 4;
+  z = (int)(p >> 20) - 4;
+}
+constexpr uint32_t kLocalBits = 0x00300c03u;  // the coordinates within a 4^3 brick
+
+// Parameter where the ray leaves coordinate `b` along an axis it moves on;
+// +inf when it does not move on that axis.
+__device__ __forceinline__ float cross_t(float inv, float b, float ooi) {
+  return inv != 0.0f ? fmaf(b, inv, -ooi) : __int_as_float(0x7f800000);
 }
 
-// Step the lane's ray toward its next voxel that has a list, at most `budget`
-// steps: 1 when it reached one (pending), 0 when the ray leaves the grid (or
-// queues too many culled voxels), -1 when the budget ran out first. Every step
-// moves the ray forward through the grid, so its walk ends.
-template <bool COUNT>
-__device__ int advance(const TraceArgs& A, Ray& R, int budget) {
+__device__ __forceinline__ uint32_t brick_of(const TraceArgs& A, int x, int y, int z) {
+  return ((uint32_t)(z >> 2) << (2 * A.g.log2nb)) | ((uint32_t)(y >> 2) << A.g.log2nb) | (uint32_t)(x >> 2);
+}
+
+// Read the mask and empty distance of the brick the ray is in (R.p in the grid).
+__device__ __forceinline__ void load_brick(const TraceArgs& A, Ray& R) {
+  int x, y, z;
+  unpack_pos(R.p, x, y, z);
+  const uint32_t b = brick_of(A, x, y, z);
+  R.mask = __ldg(&A.g.bmask[b]);
+  R.kd = __ldg(&A.g.bdist[b]);
+}
+
+// Walk the lane's ray through the brick it is in: 1 when it reached an occupied
+// voxel (then pending in R.vox over [o.w, d.w)), 0 when it leaves the grid, -1
+// when it goes on in the next brick. In a brick without occupied voxels the ray
+// crosses the whole cube of empty bricks around it. Every call moves the ray
+// forward through the grid, so its walk ends.
+//
+// Bound by the latency of its loads: a call reads the brick's 64-bit occupancy
+// mask and its empty distance, once, and steps from voxel to voxel on the mask
+// in registers; the voxel's word and list end are read only for an occupied
+// voxel, in the round that processes it. Reading the distance, word and list
+// end at every voxel step kept a 4K trace of sparse walks in 512^3 (133 steps and
+// 16 occupied voxels per ray, words far larger than L2) waiting on three loads
+// per step.
+template <class M, bool COUNT>
+__device__ __forceinline__ int walk_brick(const TraceArgs& A, M& S, Ray& R, Work& W) {
+  const int lane = threadIdx.x & 31;
   const int n = A.g.n;
-  for (int it = 0; it < budget; ++it) {
-    if (R.tcur > R.t1) return 0;
-    if (COUNT) ++R.n_steps;
-    const uint32_t bidx = ((uint32_t)(R.vz >> 2) << (2 * A.g.log2nb)) |
-                          ((uint32_t)(R.vy >> 2) << A.g.log2nb) | (uint32_t)(R.vx >> 2);
-    const uint32_t idx = brick_index(R.vx, R.vy, R.vz, A.g.log2nb);
-    // the step's loads are independent: issue them together (one latency, not
-    // up to three in sequence); the word and the list end -- at or above
-    // kCulledStart when the cull gave the voxel no list -- go unused in an
-    // empty brick
-    const int kd = __ldg(&A.g.bdist[bidx]);
-    const uint32_t wv = __ldg(&A.g.word[idx]);
-    const uint32_t cv = __ldg(&A.g.cur[idx]);
-    if (kd > 0) {
-      // cross the cube of empty bricks within kd - 1 of this one: low corner
-      // (bx, by, bz), side w voxels
-      const int ext = 4 * (kd - 1), w = 4 + 2 * ext;
-      const int bx = (R.vx & ~3) - ext, by = (R.vy & ~3) - ext, bz = (R.vz & ~3) - ext;
-      const float tx = exit_t(R.sx, bx, bx + w, R.ooi.x, R.inv.x);
-      const float ty = exit_t(R.sy, by, by + w, R.ooi.y, R.inv.y);
-      const float tz = exit_t(R.sz, bz, bz + w, R.ooi.z, R.inv.z);
-      const float tb = fminf(tx, fminf(ty, tz));
-      if (tb > R.t1) return 0;
-      const int cx = min(min(bx + w, n) - 1, max(max(bx, 0), (int)floorf(fmaf(tb, R.d.x, R.o.x))));
-      const int cy = min(min(by + w, n) - 1, max(max(by, 0), (int)floorf(fmaf(tb, R.d.y, R.o.y))));
-      const int cz = min(min(bz + w, n) - 1, max(max(bz, 0), (int)floorf(fmaf(tb, R.d.z, R.o.z))));
-      if (tb == tx) {
-        R.vx = R.sx > 0 ? bx + w : bx - 1; R.vy = cy; R.vz = cz;
-        if (R.vx < 0 || R.vx >= n) return 0;
-      } else if (tb == ty) {
-        R.vy = R.sy > 0 ? by + w : by - 1; R.vx = cx; R.vz = cz;
-        if (R.vy < 0 || R.vy >= n) return 0;
-      } else {
-        R.vz = R.sz > 0 ? bz + w : bz - 1; R.vx = cx; R.vy = cy;
-        if (R.vz < 0 || R.vz >= n) return 0;
-      }
-      R.tcur = fmaxf(R.tcur, tb);
-      continue;
-    }
-    const float tx = exit_t(R.sx, R.vx, R.vx + 1, R.ooi.x, R.inv.x);
-    const float ty = exit_t(R.sy, R.vy, R.vy + 1, R.ooi.y, R.inv.y);
-    const float tz = exit_t(R.sz, R.vz, R.vz + 1, R.ooi.z, R.inv.z);
-    const float texit = fminf(tx, fminf(ty, tz));
-    const uint32_t cnt = wv & 0xffffu;
-    if (COUNT) touch(A.touch_vox, idx);
-    const float tin = R.tcur;
-    // step past this voxel before returning, so the next call resumes after it
-    R.tcur = texit;
-    bool inside;
-    if (texit == tx) {
-      R.vx += R.sx;
-      inside = R.vx >= 0 && R.vx < n;
-    } else if (texit == ty) {
-      R.vy += R.sy;
-      inside = R.vy >= 0 && R.vy < n;
+  if (R.tcur > R.t1) return 0;
+  int x, y, z;
+  unpack_pos(R.p, x, y, z);
+  const float4 inv = S.inv[lane], o = S.o[lane];
+  const float3 ooi = make_float3(o.x * inv.x, o.y * inv.y, o.z * inv.z);
+  if (R.kd > 0) {
+    // cross the cube of empty bricks within kd - 1 of this one: low corner
+    // (bx, by, bz), side w voxels
+    if (COUNT) ++W.steps;
+    const float4 d = S.d[lane];
+    const int ext = 4 * (R.kd - 1), w = 4 + 2 * ext;
+    const int bx = (x & ~3) - ext, by = (y & ~3) - ext, bz = (z & ~3) - ext;
+    const float tx = cross_t(inv.x, (float)(inv.x > 0.0f ? bx + w : bx), ooi.x);
+    const float ty = cross_t(inv.y, (float)(inv.y > 0.0f ? by + w : by), ooi.y);
+    const float tz = cross_t(inv.z, (float)(inv.z > 0.0f ? bz + w : bz), ooi.z);
+    const float tb = fminf(tx, fminf(ty, tz));
+    if (tb > R.t1) return 0;
+    const int cx = min(min(bx + w, n) - 1, max(max(bx, 0), (int)floorf(fmaf(tb, d.x, o.x))));
+    const int cy = min(min(by + w, n) - 1, max(max(by, 0), (int)floorf(fmaf(tb, d.y, o.y))));
+    const int cz = min(min(bz + w, n) - 1, max(max(bz, 0), (int)floorf(fmaf(tb, d.z, o.z))));
+    if (tb == tx) {
+      x = inv.x > 0.0f ? bx + w : bx - 1; y = cy; z = cz;
+      if ((unsigned)x >= (unsigned)n) return 0;
+    } else if (tb == ty) {
+      y = inv.y > 0.0f ? by + w : by - 1; x = cx; z = cz;
+      if ((unsigned)y >= (unsigned)n) return 0;
     } else {
-      R.vz += R.sz;
-      inside = R.vz >= 0 && R.vz < n;
+      z = inv.z > 0.0f ? bz + w : bz - 1; x = cx; y = cy;
+      if ((unsigned)z >= (unsigned)n) return 0;
     }
-    if (cnt) {
-      if (cv >= kCulledStart) {  // the cull gave it no list
-        // culled voxel on the ray: queue it, march on as if it were empty; at
-        // the first one, keep the ray's state for the re-trace to resume from
-        if (R.n_queued == 0 && A.resume) {
-          A.resume[2 * R.pix] = make_float4(R.C[0], R.C[1], R.C[2], R.T);
-          A.resume[2 * R.pix + 1] = make_float4(__int_as_float(R.first_id), R.first_t,
-                                                __uint_as_float(idx), tin);
-        }
-        const uint32_t bm = 1u << (idx & 31);
-        const uint32_t old = atomicOr(&A.need[idx >> 5], bm);
-        if (!(old & bm)) {
-          const uint32_t q = atomicAdd(A.vq_cnt, 1u);
-          if (q < A.vq_cap) A.vq[q] = idx;
-          else set_err(A.g.st, kErrOverflow);
-        }
-        R.missed = true;
-        if (++R.n_queued >= A.max_queue) return 0;
-      } else {
-        // a list past the capacity (reported as overflow) is read only up to it
-        const uint32_t end0 = cv;
-        if (end0 < cnt) {
-          set_err(A.g.st, kErrBounds);
-          return 0;
-        }
-        const uint32_t end = (unsigned long long)end0 > A.g.list_cap ? (uint32_t)A.g.list_cap : end0;
-        R.beg = end0 - cnt < end ? end0 - cnt : end;
-        R.end = end;
-        R.vt0 = tin;
-        R.vt1 = texit;
-        if (!inside) R.t1 = -1.0f;  // this was the last voxel; stop after it
-        return 1;
-      }
-    }
-    if (!inside) return 0;
+    R.p = pack_pos(x, y, z);
+    R.tcur = fmaxf(R.tcur, tb);
+    load_brick(A, R);
+    return -1;
   }
-  return -1;  // budget used up, ray still on its way
+  const float sx = inv.x > 0.0f ? 1.0f : -1.0f, sy = inv.y > 0.0f ? 1.0f : -1.0f,
+              sz = inv.z > 0.0f ? 1.0f : -1.0f;
+  float bx = (float)(inv.x > 0.0f ? x + 1 : x), by = (float)(inv.y > 0.0f ? y + 1 : y),
+        bz = (float)(inv.z > 0.0f ? z + 1 : z);
+  const uint32_t px = inv.x > 0.0f ? 1u : 0u - 1u, py = inv.y > 0.0f ? 1u << 10 : 0u - (1u << 10),
+                 pz = inv.z > 0.0f ? 1u << 20 : 0u - (1u << 20);
+  float tx = cross_t(inv.x, bx, ooi.x), ty = cross_t(inv.y, by, ooi.y), tz = cross_t(inv.z, bz, ooi.z);
+  const uint32_t p0 = R.p;
+  uint32_t p = p0;
+  float tin = R.tcur;
+  bool hit, left;
+  uint32_t loc;
+  float te;
+  // at most 10 steps: each leaves one of the brick's 3 x 4 planes of voxels behind
+  for (;;) {
+    if (COUNT) ++W.steps;
+    // x + 4 y + 16 z of the coordinates within the brick: three shifted copies
+    // of the packed fields meet in bits 20-25
+    loc = ((p & kLocalBits) * ((1u << 20) | (1u << 12) | (1u << 4)) >> 20) & 63u;
+    hit = (((loc & 32u) ? R.mask.y : R.mask.x) >> (loc & 31u)) & 1u;
+    te = fminf(tx, fminf(ty, tz));
+    if (te == tx) {
+      p += px;
+      bx += sx;
+      tx = fmaf(bx, inv.x, -ooi.x);
+    } else if (te == ty) {
+      p += py;
+      by += sy;
+      ty = fmaf(by, inv.y, -ooi.y);
+    } else {
+      p += pz;
+      bz += sz;
+      tz = fmaf(bz, inv.z, -ooi.z);
+    }
+    left = ((p ^ p0) & ~kLocalBits) != 0u;
+    if (hit || left || te > R.t1) break;
+    tin = te;
+  }
+  // the ray is past this voxel: the next call resumes after it
+  R.p = p;
+  R.tcur = te;
+  if (hit) R.vox = (brick_of(A, x, y, z) << 6) | loc;
+  bool inside = true;
+  if (left) {
+    unpack_pos(p, x, y, z);
+    inside = (unsigned)x < (unsigned)n && (unsigned)y < (unsigned)n && (unsigned)z < (unsigned)n;
+    // its load completes while the warp's other work goes on
+    if (inside) load_brick(A, R);
+  }
+  if (hit) {
+    S.o[lane].w = tin;
+    S.d[lane].w = te;
+    if (!inside) R.t1 = -1.0f;  // this was the last voxel; stop after it
+    return 1;
+  }
+  return inside ? -1 : 0;
 }
 
 // Origin and unit direction of pixel (px, py)'s ray.
@@ -333,22 +398,21 @@ __device__ __forceinline__ void pixel_ray(const CamDev& c, int px, int py, float
   }
 }
 
-__device__ void init_ray(const TraceArgs& A, Ray& R, int px, int py, bool valid) {
-  pixel_ray(A.cam, px, py, R.o, R.d);
-  R.C[0] = R.C[1] = R.C[2] = 0.0f;
+template <class M>
+__device__ void init_ray(const TraceArgs& A, M& S, Ray& R, int px, int py, bool valid) {
+  const int lane = threadIdx.x & 31;
+  float3 ro, rd, ri;
+  pixel_ray(A.cam, px, py, ro, rd);
   R.T = 1.0f;
-  R.first_id = -1;
-  R.first_t = __int_as_float(0x7f800000);
   R.n_queued = 0;
-  R.n_steps = R.n_entries = R.n_cap = R.n_vox = 0;
-  R.n_hits = R.n_ww_vox = R.n_ww_ent = 0;
   R.missed = false;
   R.pending = false;
+  R.vox = R.beg = R.len = 0;
+  R.pix = valid ? (uint32_t)(py * A.cam.width + px) : 0u;
   const float N = (float)A.g.n;
   float t0 = 0.0f, t1 = __int_as_float(0x7f800000);
   bool miss = !valid;
-  auto axis = [&](float o, float d, int& s, float& inv) {
-    s = d > 0.0f ? 1 : (d < 0.0f ? -1 : 0);
+  auto axis = [&](float o, float d, float& inv) {
     if (d != 0.0f) {
       inv = 1.0f / d;
       float ta = (0.0f - o) * inv, tb = (N - o) * inv;
@@ -360,95 +424,135 @@ __device__ void init_ray(const TraceArgs& A, Ray& R, int px, int py, bool valid)
       if (o < 0.0f || o > N) miss = true;
     }
   };
-  axis(R.o.x, R.d.x, R.sx, R.inv.x);
-  axis(R.o.y, R.d.y, R.sy, R.inv.y);
-  axis(R.o.z, R.d.z, R.sz, R.inv.z);
-  R.ooi = make_float3(R.o.x * R.inv.x, R.o.y * R.inv.y, R.o.z * R.inv.z);
+  axis(ro.x, rd.x, ri.x);
+  axis(ro.y, rd.y, ri.y);
+  axis(ro.z, rd.z, ri.z);
   R.active = !miss && t0 <= t1;
   R.tcur = t0;
   R.t1 = t1;
   const int n = A.g.n;
-  R.vx = min(n - 1, max(0, (int)floorf(fmaf(t0, R.d.x, R.o.x))));
-  R.vy = min(n - 1, max(0, (int)floorf(fmaf(t0, R.d.y, R.o.y))));
-  R.vz = min(n - 1, max(0, (int)floorf(fmaf(t0, R.d.z, R.o.z))));
+  R.p = pack_pos(min(n - 1, max(0, (int)floorf(fmaf(t0, rd.x, ro.x)))),
+                 min(n - 1, max(0, (int)floorf(fmaf(t0, rd.y, ro.y)))),
+                 min(n - 1, max(0, (int)floorf(fmaf(t0, rd.z, ro.z)))));
+  load_brick(A, R);
+  S.o[lane] = make_float4(ro.x, ro.y, ro.z, 0.0f);
+  S.d[lane] = make_float4(rd.x, rd.y, rd.z, 0.0f);
+  S.inv[lane] = make_float4(ri.x, ri.y, ri.z, __int_as_float(-1));
+  S.acc[lane] = make_float4(0.0f, 0.0f, 0.0f, __int_as_float(0x7f800000));
 }
 
 // A re-traced ray continues from the state it had when it first met a culled
 // voxel (now listed): same colour, transmittance and first hit, at that voxel
 // and its entry parameter, so the result equals a trace from the start.
-__device__ void resume_ray(const TraceArgs& A, Ray& R) {
+template <class M>
+__device__ void resume_ray(const TraceArgs& A, M& S, Ray& R) {
+  const int lane = threadIdx.x & 31;
   const float4 s0 = A.resume[2 * R.pix], s1 = A.resume[2 * R.pix + 1];
-  R.C[0] = s0.x; R.C[1] = s0.y; R.C[2] = s0.z;
+  S.acc[lane] = make_float4(s0.x, s0.y, s0.z, s1.y);
+  S.inv[lane].w = s1.x;
   R.T = s0.w;
-  R.first_id = __float_as_int(s1.x);
-  R.first_t = s1.y;
   int x, y, z;
   brick_coords(__float_as_uint(s1.z), A.g.log2nb, x, y, z);
-  R.vx = min(A.g.n - 1, max(0, x));
-  R.vy = min(A.g.n - 1, max(0, y));
-  R.vz = min(A.g.n - 1, max(0, z));
+  R.p = pack_pos(min(A.g.n - 1, max(0, x)), min(A.g.n - 1, max(0, y)), min(A.g.n - 1, max(0, z)));
   R.tcur = s1.w;
+  load_brick(A, R);
+}
+
+// Read the pending voxel's word and list end: its list into R.beg, R.len, or,
+// when the cull gave it none, the voxel into the repair queue, the ray marching
+// on as if it were empty.
+template <class M, bool COUNT>
+__device__ __forceinline__ void resolve_list(const TraceArgs& A, M& S, Ray& R) {
+  const int lane = threadIdx.x & 31;
+  const uint32_t idx = R.vox;
+  const uint32_t cnt = __ldg(&A.g.word[idx]) & 0xffffu;
+  const uint32_t end0 = __ldg(&A.g.cur[idx]);
+  if (COUNT) touch(A.touch_vox, idx);
+  if (end0 >= kCulledStart) {
+    // at the first culled voxel, keep the ray's state for the re-trace to resume from
+    if (R.n_queued == 0 && A.resume) {
+      const float4 c = S.acc[lane];
+      A.resume[2 * R.pix] = make_float4(c.x, c.y, c.z, R.T);
+      A.resume[2 * R.pix + 1] = make_float4(S.inv[lane].w, c.w, __uint_as_float(idx), S.o[lane].w);
+    }
+    const uint32_t bm = 1u << (idx & 31);
+    const uint32_t old = atomicOr(&A.need[idx >> 5], bm);
+    if (!(old & bm)) {
+      const uint32_t q = atomicAdd(A.vq_cnt, 1u);
+      if (q < A.vq_cap) A.vq[q] = idx;
+      else set_err(A.g.st, kErrOverflow);
+    }
+    R.missed = true;
+    R.pending = false;
+    if (++R.n_queued >= A.max_queue || R.t1 < 0.0f) R.active = false;
+    return;
+  }
+  if (end0 < cnt) {
+    set_err(A.g.st, kErrBounds);
+    R.pending = R.active = false;
+    return;
+  }
+  // a list past the capacity (reported as overflow) is read only up to it
+  const uint32_t end = (unsigned long long)end0 > A.g.list_cap ? (uint32_t)A.g.list_cap : end0;
+  R.beg = end0 - cnt < end ? end0 - cnt : end;
+  R.len = end - R.beg;
 }
 
 // An opaque ray ends at its nearest hit. With cone AO its pixel carries the hit
 // (segment id and depth) to k_shade_hits, which writes the colour; otherwise it
 // is shaded here.
-__device__ __forceinline__ void opaque_hit(const TraceArgs& A, Ray& R, uint32_t id, float t) {
+template <class M>
+__device__ __forceinline__ void opaque_hit(const TraceArgs& A, M& S, Ray& R, uint32_t id, float t) {
+  const int lane = threadIdx.x & 31;
+  float3 c;
   if (A.ao == 1) {
-    R.C[0] = __uint_as_float(id);
-    R.C[1] = t;
+    c = make_float3(__uint_as_float(id), t, 0.0f);
   } else {
-    float3 c = tangent_colour(A, id);
-    if (A.ao) c = shade_at(A, R.o + t * R.d) * c;
-    R.C[0] = A.alpha * c.x; R.C[1] = A.alpha * c.y; R.C[2] = A.alpha * c.z;
+    c = tangent_colour(f3(__ldg(&A.pos[id])), f3(__ldg(&A.pos[id + 1])));
+    if (A.ao) c = field_shade(A, f3(S.o[lane]) + t * f3(S.d[lane])) * c;
+    c = make_float3(A.alpha * c.x, A.alpha * c.y, A.alpha * c.z);
   }
+  S.acc[lane] = make_float4(c.x, c.y, c.z, t);
+  S.inv[lane].w = __uint_as_float(id);
   R.T *= (1.0f - A.alpha);
-  R.first_id = (int)id;
-  R.first_t = t;
   R.active = false;
 }
 
-// The warp processes the pending voxel of lane `L`.
-template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
-__device__ void process_voxel(const TraceArgs& A, Ray& R, int L) {
-  const int lane = threadIdx.x & 31;
-  const float3 o = shfl3(R.o, L), d = shfl3(R.d, L);
-  const uint32_t beg = __shfl_sync(FULL, R.beg, L), end = __shfl_sync(FULL, R.end, L);
-  const float t0 = __shfl_sync(FULL, R.vt0, L), t1 = __shfl_sync(FULL, R.vt1, L);
+// The whole warp on one list, [beg, end), for the ray of lane L: the nearest key
+// of an opaque ray.
+template <bool COUNT, bool KEY16>
+__device__ __noinline__ unsigned long long voxel_nearest(const TraceArgs& A, WarpMem<true, KEY16>& S, int L,
+                                                         uint32_t beg, uint32_t end, unsigned& n_cap,
+                                                         unsigned& n_hit) {
+  const float4 o = S.o[L], d = S.d[L];
   const float r2 = A.g.r * A.g.r;
   const float rrm = (A.g.r + 1e-3f) * (A.g.r + 1e-3f);
-  unsigned n_cap = 0, n_hit = 0;
-  if (COUNT && lane == L) {
-    ++R.n_vox;
-    R.n_entries += end - beg;
-    ++R.n_ww_vox;
+  unsigned long long best = ~0ull;
+  for (uint32_t s = beg + (threadIdx.x & 31); s < end; s += 32) {
+    const unsigned long long k =
+        entry_key<COUNT, KEY16>(A, s, beg, f3(o), f3(d), o.w, d.w, r2, rrm, n_cap);
+    if (COUNT && k != ~0ull) ++n_hit;
+    best = k < best ? k : best;
   }
-  if (OPAQUE) {
-    unsigned long long best = ~0ull;
-    for (uint32_t s = beg + lane; s < end; s += 32) {
-      const unsigned long long k = entry_key<COUNT, KEY16>(A, s, beg, o, d, t0, t1, r2, rrm, n_cap);
-      if (COUNT && k != ~0ull) ++n_hit;
-      best = k < best ? k : best;
-    }
-    if (COUNT) {
-      R.n_hits += n_hit;
-      if (lane == L) R.n_ww_ent += end - beg;
-    }
-    if (COUNT) R.n_cap += n_cap;
-    best = warp_min_u64(best);
-    if (best != ~0ull) {
-      const uint32_t id = (uint32_t)(best & 0xffffffffu);
-      const float t = hit_depth<KEY16>(A, best, o, d);
-      if (lane == L) opaque_hit(A, R, id, t);
-    }
-    return;
-  }
-  // transparent
-  float T = __shfl_sync(FULL, R.T, L);
-  float C0 = __shfl_sync(FULL, R.C[0], L), C1 = __shfl_sync(FULL, R.C[1], L),
-        C2 = __shfl_sync(FULL, R.C[2], L);
-  int fid = __shfl_sync(FULL, R.first_id, L);
-  float ft = __shfl_sync(FULL, R.first_t, L);
+  return warp_min_u64(best);
+}
+
+// The whole warp on one list, [beg, end), for the transparent ray of lane L with
+// transmittance T: composites the voxel's hits into the ray's colour and first
+// hit and returns its transmittance.
+template <bool COUNT, bool KEY16, bool AO>
+__device__ __noinline__ float voxel_composite(const TraceArgs& A, WarpMem<false, KEY16>& S, int L,
+                                              uint32_t beg, uint32_t end, float T, unsigned& n_cap,
+                                              unsigned& n_hit, unsigned& n_scan) {
+  const int lane = threadIdx.x & 31;
+  const float4 o4 = S.o[L], d4 = S.d[L];
+  const float3 o = f3(o4), d = f3(d4);
+  const float t0 = o4.w, t1 = d4.w;
+  const float r2 = A.g.r * A.g.r;
+  const float rrm = (A.g.r + 1e-3f) * (A.g.r + 1e-3f);
+  const float4 acc = S.acc[L];
+  float C0 = acc.x, C1 = acc.y, C2 = acc.z, ft = acc.w;
+  int fid = __float_as_int(S.inv[L].w);
   const float om = 1.0f - A.alpha;
   unsigned long long last = 0ull;  // keys <= last are composited
   bool rescan = true;
@@ -457,7 +561,7 @@ __device__ void process_voxel(const TraceArgs& A, Ray& R, int L) {
 #pragma unroll
     for (int q = 0; q < kLaneKeys; ++q) buf[q] = ~0ull;
     bool dropped = false;
-    if (COUNT && lane == L) R.n_ww_ent += end - beg;
+    if (COUNT) n_scan += end - beg;
     for (uint32_t s = beg + lane; s < end; s += 32) {
       const unsigned long long k = entry_key<COUNT, KEY16>(A, s, beg, o, d, t0, t1, r2, rrm, n_cap);
       if (COUNT && k != ~0ull) ++n_hit;
@@ -502,7 +606,7 @@ __device__ void process_voxel(const TraceArgs& A, Ray& R, int L) {
       if (lane < n_out) {
         const uint32_t id = (uint32_t)(mine & 0xffffffffu);
         tq = hit_depth<KEY16>(A, mine, o, d);
-        c = tangent_colour(A, id);
+        c = tangent_colour(f3(__ldg(&A.pos[id])), f3(__ldg(&A.pos[id + 1])));
         if (A.ao) c = hit_shade<AO>(A, o + tq * d) * c;
       }
       // accumulate in key order
@@ -526,53 +630,61 @@ __device__ void process_voxel(const TraceArgs& A, Ray& R, int L) {
     // a rescan is needed only when the extraction stopped at the drop limit
     rescan = rescan && T >= kTStop && last == lim;
   }
-  if (COUNT) {
-    R.n_cap += n_cap;
-    R.n_hits += n_hit;
-  }
+  __syncwarp();  // every lane has read the ray's state
   if (lane == L) {
-    R.T = T;
-    R.C[0] = C0; R.C[1] = C1; R.C[2] = C2;
-    R.first_id = fid;
-    R.first_t = ft;
-    if (T < kTStop) R.active = false;
+    S.acc[L] = make_float4(C0, C1, C2, ft);
+    S.inv[L].w = __int_as_float(fid);
   }
+  return T;
 }
 
 // The pending voxels of the warp's lanes with lists up to A.short_list
-// entries, processed together. Lanes whose rays wait in the same voxel form a
-// group (neighbouring rays of the tile usually do); the entries of the
-// groups' distinct lists are numbered one after another and the warp takes 32
-// at a time, one entry per lane (two such rounds per step), so short lists do
-// not wait for the longest one. A lane loads its entry (segment id and end
-// points) once and line-tests it against every ray of the entry's group in
-// turn. Pairs that pass the line-distance test are queued per warp
-// in shared memory and get the capsule test 32 at a time. A hit goes to its ray's slots in shared memory
-// (the nearest key for an opaque ray; up to kRayKeys keys of a transparent
-// ray, sorted and composited by the ray's own lane afterwards). A transparent
-// ray with more hits in the voxel keeps its voxel pending for the whole-warp
-// path, which starts it again from scratch.
+// entries, processed together. Lanes whose rays wait in the same voxel form
+// groups of up to kGroup; a unit of work is one entry for one group. The units of
+// all groups are numbered one after another and the warp takes 64 at a time, two
+// per lane, so short lists do not wait for the longest one. A lane loads its
+// units' entries (segment id and end points) and line-tests them against the rays
+// of their groups; only the pairs that pass are compacted into the warp's queue,
+// which gets the capsule test 32 at a time. A hit is shaded by the lane that
+// found it. An opaque ray keeps its nearest key; a transparent ray's hits go to
+// the warp's pool, where they are ranked by key for the ray's own lane to
+// composite. Rays join a round only while their lists sum to kRoundPairs pairs;
+// a ray with a hit that found the pool full takes its voxel again in parts of its
+// interval. `wait` is set for lanes whose voxel the next round takes; a lane left
+// pending without it (more than A.ray_keys hits, or the pool full with 16+16 keys)
+// goes to the whole-warp path, which starts its voxel again from scratch.
 template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
-__device__ void process_flat(const TraceArgs& A, Ray& R) {
-  extern __shared__ unsigned long long s_key[];  // [kRayKeys][kTraceThreads]
-  __shared__ float4 s_ray[2][kTraceThreads];      // (o, t_enter), (d, t_exit)
-  __shared__ uint32_t s_cnt[kTraceThreads];
-  __shared__ unsigned long long s_best[kTraceThreads];
-  __shared__ uint2 s_q[kTraceThreads / 32][64];   // (segment id, owner lane) queued for the capsule test
+__device__ __forceinline__ void process_flat(const TraceArgs& A, WarpMem<OPAQUE, KEY16>& S, Ray& R, Work& W,
+                                             bool& wait) {
   const int lane = threadIdx.x & 31;
-  const int tid = threadIdx.x, wb = tid & ~31;
   const unsigned lt = (1u << lane) - 1u;
-  const bool take = R.pending && R.end - R.beg <= A.short_list;
-  const uint32_t len = take ? R.end - R.beg : 0u;
-  // group of lanes waiting in the same voxel (same list start); its lowest
-  // lane numbers the list's entries. Opaque rays mostly end in their first
-  // listed voxel, so their groups are small: each ray is its own group there.
-  unsigned gm = take ? 1u << lane : 0u;
-  if (!OPAQUE) {
-    const unsigned tm = __ballot_sync(FULL, take);
-    gm = __match_any_sync(FULL, take ? R.beg : 0xffffffffu) & (take ? tm : 0u);
+  bool take = R.pending && R.len <= A.short_list;
+  wait = false;
+  if (!OPAQUE && __reduce_add_sync(FULL, take ? R.len : 0u) > kRoundPairs) {
+    uint32_t sum = take ? R.len : 0u;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(FULL, sum, o);
+      if (lane >= o) sum += v;
+    }
+    if (take && sum - R.len >= kRoundPairs) {  // the next round's
+      take = false;
+      wait = true;
+    }
   }
-  const uint32_t glen = (take && __ffs(gm) - 1 == lane) ? len : 0u;
+  // Lanes waiting in the same voxel (same list start) form groups of at most
+  // kGroup; a group's lowest lane numbers the list's entries for it.
+  const unsigned tm = __ballot_sync(FULL, take);
+  const unsigned same = __match_any_sync(FULL, take ? R.beg : 0xffffffffu) & (take ? tm : 0u);
+  const bool leads = take && __popc(same & lt) % kGroup == 0;
+  unsigned gm = same & ~lt;  // from a leader on: its group's lanes
+  {
+    unsigned rest = gm;
+#pragma unroll
+    for (int q = 0; q < kGroup; ++q) rest &= rest - 1;
+    gm ^= rest;
+  }
+  const uint32_t glen = leads ? R.len : 0u;
   uint32_t incl = glen;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
@@ -580,196 +692,256 @@ __device__ void process_flat(const TraceArgs& A, Ray& R) {
     if (lane >= o) incl += v;
   }
   const uint32_t total = __shfl_sync(FULL, incl, 31);
-  if (total == 0) return;
-  if (take) {
-    s_ray[0][tid] = make_float4(R.o.x, R.o.y, R.o.z, R.vt0);
-    s_ray[1][tid] = make_float4(R.d.x, R.d.y, R.d.z, R.vt1);
-  }
-  if (OPAQUE) s_best[tid] = ~0ull;
-  else s_cnt[tid] = 0u;
+  if (OPAQUE) S.key[lane] = ~0ull;
+  else S.cnt[lane] = 0u;
   __syncwarp();
   const uint32_t first = R.beg - (incl - glen);  // entry g of a group's list is lists[first + g]
   const float r2 = A.g.r * A.g.r;
   const float rrm = (A.g.r + 1e-3f) * (A.g.r + 1e-3f);
-  unsigned n_cap = 0, n_hit = 0;
-  uint2* q = s_q[tid >> 5];
-  uint32_t qn = 0;  // queued pairs (warp-uniform)
-  // capsule test of queued pair `lane` for lanes below cnt
-  auto capsule_stage = [&](uint32_t cnt) {
+  uint32_t qn = 0, pn = 0;  // queued pairs, hits of the round (warp-uniform)
+  // capsule test of queued pair q0 + lane for lanes below cnt
+  auto capsule_stage = [&](uint32_t q0, uint32_t cnt) {
     const long long c0 = COUNT ? clock64() : 0;
+    bool hit = false;
+    unsigned long long k = 0;
+    float3 c = make_float3(0.0f, 0.0f, 0.0f);
+    int j = 0;
     if ((uint32_t)lane < cnt) {
-      const uint2 it = q[lane];
-      const uint32_t id = it.x;
-      const int j = (int)(it.y & 255u);
+      const uint32_t it = S.q[q0 + lane];
+      const uint32_t id = S.uid[it & 127u];
+      j = (int)(it >> 8);
       const float4 p0 = __ldg(&A.pos[id]), p1 = __ldg(&A.pos[id + 1]);
-      const float4 ro = s_ray[0][wb + j], rd = s_ray[1][wb + j];
-      if (COUNT) ++n_cap;
+      const float4 ro = S.o[j], rd = S.d[j];
+      if (COUNT) ++W.cap;
       const float t = capsule_entry(f3(ro), f3(rd), f3(p0), f3(p1), r2);
       if (t >= ro.w && t < rd.w && clip_keeps(A, f3(ro) + t * f3(rd), p0, p1, id)) {
-        const unsigned long long k = hit_key<KEY16>(t, id, it.y >> 8, ro.w, rd.w);
-        if (COUNT) ++n_hit;
-        if (OPAQUE) {
-          atomicMin(&s_best[wb + j], k);
-        } else {
-          const uint32_t slot = atomicAdd(&s_cnt[wb + j], 1u);
-          if (slot < A.ray_keys) s_key[slot * kTraceThreads + wb + j] = k;
+        hit = true;
+        k = hit_key<KEY16>(t, id, KEY16 ? S.uli[it & 127u] : 0u, ro.w, rd.w);
+        if (COUNT) ++W.hits;
+        if (!OPAQUE) {
+          c = tangent_colour(f3(p0), f3(p1));
+          if (A.ao) c = hit_shade<AO>(A, f3(ro) + t * f3(rd)) * c;
         }
       }
     }
-    if (COUNT) R.cyc[3] += (unsigned long long)(clock64() - c0);
+    if (OPAQUE) {
+      if (hit) atomicMin(&S.key[j], k);
+    } else {
+      const unsigned hm = __ballot_sync(FULL, hit);
+      if (hit) {
+        const uint32_t slot = pn + __popc(hm & lt);
+        const uint32_t nth = atomicAdd(&S.cnt[j], 1u);
+        if (slot < kPool) {
+          S.key[slot] = k;
+          S.col[0][slot] = c.x;
+          S.col[1][slot] = c.y;
+          S.col[2][slot] = c.z;
+          S.own[slot] = (uint16_t)((uint32_t)j | (nth << 8));
+        } else {
+          atomicOr(&S.cnt[j], kLost);
+        }
+      }
+      pn += __popc(hm);
+    }
+    if (COUNT) W.cyc[3] += (unsigned long long)(clock64() - c0);
   };
-  auto owner = [&](uint32_t gq) {
-    int j = 0;
+  // a unit of work: one entry and the rays of its group
+  struct Unit {
+    uint32_t s, id, li;
+    unsigned m;
+    float4 p0, p1;
+  };
+  auto find_unit = [&](uint32_t gq, Unit& u) {
+    u.m = u.id = u.li = u.s = 0;
+    if (__all_sync(FULL, gq >= total)) return;
+    int j = 0;  // the leader that numbers unit gq
 #pragma unroll
     for (int st = 16; st > 0; st >>= 1)
       if (__shfl_sync(FULL, incl, j + st - 1) <= gq) j += st;
-    return min(j, 31);
+    j = min(j, 31);
+    u.s = __shfl_sync(FULL, first, j) + gq;
+    u.m = __shfl_sync(FULL, gm, j);
+    if (KEY16) u.li = u.s - __shfl_sync(FULL, R.beg, j);
+    if (gq < total) u.id = __ldg(&A.g.lists[u.s]);
+    else u.m = 0;
   };
-  // queue entry: segment id, owner lane j | list index li << 8 (16+16 keys)
-  auto append = [&](bool pass, uint32_t id, int j, uint32_t li) {
-    const unsigned m = __ballot_sync(FULL, pass);
-    if (pass) q[qn + __popc(m & lt)] = make_uint2(id, (uint32_t)j | (li << 8));
-    qn += __popc(m);
-    if (qn >= 32) {
-      __syncwarp();
-      capsule_stage(32);
-      __syncwarp();
-      if ((uint32_t)lane < qn - 32) q[lane] = q[32 + lane];
-      __syncwarp();
-      qn -= 32;
+  auto load_unit = [&](Unit& u) {
+    if (u.m && u.id + 1 >= A.n_vert) {
+      set_err(A.g.st, kErrBounds);
+      u.m = 0;
     }
-  };
-  // line tests of a loaded entry against the rays in mask m, one per round
-  auto test_group = [&](unsigned m, uint32_t id, float4 p0, float4 p1, uint32_t li) {
-    while (__any_sync(FULL, m)) {
-      bool pass = false;
-      int j = 0;
-      if (m) {
-        j = __ffs(m) - 1;
-        m &= m - 1;
-        const float4 ro = s_ray[0][wb + j], rd = s_ray[1][wb + j];
-        pass = lines_may_meet(f3(ro), f3(rd), f3(p0), f3(p1), rrm);
-      }
-      append(pass, id, j, li);
+    u.p0 = u.p1 = make_float4(0.f, 0.f, 0.f, 0.f);
+    if (u.m) {
+      u.p0 = __ldg(&A.pos[u.id]);
+      u.p1 = __ldg(&A.pos[u.id + 1]);
+      if (COUNT) { touch(A.touch_list, u.s); touch(A.touch_vert, u.id); touch(A.touch_vert, u.id + 1); }
     }
   };
-  // two independent (owner search, list load, vertex loads) chains per step:
-  // the loads' latency is paid once per entry, whatever its group's size
-  if (OPAQUE) {
-    for (uint32_t t0 = 0; t0 < total; t0 += 64) {
-      const uint32_t ga = t0 + lane, gb = ga + 32;
-      const int ja = owner(ga), jb = owner(gb);
-      const uint32_t fa = __shfl_sync(FULL, first, ja), fb = __shfl_sync(FULL, first, jb);
-      const bool va = ga < total, vb = gb < total;
-      uint32_t ida = 0, idb = 0;
-      if (va) ida = __ldg(&A.g.lists[fa + ga]);
-      if (vb) idb = __ldg(&A.g.lists[fb + gb]);
-      const bool oka = va && ida + 1 < A.n_vert, okb = vb && idb + 1 < A.n_vert;
-      if ((va && !oka) || (vb && !okb)) set_err(A.g.st, kErrBounds);
-      float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0, b0 = a0, b1 = a0;
-      if (oka) { a0 = __ldg(&A.pos[ida]); a1 = __ldg(&A.pos[ida + 1]); }
-      if (okb) { b0 = __ldg(&A.pos[idb]); b1 = __ldg(&A.pos[idb + 1]); }
-      if (COUNT) {
-        if (oka) { touch(A.touch_list, fa + ga); touch(A.touch_vert, ida); touch(A.touch_vert, ida + 1); }
-        if (okb) { touch(A.touch_list, fb + gb); touch(A.touch_vert, idb); touch(A.touch_vert, idb + 1); }
-      }
-      bool pa = false, pb = false;
-      if (oka) {
-        const float4 ro = s_ray[0][wb + ja], rd = s_ray[1][wb + ja];
-        pa = lines_may_meet(f3(ro), f3(rd), f3(a0), f3(a1), rrm);
-      }
-      if (okb) {
-        const float4 ro = s_ray[0][wb + jb], rd = s_ray[1][wb + jb];
-        pb = lines_may_meet(f3(ro), f3(rd), f3(b0), f3(b1), rrm);
-      }
-      uint32_t la = 0, lb = 0;  // list indices (16+16 keys)
-      if (KEY16) {
-        la = fa + ga - __shfl_sync(FULL, R.beg, ja);
-        lb = fb + gb - __shfl_sync(FULL, R.beg, jb);
-      }
-      append(pa, ida, ja, la);
-      append(pb, idb, jb, lb);
+  // line-tests the unit's entry against its rays; the rays that pass
+  auto line_tests = [&](const Unit& u) {
+    unsigned m = u.m, pm = 0;
+    while (m) {  // two rays at a time: independent chains
+      const int j0 = __ffs(m) - 1;
+      m &= m - 1;
+      const int j1 = m ? __ffs(m) - 1 : j0;
+      m &= m - 1;
+      const float4 o0 = S.o[j0], d0 = S.d[j0], o1 = S.o[j1], d1 = S.d[j1];
+      const bool m0 = lines_may_meet(f3(o0), f3(d0), f3(u.p0), f3(u.p1), rrm);
+      const bool m1 = lines_may_meet(f3(o1), f3(d1), f3(u.p0), f3(u.p1), rrm);
+      pm |= (m0 ? 1u << j0 : 0u) | (m1 ? 1u << j1 : 0u);
     }
-  } else for (uint32_t t0 = 0; t0 < total; t0 += 64) {
-    const uint32_t ga = t0 + lane, gb = ga + 32;
-    const int ja = owner(ga), jb = owner(gb);
-    const uint32_t fa = __shfl_sync(FULL, first, ja), fb = __shfl_sync(FULL, first, jb);
-    const unsigned ma = __shfl_sync(FULL, gm, ja), mb = __shfl_sync(FULL, gm, jb);
-    const bool va = ga < total, vb = gb < total;
-    uint32_t ida = 0, idb = 0;
-    if (va) ida = __ldg(&A.g.lists[fa + ga]);
-    if (vb) idb = __ldg(&A.g.lists[fb + gb]);
-    const bool oka = va && ida + 1 < A.n_vert, okb = vb && idb + 1 < A.n_vert;
-    if ((va && !oka) || (vb && !okb)) set_err(A.g.st, kErrBounds);
-    float4 a0 = make_float4(0.f, 0.f, 0.f, 0.f), a1 = a0, b0 = a0, b1 = a0;
-    if (oka) { a0 = __ldg(&A.pos[ida]); a1 = __ldg(&A.pos[ida + 1]); }
-    if (okb) { b0 = __ldg(&A.pos[idb]); b1 = __ldg(&A.pos[idb + 1]); }
-    if (COUNT) {
-      if (oka) { touch(A.touch_list, fa + ga); touch(A.touch_vert, ida); touch(A.touch_vert, ida + 1); }
-      if (okb) { touch(A.touch_list, fb + gb); touch(A.touch_vert, idb); touch(A.touch_vert, idb + 1); }
-    }
-    uint32_t la = 0, lb = 0;  // list indices (16+16 keys)
+    return pm;
+  };
+  // Two units per lane and step, so that their load chains overlap; the next
+  // step's segment ids are on their way while this step's pairs are tested. The
+  // lanes' passing pairs go to the queue at places given by a prefix sum of
+  // their numbers. The capsule test stands at one place: copies of it for each
+  // unit and for the last, partial batch made the loop's code outgrow the
+  // instruction cache (5 of 13 stall cycles per instruction on the bundles).
+  Unit a, b;
+  find_unit(lane, a);
+  find_unit(32 + lane, b);
+  uint32_t tab = 0;  // this step's half of the unit table
+  for (uint32_t t0 = 0; t0 < total; t0 += 64) {
+    const bool last = t0 + 64 >= total;
+    load_unit(a);
+    load_unit(b);
+    S.uid[tab + lane] = a.id;
+    S.uid[tab + 32 + lane] = b.id;
     if (KEY16) {
-      la = fa + ga - __shfl_sync(FULL, R.beg, ja);
-      lb = fb + gb - __shfl_sync(FULL, R.beg, jb);
+      S.uli[tab + lane] = (uint16_t)a.li;
+      S.uli[tab + 32 + lane] = (uint16_t)b.li;
     }
-    test_group(oka ? ma : 0u, ida, a0, a1, la);
-    test_group(okb ? mb : 0u, idb, b0, b1, lb);
+    Unit na, nb;
+    na.m = nb.m = na.id = nb.id = na.li = nb.li = na.s = nb.s = 0;
+    if (!last) {
+      find_unit(t0 + 64 + lane, na);
+      find_unit(t0 + 96 + lane, nb);
+    }
+    unsigned pa = line_tests(a), pb = line_tests(b);
+    const uint32_t np = __popc(pa) + __popc(pb);
+    uint32_t at = np;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t v = __shfl_up_sync(FULL, at, o);
+      if (lane >= o) at += v;
+    }
+    const uint32_t end = qn + __shfl_sync(FULL, at, 31);
+    at += qn - np;
+    for (; pa; pa &= pa - 1) S.q[at++] = (uint16_t)((tab + lane) | (uint32_t)(__ffs(pa) - 1) << 8);
+    for (; pb; pb &= pb - 1) S.q[at++] = (uint16_t)((tab + 32 + lane) | (uint32_t)(__ffs(pb) - 1) << 8);
+    __syncwarp();
+    // full batches, and what is left of the last step's units: the next step
+    // overwrites their half of the table
+    const uint32_t must = last ? end : qn;
+    uint32_t done = 0;
+    while (end - done >= 32 || done < must) {
+      capsule_stage(done, min(end - done, 32u));
+      done = min(done + 32, end);
+    }
+    qn = end - done;  // below 32: to the front for the next step
+    const uint16_t rest = S.q[done + min((uint32_t)lane, qn)];
+    __syncwarp();
+    if ((uint32_t)lane < qn) S.q[lane] = rest;
+    a = na;
+    b = nb;
+    tab ^= 64u;
   }
   __syncwarp();
-  capsule_stage(qn);
-  __syncwarp();
-  if (COUNT) {
-    R.n_cap += n_cap;
-    R.n_hits += n_hit;
-  }
-  if (!take) return;
   if (OPAQUE) {
+    if (!take) return;
     if (COUNT) {
-      ++R.n_vox;
-      R.n_entries += len;
+      ++W.vox;
+      W.entries += R.len;
     }
-    const unsigned long long best = s_best[tid];
-    if (best != ~0ull) {
-      const uint32_t id = (uint32_t)(best & 0xffffffffu);
-      opaque_hit(A, R, id, hit_depth<KEY16>(A, best, R.o, R.d));
-    }
+    const unsigned long long best = S.key[lane];
+    if (best != ~0ull)
+      opaque_hit(A, S, R, (uint32_t)(best & 0xffffffffu),
+                 hit_depth<KEY16>(A, best, f3(S.o[lane]), f3(S.d[lane])));
     R.pending = false;
     if (R.t1 < 0.0f) R.active = false;
     return;
   }
-  const uint32_t nk = s_cnt[tid];
-  if (nk > A.ray_keys) return;  // stays pending: the whole-warp path redoes it
+  bool redo = false;  // the ray's voxel is not composited in this round
+  if (pn) {
+    const uint32_t raw = S.cnt[lane];
+    redo = (raw & ~kLost) > A.ray_keys || (raw & kLost);
+    if (take && redo) {
+      // Hits past the pool: the ray takes the voxel again up to a depth before
+      // which the pool should hold every ray's hits, and then the rest. (The
+      // 16+16 key quantizes depths over the whole interval, and a limit on a
+      // ray's hits asks for the whole-warp path.)
+      const float a = S.o[lane].w, b = S.d[lane].w;
+      const float m = fmaf(b - a, 0.4f * (float)kPool / (float)pn, a);
+      wait = !KEY16 && (raw & ~kLost) <= A.ray_keys && m > a && m < b;
+      S.d[lane].w = wait ? m : R.tcur;
+    }
+    const uint32_t nk = redo ? 0u : raw;
+    const uint32_t hits = min(pn, kPool);
+    uint32_t off = lane;
+    if (__any_sync(FULL, raw > 1u)) {
+      // pool slots ray after ray, then each ray's by key: a hit's place is the
+      // number of its ray's hits with smaller keys
+      off = nk;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(FULL, off, o);
+        if (lane >= o) off += v;
+      }
+      off -= nk;
+      for (uint32_t q0 = 0; q0 < hits; q0 += 32) {
+        const uint32_t q = q0 + lane;
+        const uint32_t ow = q < hits ? S.own[q] : 0u;
+        const uint32_t oo = __shfl_sync(FULL, off, ow & 31u), on = __shfl_sync(FULL, nk, ow & 31u);
+        if (q < hits && on) S.slot[oo + (ow >> 8)] = (uint8_t)q;
+      }
+      __syncwarp();
+      for (uint32_t q0 = 0; q0 < hits; q0 += 32) {
+        const uint32_t q = q0 + lane;
+        const uint32_t ow = q < hits ? S.own[q] : 0u;
+        const uint32_t oo = __shfl_sync(FULL, off, ow & 31u), on = __shfl_sync(FULL, nk, ow & 31u);
+        if (q < hits && on) {
+          const unsigned long long k = S.key[q];
+          uint32_t place = 0;
+          for (uint32_t i = 0; i < on; ++i) place += S.key[S.slot[oo + i]] < k;
+          S.order[oo + place] = (uint8_t)q;
+        }
+      }
+    } else if (lane < hits) {
+      S.order[S.own[lane] & 31u] = (uint8_t)lane;  // at most one hit a ray, so at most 32
+    }
+    __syncwarp();
+    if (nk) {
+      float4 acc = S.acc[lane];
+      const float om = 1.0f - A.alpha;
+      float T = R.T;
+      for (uint32_t i = 0; i < nk && T >= kTStop; ++i) {
+        const uint32_t q = S.order[off + i];
+        const float w = T * A.alpha;
+        acc.x = fmaf(w, S.col[0][q], acc.x);
+        acc.y = fmaf(w, S.col[1][q], acc.y);
+        acc.z = fmaf(w, S.col[2][q], acc.z);
+        T *= om;
+        if (i == 0 && __float_as_int(S.inv[lane].w) < 0) {
+          const unsigned long long k = S.key[q];
+          S.inv[lane].w = __uint_as_float((uint32_t)(k & 0xffffffffu));
+          acc.w = hit_depth<KEY16>(A, k, f3(S.o[lane]), f3(S.d[lane]));
+        }
+      }
+      R.T = T;
+      S.acc[lane] = acc;
+    }
+  }
+  if (!take || redo) return;
+  if (!KEY16 && R.T >= kTStop && S.d[lane].w < R.tcur) {  // the rest of the voxel's interval
+    S.o[lane].w = S.d[lane].w;
+    S.d[lane].w = R.tcur;
+    wait = true;
+    return;
+  }
   if (COUNT) {
-    ++R.n_vox;
-    R.n_entries += len;
-  }
-  unsigned long long* kb = s_key + tid;
-  for (uint32_t q = 1; q < nk; ++q) {
-    const unsigned long long k = kb[q * kTraceThreads];
-    uint32_t p = q;
-    while (p > 0 && kb[(p - 1) * kTraceThreads] > k) {
-      kb[p * kTraceThreads] = kb[(p - 1) * kTraceThreads];
-      --p;
-    }
-    kb[p * kTraceThreads] = k;
-  }
-  const float om = 1.0f - A.alpha;
-  for (uint32_t q = 0; q < nk && R.T >= kTStop; ++q) {
-    const unsigned long long kq = kb[q * kTraceThreads];
-    const uint32_t id = (uint32_t)(kq & 0xffffffffu);
-    const float t = hit_depth<KEY16>(A, kq, R.o, R.d);
-    float3 c = tangent_colour(A, id);
-    if (A.ao) c = hit_shade<AO>(A, R.o + t * R.d) * c;
-    const float w = R.T * A.alpha;
-    R.C[0] = fmaf(w, c.x, R.C[0]);
-    R.C[1] = fmaf(w, c.y, R.C[1]);
-    R.C[2] = fmaf(w, c.z, R.C[2]);
-    R.T *= om;
-    if (R.first_id < 0) {
-      R.first_id = (int)id;
-      R.first_t = t;
-    }
+    ++W.vox;
+    W.entries += R.len;
   }
   R.pending = false;
   if (R.T < kTStop || R.t1 < 0.0f) R.active = false;
@@ -785,288 +957,220 @@ __device__ __forceinline__ void lap(unsigned long long& c, long long& t) {
   }
 }
 
+// Trace the rays of the warp's lanes to their ends.
 template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
-__device__ void trace_warp(const TraceArgs& A, Ray& R) {
+__device__ __forceinline__ void trace_warp(const TraceArgs& A, WarpMem<OPAQUE, KEY16>& S, Ray& R, Work& W) {
   const int lane = threadIdx.x & 31;
   long long t = COUNT ? clock64() : 0;
   for (;;) {
     if (R.active && !R.pending) {
-      const int rc = advance<COUNT>(A, R, kStepRound);
+      const int rc = walk_brick<WarpMem<OPAQUE, KEY16>, COUNT>(A, S, R, W);
       R.pending = rc == 1;
       if (rc == 0) R.active = false;
     }
-    // The warp steps its walking rays one voxel (or empty cube) per round and
+    // The warp walks its rays one brick (or empty cube) per round and
     // processes the waiting lists once a quarter of the rays still in flight
-    // wait at one (or none can step on). Stepping each ray to its next list in
-    // one go left most lanes idle while the longest walk went on (5.9 of 32
-    // lanes active per instruction on a sparse 512^3 set): bounded rounds cut
-    // that trace by 41-47% and the dense bundles' by 4%.
+    // wait at one (or none can walk on): walking each ray to its next list in
+    // one go leaves most lanes idle while the longest walk goes on.
     const unsigned pend = __ballot_sync(FULL, R.pending);
     const unsigned walk = __ballot_sync(FULL, R.active && !R.pending);
     if (!pend && !walk) break;
     if (walk && 4 * __popc(pend) < __popc(pend | walk)) continue;
-    lap<COUNT>(R.cyc[0], t);
-    process_flat<OPAQUE, COUNT, KEY16, AO>(A, R);
-    lap<COUNT>(R.cyc[1], t);
-    // long lists: the whole warp on one list at a time
-    unsigned pm = __ballot_sync(FULL, R.pending);
-    while (pm) {
-      const int L = __ffs(pm) - 1;
-      pm &= pm - 1;
-      process_voxel<OPAQUE, COUNT, KEY16, AO>(A, R, L);
-      if (lane == L) {
-        R.pending = false;
-        if (R.t1 < 0.0f) R.active = false;
-      }
-    }
-    lap<COUNT>(R.cyc[2], t);
-  }
-  lap<COUNT>(R.cyc[0], t);
-}
-
-template <bool COUNT>
-__device__ __forceinline__ void finish(const TraceArgs& A, const Ray& R, bool valid) {
-  if (COUNT) {
-    unsigned long long e = R.n_entries, c = R.n_cap, v = R.n_vox, st = R.n_steps;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      e += __shfl_xor_sync(FULL, e, o);
-      c += __shfl_xor_sync(FULL, c, o);
-      v += __shfl_xor_sync(FULL, v, o);
-      st += __shfl_xor_sync(FULL, st, o);
-    }
-    unsigned long long h = R.n_hits, wv = R.n_ww_vox, we = R.n_ww_ent;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      h += __shfl_xor_sync(FULL, h, o);
-      wv += __shfl_xor_sync(FULL, wv, o);
-      we += __shfl_xor_sync(FULL, we, o);
-    }
-    if ((threadIdx.x & 31) == 0) {
-      atomicAdd(&A.g.st->tr_entries, e);
-      atomicAdd(&A.g.st->tr_capsule, c);
-      atomicAdd(&A.g.st->tr_voxels, v);
-      atomicAdd(&A.g.st->tr_steps, st);
-      atomicAdd(&A.g.st->tr_hits, h);
-      atomicAdd(&A.g.st->tr_ww_voxels, wv);
-      atomicAdd(&A.g.st->tr_ww_entries, we);
-      for (int k = 0; k < 4; ++k) atomicAdd(&A.g.st->tr_cycles[k], R.cyc[k]);
-    }
-  }
-  if (!valid) return;
-  if (R.missed) {
-    const uint32_t q = atomicAdd(A.pq_cnt, 1u);
-    if (q < A.pq_cap) A.pq[q] = R.pix;
-    else set_err(A.g.st, kErrOverflow);
-    return;
-  }
-  A.rgba[R.pix] = make_float4(R.C[0], R.C[1], R.C[2], 1.0f - R.T);
-  if (A.first_id) A.first_id[R.pix] = R.first_id;
-  if (A.first_t) A.first_t[R.pix] = R.first_t;
-}
-
-// Transparent main trace: each warp owns one fixed tile of 32 pixels, TW wide
-// and 32 / TW tall (a block 2x2 tiles), and its lanes write their pixels
-// together at the end. Measured faster than persistent refilling here, since
-// the tile's rays share lists. The tile shape is a tuned parameter (default
-// 4 x 8, measured slightly faster than 8 x 4 or 16 x 2 on the bundles frame).
-template <bool OPAQUE, bool COUNT, bool KEY16, bool AO, int TW>
-__global__ void __launch_bounds__(kTraceThreads, COUNT ? 1 : 4) k_trace_tile(TraceArgs A) {
-  constexpr int TH = 32 / TW;
-  const int lane = threadIdx.x & 31;
-  const int warp = threadIdx.x >> 5;
-  const int px = blockIdx.x * (2 * TW) + (warp & 1) * TW + (lane % TW);
-  const int py = blockIdx.y * (2 * TH) + (warp >> 1) * TH + (lane / TW);
-  const bool valid = px < A.cam.width && py < A.cam.height;
-  Ray R;
-  R.cyc[0] = R.cyc[1] = R.cyc[2] = R.cyc[3] = 0;
-  R.pix = valid ? (uint32_t)(py * A.cam.width + px) : 0u;
-  init_ray(A, R, px, py, valid);
-  trace_warp<OPAQUE, COUNT, KEY16, AO>(A, R);
-  finish<COUNT>(A, R, valid);
-}
-
-// Write a finished pixel (or queue it for the repair re-trace).
-__device__ __forceinline__ void write_pixel(const TraceArgs& A, const Ray& R) {
-  if (R.missed) {
-    const uint32_t q = atomicAdd(A.pq_cnt, 1u);
-    if (q < A.pq_cap) A.pq[q] = R.pix;
-    else set_err(A.g.st, kErrOverflow);
-    return;
-  }
-  A.rgba[R.pix] = make_float4(R.C[0], R.C[1], R.C[2], 1.0f - R.T);
-  if (A.first_id) A.first_id[R.pix] = R.first_id;
-  if (A.first_t) A.first_t[R.pix] = R.first_t;
-}
-
-// Opaque and repair traces use persistent warps: a lane whose ray is finished
-// writes its pixel and goes idle; idle lanes take the next work items (one
-// atomic per refill). Work item w of the image is pixel (w mod 32) of the
-// (w / 32)-th 8x4 tile, so a full refill is a coherent tile; in the repair
-// re-trace, item w is the w-th queued pixel.
-template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
-__global__ void __launch_bounds__(kTraceThreads, COUNT ? 1 : (OPAQUE ? 5 : 4)) k_trace(TraceArgs A) {
-  const int lane = threadIdx.x & 31;
-  const uint32_t W = (uint32_t)A.cam.width, H = (uint32_t)A.cam.height;
-  const uint32_t tiles_x = (W + 7) / 8;
-  const uint32_t total = A.pix_list ? min(*A.pix_count, A.pq_cap) : tiles_x * ((H + 3) / 4) * 32u;
-  Ray R;
-  R.active = R.pending = false;
-  R.n_steps = R.n_entries = R.n_cap = R.n_vox = 0;
-  R.n_hits = R.n_ww_vox = R.n_ww_ent = 0;
-  R.cyc[0] = R.cyc[1] = R.cyc[2] = R.cyc[3] = 0;
-  unsigned c_steps = 0, c_entries = 0, c_cap = 0, c_vox = 0, c_hits = 0, c_wwv = 0, c_wwe = 0;
-  long long tclk = COUNT ? clock64() : 0;
-  bool has = false;
-  // Opaque main trace: refill once half the warp is idle. Queued repair
-  // pixels are scattered: a warp takes at most its share of the queue, one
-  // pixel each when few are queued.
-  const uint32_t n_warps = gridDim.x * (blockDim.x >> 5);
-  const int threshold = A.pix_list ? 1 : 16;
-  const int cap = A.pix_list ? (int)min(32u, max(1u, (total + n_warps - 1) / n_warps)) : 32;
-  for (;;) {
-    const unsigned idle = __ballot_sync(FULL, !has);
-    bool exhausted = false;
-    if (__popc(idle) >= threshold) {
-      const int take = min(__popc(idle), cap);
-      uint32_t base = 0;
-      if (lane == 0) base = atomicAdd(A.work_next, (uint32_t)take);
-      base = __shfl_sync(FULL, base, 0);
-      exhausted = base >= total;
-      const int rank = __popc(idle & ((1u << lane) - 1u));
-      if (!has && rank < take) {
-        const uint32_t w = base + (uint32_t)rank;
-        if (w < total) {
-          uint32_t px, py;
-          if (A.pix_list) {
-            const uint32_t pix = A.pix_list[w];
-            px = pix % W;
-            py = pix / W;
-          } else {
-            const uint32_t tile = w >> 5, within = w & 31u;
-            px = (tile % tiles_x) * 8 + (within & 7u);
-            py = (tile / tiles_x) * 4 + (within >> 3);
+    lap<COUNT>(W.cyc[0], t);
+    if (R.pending) resolve_list<WarpMem<OPAQUE, KEY16>, COUNT>(A, S, R);
+    __syncwarp();
+    bool more;
+    do {
+      bool wait;
+      process_flat<OPAQUE, COUNT, KEY16, AO>(A, S, R, W, wait);
+      lap<COUNT>(W.cyc[1], t);
+      // long lists: the whole warp on one list at a time
+      unsigned pm = __ballot_sync(FULL, R.pending && !wait);
+      while (pm) {
+        const int L = __ffs(pm) - 1;
+        pm &= pm - 1;
+        const uint32_t beg = __shfl_sync(FULL, R.beg, L), end = beg + __shfl_sync(FULL, R.len, L);
+        unsigned n_cap = 0, n_hit = 0, n_scan = 0;
+        if constexpr (OPAQUE) {
+          const unsigned long long best = voxel_nearest<COUNT, KEY16>(A, S, L, beg, end, n_cap, n_hit);
+          n_scan = end - beg;
+          if (lane == L && best != ~0ull)
+            opaque_hit(A, S, R, (uint32_t)(best & 0xffffffffu),
+                       hit_depth<KEY16>(A, best, f3(S.o[L]), f3(S.d[L])));
+        } else {
+          const float T = voxel_composite<COUNT, KEY16, AO>(A, S, L, beg, end,
+                                                            __shfl_sync(FULL, R.T, L), n_cap, n_hit, n_scan);
+          if (lane == L) {
+            R.T = T;
+            if (T < kTStop) R.active = false;
           }
-          if (px < W && py < H) {
-            if (COUNT) {
-              c_steps += R.n_steps; c_entries += R.n_entries; c_cap += R.n_cap; c_vox += R.n_vox;
-              c_hits += R.n_hits; c_wwv += R.n_ww_vox; c_wwe += R.n_ww_ent;
-            }
-            R.pix = py * W + px;
-            init_ray(A, R, (int)px, (int)py, true);
-            if (A.pix_list && A.resume) resume_ray(A, R);
-            has = true;
+        }
+        __syncwarp();
+        if (lane == L) {
+          R.pending = false;
+          if (R.t1 < 0.0f) R.active = false;
+        }
+        if (COUNT) {
+          W.cap += n_cap;
+          W.hits += n_hit;
+          if (lane == L) {
+            ++W.vox;
+            ++W.ww_vox;
+            W.entries += end - beg;
+            W.ww_ent += n_scan;
           }
         }
       }
-    }
-    if (!__any_sync(FULL, has)) {
-      if (__all_sync(FULL, exhausted)) break;
-      continue;
-    }
-    if (has && R.active && !R.pending) {
-      R.pending = advance<COUNT>(A, R, 3 * A.g.n + 16) == 1;
-      if (!R.pending) R.active = false;
-    }
-    lap<COUNT>(R.cyc[0], tclk);
-    process_flat<OPAQUE, COUNT, KEY16, AO>(A, R);
-    lap<COUNT>(R.cyc[1], tclk);
-    // long lists: the whole warp on one list at a time
-    unsigned pm = __ballot_sync(FULL, R.pending);
-    while (pm) {
-      const int L = __ffs(pm) - 1;
-      pm &= pm - 1;
-      process_voxel<OPAQUE, COUNT, KEY16, AO>(A, R, L);
-      if (lane == L) {
-        R.pending = false;
-        if (R.t1 < 0.0f) R.active = false;
-      }
-    }
-    lap<COUNT>(R.cyc[2], tclk);
-    if (has && !R.active && !R.pending) {
-      write_pixel(A, R);
-      has = false;
-    }
+      lap<COUNT>(W.cyc[2], t);
+      more = __any_sync(FULL, R.pending);
+    } while (more);
   }
-  if (COUNT) {
-    lap<COUNT>(R.cyc[0], tclk);
-    unsigned long long e = c_entries + R.n_entries, c = c_cap + R.n_cap, v = c_vox + R.n_vox,
-                       st = c_steps + R.n_steps, h = c_hits + R.n_hits, wv = c_wwv + R.n_ww_vox,
-                       we = c_wwe + R.n_ww_ent;
+  lap<COUNT>(W.cyc[0], t);
+}
+
+template <bool COUNT>
+__device__ __forceinline__ void count_work(const TraceArgs& A, const Work& W) {
+  if (!COUNT) return;
+  unsigned long long v[7] = {W.entries, W.cap, W.vox, W.steps, W.hits, W.ww_vox, W.ww_ent};
+  unsigned long long* out[7] = {&A.g.st->tr_entries, &A.g.st->tr_capsule, &A.g.st->tr_voxels,
+                                &A.g.st->tr_steps, &A.g.st->tr_hits, &A.g.st->tr_ww_voxels,
+                                &A.g.st->tr_ww_entries};
+  for (int i = 0; i < 7; ++i) {
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
-      e += __shfl_xor_sync(FULL, e, o);
-      c += __shfl_xor_sync(FULL, c, o);
-      v += __shfl_xor_sync(FULL, v, o);
-      st += __shfl_xor_sync(FULL, st, o);
-      h += __shfl_xor_sync(FULL, h, o);
-      wv += __shfl_xor_sync(FULL, wv, o);
-      we += __shfl_xor_sync(FULL, we, o);
-    }
-    if (lane == 0) {
-      atomicAdd(&A.g.st->tr_entries, e);
-      atomicAdd(&A.g.st->tr_capsule, c);
-      atomicAdd(&A.g.st->tr_voxels, v);
-      atomicAdd(&A.g.st->tr_steps, st);
-      atomicAdd(&A.g.st->tr_hits, h);
-      atomicAdd(&A.g.st->tr_ww_voxels, wv);
-      atomicAdd(&A.g.st->tr_ww_entries, we);
-      for (int k = 0; k < 4; ++k) atomicAdd(&A.g.st->tr_cycles[k], R.cyc[k]);
-    }
+    for (int o = 16; o > 0; o >>= 1) v[i] += __shfl_xor_sync(FULL, v[i], o);
+    if ((threadIdx.x & 31) == 0) atomicAdd(out[i], v[i]);
   }
+  if ((threadIdx.x & 31) == 0)
+    for (int k = 0; k < 4; ++k) atomicAdd(&A.g.st->tr_cycles[k], W.cyc[k]);
 }
 
-// Persistent grid: as many blocks as can be resident at once.
-template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
-int persistent_blocks(size_t smem) {
-  static int blocks = 0;  // per instantiation; the device does not change under a grid
-  if (!blocks) {
-    int dev = 0, sms = 0, per_sm = 0;
-    cudaGetDevice(&dev);
-    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_trace<OPAQUE, COUNT, KEY16, AO>, kTraceThreads, smem);
-    blocks = max(1, sms) * max(1, per_sm);
+// Write a finished pixel (or queue it for the repair re-trace).
+template <class M>
+__device__ __forceinline__ void write_pixel(const TraceArgs& A, const M& S, const Ray& R) {
+  const int lane = threadIdx.x & 31;
+  if (R.missed) {
+    const uint32_t q = atomicAdd(A.pq_cnt, 1u);
+    if (q < A.pq_cap) A.pq[q] = R.pix;
+    else set_err(A.g.st, kErrOverflow);
+    return;
   }
-  return blocks;
+  const float4 c = S.acc[lane];
+  A.rgba[R.pix] = make_float4(c.x, c.y, c.z, 1.0f - R.T);
+  if (A.first_id) A.first_id[R.pix] = __float_as_int(S.inv[lane].w);
+  if (A.first_t) A.first_t[R.pix] = c.w;
+}
+
+// Resident blocks per SM the trace kernels are compiled for: 96 registers for
+// the transparent trace (6 blocks at 80 spill: sparse walks at 4K 25.8 ms against
+// 20.8; 4 blocks 24.6), 72 for the opaque one.
+template <bool OPAQUE, bool COUNT, bool AO>
+constexpr int kMinBlocks = COUNT ? 1 : (OPAQUE ? 6 : (AO ? 4 : 5));
+
+// Main trace. A warp takes one tile of A.tile_n pixels, tile_w wide, at a time,
+// four neighbouring tiles (2x2) in a row to keep what their rays share in L1, and
+// its lanes write their pixels together at the end. Warps take their tiles from
+// a counter: the cost of a tile varies with the lists behind it, and a fixed
+// tile per warp left the slots of a block's finished warps idle until its slowest
+// was done.
+template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
+__global__ void __launch_bounds__(kTraceThreads, kMinBlocks<OPAQUE, COUNT, AO>) k_trace_tile(const __grid_constant__ TraceArgs A) {
+  __shared__ WarpMem<OPAQUE, KEY16> s_mem[kTraceThreads / 32];
+  const int lane = threadIdx.x & 31;
+  WarpMem<OPAQUE, KEY16>& S = s_mem[threadIdx.x >> 5];
+  const int tw = A.tile_w, th = A.tile_n / tw;
+  const uint32_t quads_x = (uint32_t)(A.cam.width + 2 * tw - 1) / (uint32_t)(2 * tw);
+  const uint32_t quads_y = (uint32_t)(A.cam.height + 2 * th - 1) / (uint32_t)(2 * th);
+  Work W;
+  for (bool more = true; more; more = !OPAQUE) {
+    uint32_t tile = blockIdx.x * (kTraceThreads / 32) + (threadIdx.x >> 5);
+    if (!OPAQUE) {
+      if (lane == 0) tile = atomicAdd(A.work_next, 1u);
+      tile = __shfl_sync(FULL, tile, 0);
+    }
+    const uint32_t quad = tile >> 2;
+    if (quad >= quads_x * quads_y) break;
+    const int px = (int)(quad % quads_x) * 2 * tw + (int)(tile & 1u) * tw + (lane & (tw - 1));
+    const int py = (int)(quad / quads_x) * 2 * th + (int)((tile >> 1) & 1u) * th + lane / tw;
+    const bool valid = lane < A.tile_n && px < A.cam.width && py < A.cam.height;
+    Ray R;
+    init_ray(A, S, R, px, py, valid);
+    __syncwarp();
+    trace_warp<OPAQUE, COUNT, KEY16, AO>(A, S, R, W);
+    if (valid) write_pixel(A, S, R);
+    __syncwarp();
+  }
+  count_work<COUNT>(A, W);
+}
+
+// Repair re-trace of the queued pixels: each warp takes its share of the queue
+// (one pixel each when few are queued), at most 32 at a time.
+template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
+__global__ void __launch_bounds__(kTraceThreads, kMinBlocks<OPAQUE, COUNT, AO>) k_trace_list(const __grid_constant__ TraceArgs A) {
+  __shared__ WarpMem<OPAQUE, KEY16> s_mem[kTraceThreads / 32];
+  const int lane = threadIdx.x & 31;
+  WarpMem<OPAQUE, KEY16>& S = s_mem[threadIdx.x >> 5];
+  const uint32_t total = min(*A.pix_count, A.pq_cap);
+  const uint32_t n_warps = gridDim.x * (blockDim.x >> 5);
+  const uint32_t share = min(32u, (total + n_warps - 1) / n_warps);
+  Work W;
+  while (total) {
+    uint32_t base = 0;
+    if (lane == 0) base = atomicAdd(A.work_next, share);
+    base = __shfl_sync(FULL, base, 0);
+    if (base >= total) break;
+    const bool valid = (uint32_t)lane < share && base + lane < total;
+    const uint32_t pix = valid ? A.pix_list[base + lane] : 0u;
+    Ray R;
+    init_ray(A, S, R, (int)(pix % (uint32_t)A.cam.width), (int)(pix / (uint32_t)A.cam.width), valid);
+    if (valid && A.resume) resume_ray(A, S, R);
+    __syncwarp();
+    trace_warp<OPAQUE, COUNT, KEY16, AO>(A, S, R, W);
+    if (valid) write_pixel(A, S, R);
+    __syncwarp();
+  }
+  count_work<COUNT>(A, W);
 }
 
 template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
-void launch_one(const TraceArgs& a, size_t smem, cudaStream_t s) {
-  if constexpr (!OPAQUE) {
-    if (!a.pix_list) {
-      // the instrumented and 16+16-key traces use the default tile
-      const int tw = (COUNT || KEY16) ? 4 : a.tile_w;
-      const int th = 32 / tw;
-      const dim3 grid((a.cam.width + 2 * tw - 1) / (2 * tw), (a.cam.height + 2 * th - 1) / (2 * th));
-      if constexpr (COUNT || KEY16) {
-        k_trace_tile<OPAQUE, COUNT, KEY16, AO, 4><<<grid, kTraceThreads, smem, s>>>(a);
-      } else {
-        if (tw == 2) k_trace_tile<OPAQUE, COUNT, KEY16, AO, 2><<<grid, kTraceThreads, smem, s>>>(a);
-        else if (tw == 8) k_trace_tile<OPAQUE, COUNT, KEY16, AO, 8><<<grid, kTraceThreads, smem, s>>>(a);
-        else if (tw == 16) k_trace_tile<OPAQUE, COUNT, KEY16, AO, 16><<<grid, kTraceThreads, smem, s>>>(a);
-        else k_trace_tile<OPAQUE, COUNT, KEY16, AO, 4><<<grid, kTraceThreads, smem, s>>>(a);
-      }
-      return;
-    }
+void launch_one(const TraceArgs& a, cudaStream_t s) {
+  if (a.pix_list) {
+    k_trace_list<OPAQUE, COUNT, KEY16, AO><<<152 * 4, kTraceThreads, 0, s>>>(a);
+    return;
   }
-  k_trace<OPAQUE, COUNT, KEY16, AO><<<persistent_blocks<OPAQUE, COUNT, KEY16, AO>(smem), kTraceThreads, smem, s>>>(a);
+  const int tw = a.tile_w, th = a.tile_n / tw;
+  // opaque: a block per 2x2 tiles; transparent: as many blocks as the kernel is
+  // compiled to keep resident
+  const unsigned blocks = OPAQUE ? ((a.cam.width + 2 * tw - 1) / (2 * tw)) * ((a.cam.height + 2 * th - 1) / (2 * th))
+                                 : 152 * (COUNT ? 4 : kMinBlocks<OPAQUE, COUNT, AO>);
+  k_trace_tile<OPAQUE, COUNT, KEY16, AO><<<blocks, kTraceThreads, 0, s>>>(a);
 }
 
 template <bool COUNT, bool KEY16>
-void launch_mode(const TraceArgs& a, int K, size_t smem, cudaStream_t s) {
-  if (K == 1) launch_one<true, COUNT, KEY16, false>(a, smem, s);  // AO: k_shade_hits
-  else if (a.ao == 1) launch_one<false, COUNT, KEY16, true>(a, smem, s);
-  else launch_one<false, COUNT, KEY16, false>(a, smem, s);
+void launch_mode(const TraceArgs& a, int K, cudaStream_t s) {
+  if (K == 1) launch_one<true, COUNT, KEY16, false>(a, s);  // AO: k_shade_hits
+  else if (a.ao == 1) launch_one<false, COUNT, KEY16, true>(a, s);
+  else launch_one<false, COUNT, KEY16, false>(a, s);
 }
 
-int launch_trace(const TraceArgs& a, int K, cudaStream_t s) {
-  const size_t smem = K == 1 ? 0 : sizeof(unsigned long long) * kRayKeys * kTraceThreads;
+int launch_trace(const TraceArgs& args, int K, cudaStream_t s) {
+  TraceArgs a = args;
+  a.tile_n = 32;
+  if (K > 1) {
+    // A small image's tiles shrink until there are warps enough to fill the GPU:
+    // a tile is a serial chain of rounds, and its units of work are entries, not
+    // rays, so few rays still fill a warp's lanes (157x93 pixels at alpha 0.1:
+    // 0.75 ms with 32 rays a tile, 0.46 with 16, 0.31 with 8, 0.22 with 4;
+    // where tiles of 32 fill the GPU, 16 cost a third more).
+    const long long npx = (long long)a.cam.width * a.cam.height;
+    while (a.tile_n > 4 && npx / a.tile_n < kResidentWarps) a.tile_n >>= 1;
+    if (a.tile_n < 32) a.tile_w = a.tile_n == 16 ? 4 : 2;
+  }
   if (a.count) {
-    if (a.key16) launch_mode<true, true>(a, K, smem, s);
-    else launch_mode<true, false>(a, K, smem, s);
+    if (a.key16) launch_mode<true, true>(a, K, s);
+    else launch_mode<true, false>(a, K, s);
   } else {
-    if (a.key16) launch_mode<false, true>(a, K, smem, s);
-    else launch_mode<false, false>(a, K, smem, s);
+    if (a.key16) launch_mode<false, true>(a, K, s);
+    else launch_mode<false, false>(a, K, s);
   }
   return 1;
 }
@@ -1090,7 +1194,8 @@ __global__ void __launch_bounds__(kTraceThreads) k_shade_hits(TraceArgs A) {
   if (id >= A.n_vert || id + 1 >= A.n_vert) return;
   float3 o, d;
   pixel_ray(A.cam, px, py, o, d);
-  const float3 c = ao_lane(A, o + v.y * d) * tangent_colour(A, id);
+  const float3 c = ao_lane(A, o + v.y * d) *
+                   tangent_colour(f3(__ldg(&A.pos[id])), f3(__ldg(&A.pos[id + 1])));
   *out = make_float4(A.alpha * c.x, A.alpha * c.y, A.alpha * c.z, v.w);
 }
 

@@ -20,8 +20,8 @@ constexpr float kCoordMax = 768.0f;
 constexpr float kTStop = 1e-4f;                // transmittance where a ray stops
 constexpr int kMaxRepairRounds = 4;
 constexpr uint32_t kRayQueueLimit = 8;          // culled voxels one ray queues per round
-constexpr uint32_t kShortList = 1024;           // trace: longer lists go to the whole-warp path
-constexpr int kRayKeys = 32;                    // trace: hit slots per transparent ray on the shared-entry path
+constexpr uint32_t kShortList = 1024;           // trace: largest limit of the shared-entry path's list length
+constexpr int kRayKeys = 32;                    // trace: largest limit of a ray's hits on that path
 constexpr int kBrickDistMax = 15;               // cap of the empty-brick distance field
 constexpr int kMipsF32 = 0, kMipsF16 = 1, kMipsBF16 = 2;  // occupancy pyramid storage
 
@@ -109,6 +109,7 @@ struct GridDev {
   uint32_t* cur;           // [n^3] list end cursor (start = cur - count); >= kCulledStart: no list
   uint32_t* vis;           // [n^3 / 32] voxel has a list
   const uint8_t* bdist;    // [bricks] Chebyshev distance (bricks) to an occupied brick, capped
+  const uint2* bmask;      // [bricks] bit x + 4 y + 16 z: that voxel of the brick is occupied
   uint32_t* lists;         // [list_cap]
   unsigned long long list_cap;
   uint2* xq;               // [xq_cap] undecided (segment id, packed voxel) pairs
@@ -371,13 +372,30 @@ __device__ __forceinline__ bool lines_may_meet(float3 o, float3 d, float3 a, flo
   return s * s <= rr_margin * nn;
 }
 
+// The hardware's approximate reciprocal square root and division, without the
+// scaling steps that serve denormal operands (about four instructions each).
+// For normal operands the results are those of rsqrtf and __fdividef. Here the
+// operands are squared lengths of at least 2^-28 (coordinates are multiples of
+// 2^-14), discriminants (differences from r^2, so 0 or far above 2^-126) and
+// their quotients by numbers above 1e-30.
+__device__ __forceinline__ float rsqrt_normal(float x) {
+  float y;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+__device__ __forceinline__ float div_normal(float a, float b) {
+  float y;
+  asm("div.approx.ftz.f32 %0, %1, %2;" : "=f"(y) : "f"(a), "f"(b));
+  return y;
+}
+
 // First entry of the line o + t d (|d| = 1) into the ball of radius^2 r2
 // centred at o - oc; +inf when the line misses it.
 __device__ __forceinline__ float ball_entry(float3 oc, float3 d, float r2) {
   const float bq = dot3(oc, d);
   const float3 w = oc - bq * d;
   const float disc = r2 - dot3(w, w);
-  return disc >= 0.0f ? -bq - (disc > 0.0f ? disc * rsqrtf(disc) : 0.0f) : __int_as_float(0x7f800000);
+  return disc >= 0.0f ? -bq - (disc > 0.0f ? disc * rsqrt_normal(disc) : 0.0f) : __int_as_float(0x7f800000);
 }
 
 // First entry of the line o + t d (|d| = 1) into the capsule (a, b, r); +inf
@@ -386,28 +404,29 @@ __device__ __forceinline__ float ball_entry(float3 oc, float3 d, float r2) {
 // cylinder, and where it enters the cylinder decides the rest: between the two
 // end planes that entry is the capsule's; before a (after b) the line can
 // reach the rest of the capsule only through the ball at a (at b), whose entry
-// is then the capsule's. The perpendicular offsets are formed explicitly so
-// that the discriminants do not cancel when the origin is far away.
+// is then the capsule's -- one ball test at the selected end, so that a warp
+// whose lanes need different ends runs it once. The perpendicular offsets are
+// formed explicitly so that the discriminants do not cancel when the origin is
+// far away.
 __device__ __forceinline__ float capsule_entry(float3 o, float3 d, float3 a, float3 b, float r2) {
   const float3 oa = o - a;
   const float3 ba = b - a;
   const float L2 = dot3(ba, ba);
   if (!(L2 > 0.0f)) return ball_entry(oa, d, r2);
-  const float inv = __fdividef(1.0f, L2);
+  const float inv = div_normal(1.0f, L2);
   const float3 dp = d - (dot3(d, ba) * inv) * ba;
   const float3 op = oa - (dot3(oa, ba) * inv) * ba;
   const float A = dot3(dp, dp);
   if (!(A > 1e-30f))  // along the axis: the nearer ball
     return fminf(ball_entry(oa, d, r2), ball_entry(o - b, d, r2));
-  const float ts = __fdividef(-dot3(op, dp), A);
+  const float ts = div_normal(-dot3(op, dp), A);
   const float3 w = op + ts * dp;
   const float disc = r2 - dot3(w, w);
   if (disc < 0.0f) return __int_as_float(0x7f800000);
-  const float q = __fdividef(disc, A);
-  const float t = ts - (q > 0.0f ? q * rsqrtf(q) : 0.0f);
+  const float q = div_normal(disc, A);
+  const float t = ts - (q > 0.0f ? q * rsqrt_normal(q) : 0.0f);
   const float y = dot3(oa + t * d, ba);
-  if (y < 0.0f) return ball_entry(oa, d, r2);
-  if (y > L2) return ball_entry(o - b, d, r2);
+  if (y < 0.0f || y > L2) return ball_entry(y < 0.0f ? oa : o - b, d, r2);
   return t;
 }
 
