@@ -64,7 +64,9 @@ typedef struct {
                              word; 0 selects 32 */
   uint64_t max_fragments; /* list capacity in entries (all voxels), also the
                              capacity of the fragment record and rank
-                             buffers (10 bytes per entry); 0 selects
+                             buffers (10 bytes per entry; sets of fewer
+                             than 44k vertices hold up to 1M entries more
+                             of these); 0 selects
                              0.9 (L + 2 rl + 2)(2 rl + 2)^2, at least 16,
                              entries per uploaded vertex, with L the mean
                              segment length of the vrt_upload_segments call

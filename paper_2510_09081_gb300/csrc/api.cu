@@ -45,8 +45,9 @@ struct vrt_grid_s {
   unsigned long long list_cap = 0;
   uint2* xq = nullptr;      // pairs the fp32 filter left to the exact path
   uint32_t xq_cap = 0;
-  unsigned long long* rec = nullptr;  // fragment records of pass 1 (list_cap entries)
-  uint16_t* rank = nullptr;           // each record's rank within its voxel (list_cap entries)
+  unsigned long long rec_cap = 0;
+  unsigned long long* rec = nullptr;  // fragment records of pass 1 (rec_cap entries)
+  uint16_t* rank = nullptr;           // each record's rank within its voxel (rec_cap entries)
   unsigned long long* tile_state = nullptr;
   uint32_t n_tiles = 0;
   void* mips = nullptr;            // occupancy pyramid (room for fp32 texels)
@@ -166,7 +167,7 @@ GridDev gdev(vrt_grid g) {
   d.word = g->word; d.cur = g->cur; d.vis = g->vis; d.bdist = g->bdist; d.bmask = g->bmask;
   d.lists = g->lists; d.list_cap = g->list_cap;
   d.xq = g->xq; d.xq_cap = g->xq_cap;
-  d.rec = g->rec; d.rank = g->rank; d.rec_cap = (uint32_t)g->list_cap;
+  d.rec = g->rec; d.rank = g->rank; d.rec_cap = (uint32_t)g->rec_cap;
   d.st = g->st;
   return d;
 }
@@ -570,16 +571,22 @@ vrt_status vrt_upload_segments(vrt_grid g, const float* xyz, int32_t stride, int
   unsigned long long cap = g->max_frag_desc ? g->max_frag_desc
                                             : (unsigned long long)(per * (double)std::max(V, 1ll));
   cap = std::min<unsigned long long>(cap, kCulledStart - 1ull);
-  if (cap != g->list_cap || !g->lists) {
+  // Pass 1 takes record slots for candidates, warp by warp; a small set's warps
+  // take fewer segments, so more of the unused slots fall inside the capacity:
+  // room for them.
+  unsigned long long rec_cap = cap;
+  if (pass1_segments_per_warp(V) < 32) rec_cap += std::min<unsigned long long>(4ull * cap, 1ull << 20);
+  if (cap != g->list_cap || rec_cap != g->rec_cap || !g->lists) {
     VRT_CUDA(g, cudaStreamSynchronize(g->stream));
     dfree(g, g->lists);
     dfree(g, g->rec);
     dfree(g, g->rank);
-    g->list_cap = 0;
+    g->list_cap = g->rec_cap = 0;
     VRT_CUDA(g, dalloc(g, &g->lists, (size_t)cap));
-    VRT_CUDA(g, dalloc(g, &g->rec, (size_t)cap));
-    VRT_CUDA(g, dalloc(g, &g->rank, (size_t)cap));
+    VRT_CUDA(g, dalloc(g, &g->rec, (size_t)rec_cap));
+    VRT_CUDA(g, dalloc(g, &g->rank, (size_t)rec_cap));
     g->list_cap = cap;
+    g->rec_cap = rec_cap;
   }
   {
     vrt_status s = size_exact_queue(g);

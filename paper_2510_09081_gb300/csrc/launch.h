@@ -87,6 +87,18 @@ int launch_shade_repair(const ShadeArgs& a, cudaStream_t s);
 // Ingest of vertices [lo, hi) (nothing when hi <= lo).
 int launch_ingest(const float* raw, const uint8_t* flags, long long lo, long long hi, float4* pos,
                   float4* nrm, DevStatus* st, cudaStream_t s);
+constexpr int kPass1Threads = 128;
+constexpr int kPass1Blocks = 9;  // resident per SM: 56 registers, 24 KB of shared memory
+// Segments a warp of pass 1 takes, of a set of V vertices. They are a serial chain
+// of steps over their candidates, and a step takes 32 candidates whatever their
+// segments, so a small set is spread over more warps: 4.5k segments of 57
+// fragments each 0.105 ms with 32 segments a warp, 0.056 with 8, 0.046 with 4; 20k
+// of 7 0.050, 0.046, 0.048; at 98k it no longer pays (0.044 with 32, 0.047 with 16).
+inline int pass1_segments_per_warp(long long V) {
+  int n = 32;
+  while (n > 4 && V / n < 152ll * kPass1Blocks) n >>= 1;
+  return n;
+}
 // Pass 1 over the segments in the order `order` (V vertex indices, each
 // polyline's vertices consecutive; a polyline's last vertex starts no
 // segment), or in index order when `order` is null.

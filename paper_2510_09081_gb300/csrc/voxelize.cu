@@ -12,10 +12,11 @@
 // |d_ai / d_a0| + 2 * half-extent), so candidate q of a segment decodes in O(1).
 //
 // Work layout: each lane loads one segment (coalesced), sets up its walk and
-// stores it, packed, in shared memory; the warp numbers the candidates of its
-// 32 segments consecutively and takes them 32 at a time, each lane reading the
-// walk of the segment its candidate belongs to, so segments of different
-// lengths do not leave lanes idle. The fp32 filter decides almost every candidate; pairs it
+// stores it in shared memory; the warp numbers the candidates of its 32 segments
+// consecutively and takes them 32 at a time, each lane reading the record of the
+// segment its candidate belongs to, so segments of different lengths do not
+// leave lanes idle, and neighbouring lanes have neighbouring voxels (their atomics
+// share sectors). The fp32 filter decides almost every candidate; pairs it
 // cannot decide go to a queue that a separate kernel decides exactly (keeping
 // the 128-bit integer path out of the hot kernels' registers).
 //
@@ -33,23 +34,33 @@
 
 namespace vrt {
 
+constexpr int kPass1Warps = kPass1Threads / 32;
 constexpr float kWalkEps = 1e-3f;
 constexpr unsigned FULLW = 0xffffffffu;
 
-struct Walk {
-  float3 a, b;
-  float am, a1, a2, s1, s2, rho1, rho2, lo_m, hi_m;
-  float inv_w12, inv_w2;  // reciprocals of W1 * W2 and W2 for the uniform decode
-  int m, c0, W1, W2;
-  bool exact;             // candidates are exactly the slab boxes' voxels
-  bool boxed;             // exact, with at most kBoxedSlabs slabs: boxes kept
-  uint32_t pre[4];        // exact: 16-bit cumulative counts after slabs 0..7
-  uint32_t box[6];        // boxed: slab k's box, j0 | l0 << 10 | (l1 - l0 + 1) << 20
-  uint32_t n;             // candidates
-};
+constexpr int kBoxSlabs = 9;        // slabs whose boxes a segment's record holds
+constexpr int kTableSlabs = 8;      // slabs an owner table's byte can name
+constexpr uint32_t kWindow = 512;  // candidates of a warp whose owners are tabulated at a time
 
-constexpr int kExactSlabs = 9;  // slabs whose boxes the exact decode indexes
-constexpr int kBoxedSlabs = 6;  // slabs whose boxes the packed walk can hold
+// One segment in shared memory. Short segments (up to kBoxSlabs slabs; nearly all)
+// keep the box of each slab: x = j0 | l0 << 10 | w2 << 20 (first voxel on the two
+// minor axes, width on the second), y = candidates of the segment before the slab
+// | ceil(4096 / w2) << 16. Longer ones keep what slab_box needs, and index every
+// slab's box with the widest slab's widths.
+struct Seg {
+  float4 a;   // v0; reciprocal of |d|^2 (0 for a point)
+  float4 d;   // v1 - v0; largest squared distance stage 1 accepts
+  float4 n0;  // clip normal at v0; m | c0 << 2 | clip flags << 12 | boxed << 14
+  float4 n1;  // clip normal at v1; the segment's first candidate number
+  union {
+    uint2 box[kBoxSlabs];
+    struct {
+      float s1, s2, rho1, rho2, lo_m, hi_m, inv_w12, inv_w2;
+      int w1, w2;
+    } g;
+  };
+};
+static_assert(sizeof(Seg) == 144, "records next to each other start four banks apart");
 
 // Minor-axis voxel ranges of slab c (clamped to the grid): the axis line
 // a_k + (x - a_m) s_k over the slab's part of [lo_m, hi_m], widened by rho_k.
@@ -65,155 +76,101 @@ __device__ __forceinline__ void slab_box(float am, float a1, float a2, float s1,
   l1 = min(n - 1, (int)floorf(fmaxf(p2a, p2b) + rho2));
 }
 
-__device__ __forceinline__ void walk_setup(float3 a, float3 b, const GridDev& g, Walk& w) {
+// Set up the walk of segment a, b into its record (all but n0.w's flags' clip part
+// and n1, which the caller fills): the numbers its candidates take, and in `voxels`
+// how many of them are voxels. Approximate division and square roots serve:
+// kWalkEps widens every box by far more than their error.
+__device__ __forceinline__ uint32_t walk_setup(float3 a, float3 b, const GridDev& g, Seg& S,
+                                               uint32_t& bits, bool& short_walk,
+                                               uint32_t& voxels) {
   const float rl = g.rl;
   const int n = g.n;
   const float3 d = b - a;
   const float ax = fabsf(d.x), ay = fabsf(d.y), az = fabsf(d.z);
   const int m = (ax >= ay && ax >= az) ? 0 : (ay >= az ? 1 : 2);
   const int k1 = m == 0 ? 1 : 0, k2 = m == 2 ? 1 : 2;
-  w.a = a;
-  w.b = b;
-  w.m = m;
-  w.am = cmp3(a, m);
-  const float dm = cmp3(b, m) - w.am;
-  w.s1 = dm != 0.0f ? cmp3(d, k1) / dm : 0.0f;
-  w.s2 = dm != 0.0f ? cmp3(d, k2) / dm : 0.0f;
-  w.rho1 = rl * sqrtf(fmaf(w.s1, w.s1, 1.0f)) + kWalkEps;
-  w.rho2 = rl * sqrtf(fmaf(w.s2, w.s2, 1.0f)) + kWalkEps;
-  w.lo_m = fminf(w.am, w.am + dm) - rl;
-  w.hi_m = fmaxf(w.am, w.am + dm) + rl;
-  w.a1 = cmp3(a, k1);
-  w.a2 = cmp3(a, k2);
-  w.c0 = max(0, (int)floorf(w.lo_m - kWalkEps));
-  const int c1 = min(n - 1, (int)floorf(w.hi_m + kWalkEps));
-  // Up to kExactSlabs slabs: candidates are the voxels of each slab's own box,
-  // numbered slab after slab (cumulative counts kept); longer segments index
-  // every slab's box with the widest slab's widths.
-  int W1 = 1, W2 = 1;
-  uint32_t total = 0;
-  w.pre[0] = w.pre[1] = w.pre[2] = w.pre[3] = 0xffffffffu;
-#pragma unroll
-  for (int k = 0; k < kExactSlabs; ++k) {  // unrolled: pre[] stays in registers
-    const int c = w.c0 + k;
-    if (c > c1) break;
-    int j0, j1, l0, l1;
-    slab_box(w.am, w.a1, w.a2, w.s1, w.s2, w.rho1, w.rho2, w.lo_m, w.hi_m, n, c, j0, j1, l0, l1);
-    W1 = max(W1, j1 - j0 + 1);
-    W2 = max(W2, l1 - l0 + 1);
-    total += (uint32_t)(max(0, j1 - j0 + 1) * max(0, l1 - l0 + 1));
-    if (k < kBoxedSlabs)
-      w.box[k] = ((uint32_t)j0 & 1023u) | (((uint32_t)l0 & 1023u) << 10) |
-                 ((uint32_t)max(1, l1 - l0 + 1) << 20);
-    if (k < 8) {  // cumulative count after slab k
-      const uint32_t v = min(total, 0xffffu);
-      w.pre[k >> 1] = (w.pre[k >> 1] & ~(0xffffu << (16 * (k & 1)))) | (v << (16 * (k & 1)));
+  const float am = cmp3(a, m), dm = cmp3(d, m);
+  const float inv = dm != 0.0f ? div_normal(1.0f, dm) : 0.0f;  // |dm| >= 2^-14
+  const float s1 = cmp3(d, k1) * inv, s2 = cmp3(d, k2) * inv;
+  const float q1 = fmaf(s1, s1, 1.0f), q2 = fmaf(s2, s2, 1.0f);
+  const float rho1 = fmaf(rl * q1, rsqrt_normal(q1), kWalkEps);
+  const float rho2 = fmaf(rl * q2, rsqrt_normal(q2), kWalkEps);
+  const float lo_m = fminf(am, am + dm) - rl, hi_m = fmaxf(am, am + dm) + rl;
+  const float a1 = cmp3(a, k1), a2 = cmp3(a, k2);
+  const int c0 = max(0, (int)floorf(lo_m - kWalkEps));
+  const int c1 = min(n - 1, (int)floorf(hi_m + kWalkEps));
+  const int slabs = c1 - c0 + 1;
+  const float dd = dot3(d, d);
+  // Stage 1's rounding allowance: six times seg_box_tol's, at the largest local
+  // coordinate a candidate of this segment can have, which covers the rounding
+  // of the nearest point's parameter too (its distance along the axis from the
+  // true nearest point, which would otherwise enter the lower bound).
+  const float M = fmaxf(ax, fmaxf(ay, az)) + 1.5f * rl + 4.0f;
+  S.a = make_float4(a.x, a.y, a.z, dd > 0.0f ? div_normal(1.0f, dd) : 0.0f);
+  S.d = make_float4(d.x, d.y, d.z, fmaf(rl, rl, -2.9e-6f * M * M));
+  const bool boxed = slabs <= kBoxSlabs;
+  short_walk = slabs <= kTableSlabs;
+  bits = (uint32_t)m | ((uint32_t)c0 << 2) | (boxed ? 1u << 14 : 0u);
+  voxels = 0;
+  if (slabs <= 0) return 0;
+  if (boxed) {
+    uint32_t total = 0;
+    for (int k = 0; k < slabs; ++k) {
+      int j0, j1, l0, l1;
+      slab_box(am, a1, a2, s1, s2, rho1, rho2, lo_m, hi_m, n, c0 + k, j0, j1, l0, l1);
+      // widths stay below 16: |s| <= 1 and the radius is at most 4
+      const uint32_t w1 = (uint32_t)max(0, j1 - j0 + 1), w2 = (uint32_t)max(0, l1 - l0 + 1);
+      const uint32_t wd = max(1u, w2);
+      S.box[k] = make_uint2(((uint32_t)j0 & 1023u) | (((uint32_t)l0 & 1023u) << 10) | (wd << 20),
+                            total | ((4095u + wd) / wd) << 16);
+      total += w1 * w2;
     }
+    for (int k = slabs; k < kBoxSlabs; ++k) S.box[k].y = 0xffffu;  // past every candidate
+    voxels = total;
+    return total;
   }
-  for (int c = w.c0 + kExactSlabs; c <= c1; ++c) {  // longer segments: widths only
+  int W1 = 1, W2 = 1;
+  for (int c = c0; c <= c1; ++c) {
     int j0, j1, l0, l1;
-    slab_box(w.am, w.a1, w.a2, w.s1, w.s2, w.rho1, w.rho2, w.lo_m, w.hi_m, n, c, j0, j1, l0, l1);
+    slab_box(am, a1, a2, s1, s2, rho1, rho2, lo_m, hi_m, n, c, j0, j1, l0, l1);
     W1 = max(W1, j1 - j0 + 1);
     W2 = max(W2, l1 - l0 + 1);
+    voxels += (uint32_t)(max(0, j1 - j0 + 1) * max(0, l1 - l0 + 1));
   }
-  const int slabs = c1 - w.c0 + 1;
-  w.W1 = W1;
-  w.W2 = W2;
-  w.exact = slabs > 0 && slabs <= kExactSlabs && total < 0xffffu;
-  w.boxed = w.exact && slabs <= kBoxedSlabs;
-  w.n = slabs <= 0 ? 0u : (w.exact ? total : (uint32_t)slabs * (uint32_t)(W1 * W2));
-  w.inv_w12 = 1.0f / (float)(W1 * W2);
-  w.inv_w2 = 1.0f / (float)W2;
+  S.g.s1 = s1; S.g.s2 = s2; S.g.rho1 = rho1; S.g.rho2 = rho2;
+  S.g.lo_m = lo_m; S.g.hi_m = hi_m;
+  S.g.inv_w12 = 1.0f / (float)(W1 * W2);
+  S.g.inv_w2 = 1.0f / (float)W2;
+  S.g.w1 = W1; S.g.w2 = W2;
+  return (uint32_t)slabs * (uint32_t)(W1 * W2);
 }
 
-// A walk as five float4s in shared memory (plus the clip normals in two more):
-//   w0 = (a, s1), w1 = (b, s2), w2 = (rho1, rho2, lo_m, hi_m),
-//   w3 = (1 / (W1 W2), 1 / W2, bits, first candidate number of the warp),
-//   w4 = cumulative counts after slabs 0..7, 16 bits each (exact decode),
-//   bits = m | c0 << 2 | W1 << 11 | W2 << 19 | clip flags << 27 | exact << 29
-//          | boxed << 30.
-// A boxed walk keeps its slab boxes, as walk_setup found them, where the
-// uniform decode's fields would be: slabs 0-3 in w2, slabs 4-5 in w3.x, w3.y.
-// W1, W2 <= 2 + |s_k| + 2 rho_k < 16 since radius <= 4, and c0 < 512.
-struct PackedWalk {
-  float4 w0, w1, w2, w3;
-  uint4 w4;
-};
-
-__device__ __forceinline__ PackedWalk pack_walk(const Walk& w, uint32_t clip, uint32_t first) {
-  PackedWalk p;
-  p.w0 = make_float4(w.a.x, w.a.y, w.a.z, w.s1);
-  p.w1 = make_float4(w.b.x, w.b.y, w.b.z, w.s2);
-  const uint32_t bits = (uint32_t)w.m | ((uint32_t)w.c0 << 2) | ((uint32_t)w.W1 << 11) |
-                        ((uint32_t)w.W2 << 19) | (clip << 27) | ((uint32_t)w.exact << 29) |
-                        ((uint32_t)w.boxed << 30);
-  if (w.boxed) {
-    p.w2 = make_float4(__uint_as_float(w.box[0]), __uint_as_float(w.box[1]),
-                       __uint_as_float(w.box[2]), __uint_as_float(w.box[3]));
-    p.w3 = make_float4(__uint_as_float(w.box[4]), __uint_as_float(w.box[5]), __uint_as_float(bits),
-                       __uint_as_float(first));
-  } else {
-    p.w2 = make_float4(w.rho1, w.rho2, w.lo_m, w.hi_m);
-    p.w3 = make_float4(w.inv_w12, w.inv_w2, __uint_as_float(bits), __uint_as_float(first));
-  }
-  p.w4 = make_uint4(w.pre[0], w.pre[1], w.pre[2], w.pre[3]);
-  return p;
-}
-
-// Candidate q of a packed walk: its voxel, or false when q falls outside its
-// slab's box (uniform decode only).
-__device__ __forceinline__ bool decode_candidate(const PackedWalk& p, int n, uint32_t q, int& x,
-                                                 int& y, int& z) {
-  const uint32_t bits = __float_as_uint(p.w3.z);
-  const int m = bits & 3, c0 = (bits >> 2) & 511, W1 = (bits >> 11) & 255, W2 = (bits >> 19) & 255;
-  const float am = m == 0 ? p.w0.x : (m == 1 ? p.w0.y : p.w0.z);
-  const float a1 = m == 0 ? p.w0.y : p.w0.x;
-  const float a2 = m == 2 ? p.w0.y : p.w0.z;
-  // (q + 1/2) / w is at least 1/(2w) from an integer, far beyond fp32 error for
-  // these small counts, so truncation gives the exact quotient
-  int slab, rem;
-  if (bits & (1u << 29)) {  // exact: the slab whose cumulative range holds q
-    // the number of cumulative counts <= q (non-decreasing, 16 bits each, two
-    // per word; q < 65535), by packed half-word comparisons
-    const uint32_t qq = q * 0x00010001u;
-    slab = (__popc(__vcmpleu2(p.w4.x, qq)) + __popc(__vcmpleu2(p.w4.y, qq)) +
-            __popc(__vcmpleu2(p.w4.z, qq)) + __popc(__vcmpleu2(p.w4.w, qq))) >> 4;
-    const int s1 = slab - 1;
-    const uint32_t word = s1 < 2 ? p.w4.x : (s1 < 4 ? p.w4.y : (s1 < 6 ? p.w4.z : p.w4.w));
-    const uint32_t base = slab ? (word >> (16 * (s1 & 1))) & 0xffffu : 0u;
-    rem = (int)(q - base);
-  } else {
-    slab = (int)(((float)q + 0.5f) * p.w3.x);
-    rem = (int)q - slab * (W1 * W2);
-  }
-  const int c = c0 + slab;
-  if (bits & (1u << 30)) {  // boxed: the slab's box as walk_setup found it; q lies inside it
-    const uint32_t bx = __float_as_uint(
-        slab < 2 ? (slab == 0 ? p.w2.x : p.w2.y)
-                 : (slab < 4 ? (slab == 2 ? p.w2.z : p.w2.w) : (slab == 4 ? p.w3.x : p.w3.y)));
-    const int w2 = (int)(bx >> 20);
-    // an approximate reciprocal suffices: (rem + 1/2) / w2 lies at least 1/(2 w2)
-    // from an integer and rem < 256
-    const int dj = (int)(((float)rem + 0.5f) * __fdividef(1.0f, (float)w2));
-    const int j = (int)(bx & 1023u) + dj, l = (int)((bx >> 10) & 1023u) + rem - dj * w2;
-    x = m == 0 ? c : j;
-    y = m == 1 ? c : (m == 0 ? j : l);
-    z = m == 2 ? c : l;
-    return true;
-  }
-  int j0, j1, l0, l1;
-  slab_box(am, a1, a2, p.w0.w, p.w1.w, p.w2.x, p.w2.y, p.w2.z, p.w2.w, n, c, j0, j1, l0, l1);
-  const int w2 = (bits & (1u << 29)) ? l1 - l0 + 1 : W2;
-  // an approximate reciprocal suffices: (rem + 1/2) / w2 lies at least 1/(2 w2)
-  // from an integer and rem < 256
-  const float inv_w2 = (bits & (1u << 29)) ? __fdividef(1.0f, (float)w2) : p.w3.y;
-  const int dj = (int)(((float)rem + 0.5f) * inv_w2);
-  const int dl = rem - dj * w2;
-  const int j = j0 + dj, l = l0 + dl;
-  if (j > j1 || l > l1) return false;
+// Minor-axis voxels j, l of slab c to x, y, z.
+__device__ __forceinline__ void place(uint32_t m, int c, int j, int l, int& x, int& y, int& z) {
   x = m == 0 ? c : j;
   y = m == 1 ? c : (m == 0 ? j : l);
   z = m == 2 ? c : l;
+}
+
+// Candidate q of a segment that is not boxed: its voxel, or false when q falls
+// outside its slab's box.
+__device__ __forceinline__ bool decode_long(const Seg& S, uint32_t bits, int n, uint32_t q, int& x,
+                                            int& y, int& z) {
+  const uint32_t m = bits & 3u;
+  const float am = m == 0 ? S.a.x : (m == 1 ? S.a.y : S.a.z);
+  const float a1 = m == 0 ? S.a.y : S.a.x;
+  const float a2 = m == 2 ? S.a.y : S.a.z;
+  // (q + 1/2) / w is at least 1/(2w) from an integer, far beyond fp32 error for
+  // these small counts, so truncation gives the exact quotient
+  const int slab = (int)(((float)q + 0.5f) * S.g.inv_w12);
+  const int rem = (int)q - slab * (S.g.w1 * S.g.w2);
+  const int c = (int)((bits >> 2) & 1023u) + slab;
+  int j0, j1, l0, l1;
+  slab_box(am, a1, a2, S.g.s1, S.g.s2, S.g.rho1, S.g.rho2, S.g.lo_m, S.g.hi_m, n, c, j0, j1, l0, l1);
+  const int dj = (int)(((float)rem + 0.5f) * S.g.inv_w2);
+  const int j = j0 + dj, l = l0 + rem - dj * S.g.w2;
+  if (j > j1 || l > l1) return false;
+  place(m, c, j, l, x, y, z);
   return true;
 }
 
@@ -273,6 +230,23 @@ __device__ __forceinline__ void flush_counters(DevStatus* st, unsigned long long
   }
 }
 
+// Candidate number at which slab q of a boxed segment ends: the next slab's start
+// (slabs past the last start beyond the segment's end).
+__device__ __forceinline__ uint32_t slab_end(const Seg& S, int q, uint32_t first, uint32_t end) {
+  return q + 1 < kBoxSlabs ? min(end, first + (S.box[q + 1].y & 0xffffu)) : end;
+}
+
+// Occupancy code (Alg. 3 around Alg. 2, quantized) of a voxel whose centre lies at
+// pa from v0, pb from v1 and at squared distance q2 from the axis.
+__device__ __forceinline__ uint32_t occupancy_code(const GridDev& g, float3 pa, float3 pb, float q2,
+                                                   float3 n0, float3 n1, bool en0, bool en1) {
+  float s = (q2 > 0.0f ? q2 * rsqrt_normal(q2) : 0.0f) - g.r_clamp;
+  if (en0) s = fmaxf(s, -dot3(pa, n0));
+  if (en1) s = fmaxf(s, dot3(pb, n1));
+  const float occ = fminf(1.0f, fmaxf(0.0f, 0.5f - s)) * g.corr;
+  return (uint32_t)floorf(fmaf(g.occ_scale, occ, 0.5f));
+}
+
 // The packed-word increment (occupancy code << 16) | 1 of one fragment (Alg. 3
 // at the voxel centre, quantized); counts it in F and sq.
 __device__ __forceinline__ uint32_t fragment_word(const GridDev& g, float3 a, float3 b, float3 n0,
@@ -330,168 +304,255 @@ __device__ __forceinline__ void flush_culled(const GridDev& g, unsigned long lon
   __syncwarp();
 }
 
-__global__ void __launch_bounds__(256) k_pass1(const float4* __restrict__ pos,
-                                               const float4* __restrict__ nrm,
-                                               const uint32_t* __restrict__ order, long long V,
-                                               GridDev g) {
-  const int lane = threadIdx.x & 31;
-  const long long base = ((long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5)) * 32;
+// Bound by instruction issue (82% of the issue slots before and after), so a
+// candidate's work is cut to what it needs: the owner and slab of a candidate come
+// from a byte table the warp's lanes fill (one load instead of a search over the
+// lanes and comparisons over the slabs), the slab's box and the segment's
+// reciprocal length from its record, and the filter's point on the axis, its
+// offset from the voxel centre and their distance serve the occupancy too (Alg. 2
+// measures the same point). Records of 128 bytes put all lanes' loads on the
+// same banks (72% of the shared-memory pipe); 144 bytes do not. Bundles (114M
+// fragments, 256^3) 2.40 -> 1.74 ms, ABC flow (195M, 512^3) 4.71 -> 3.71 ms; without
+// the atomics 10% less, so they are not what bounds it.
+__global__ void __launch_bounds__(kPass1Threads, kPass1Blocks) k_pass1(const float4* __restrict__ pos,
+                                                  const float4* __restrict__ nrm,
+                                                  const uint32_t* __restrict__ order, long long V,
+                                                  int segs_per_warp, GridDev g) {
+  __shared__ Seg s_seg[kPass1Threads];
+  __shared__ uint32_t s_id[kPass1Threads];          // segment id of each lane's record
+  __shared__ uint8_t s_own[kPass1Warps][kWindow];   // candidate -> lane | slab << 5 (boxed segments)
+  // Candidates the first filter stage leaves undecided (a few percent) wait in
+  // a per-warp queue and get the Newton stage 32 at a time, so the warp does
+  // not run it for one or two lanes per step.
+  __shared__ uint2 s_uq[kPass1Warps][64];           // (owner lane, packed voxel)
+  __shared__ uint32_t s_wtot[kPass1Warps];
+  __shared__ unsigned long long s_rbase;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, tid = threadIdx.x;
+  const long long base = ((long long)blockIdx.x * kPass1Warps + wid) * segs_per_warp;
   // slots in spatial order (nearby segments in the same and neighbouring
   // warps keep the packed-word atomics within a smaller part of the grid)
   const long long k = base + lane;
-  const long long i = k < V ? (order ? (long long)__ldg(&order[k]) : k) : V;
-  Walk w;
-  w.n = 0;
-  float3 n0 = make_float3(0.f, 0.f, 0.f), n1 = n0;
-  uint32_t en = 0;
+  const long long i = lane < segs_per_warp && k < V ? (order ? (long long)__ldg(&order[k]) : k) : V;
+  uint32_t count = 0, bits = 0, voxels = 0;
+  bool short_walk = true;
   if (i + 1 < V) {
     const float4 p0 = pos[i];
     const uint32_t f0 = __float_as_uint(p0.w);
     if (!(f0 & kLast)) {
       const float4 p1 = pos[i + 1];
-      walk_setup(f3(p0), f3(p1), g, w);
-      n0 = f3(nrm[i]);
-      n1 = f3(nrm[i + 1]);
-      en = ((f0 & kClipOn) ? 1u : 0u) | ((__float_as_uint(p1.w) & kClipOn) ? 2u : 0u);
+      const float4 m0 = nrm[i], m1 = nrm[i + 1];
+      Seg& S = s_seg[tid];
+      count = walk_setup(f3(p0), f3(p1), g, S, bits, short_walk, voxels);
+      bits |= ((f0 & kClipOn) ? 1u << 12 : 0u) | ((__float_as_uint(p1.w) & kClipOn) ? 1u << 13 : 0u);
+      S.n0 = make_float4(m0.x, m0.y, m0.z, __uint_as_float(bits));
+      S.n1 = make_float4(m1.x, m1.y, m1.z, 0.0f);
+      s_id[tid] = (uint32_t)i;
     }
   }
-  unsigned long long F = 0, sq = 0, ex = 0;
-  const unsigned lt = (1u << lane) - 1u;
-  // every lane's walk, packed, read by the lanes that take its candidates
-  __shared__ PackedWalk s_w[256];
-  __shared__ float4 s_n[2][256];  // clip normals at v0 and v1
-  __shared__ uint32_t s_seg[256];  // segment id of each lane's walk
-  const int tid = threadIdx.x, wb = tid & ~31;
-  uint32_t wcount = 0;  // records this warp has written (uniform)
-  // segment id of lane j's walk
-  auto seg_of = [&](int j) { return order ? s_seg[wb + j] : (uint32_t)(base + j); };
-  // The warp's candidates, segment after segment, are numbered 0..total-1;
-  // lane l takes number t0 + l and finds its segment by a binary search over
-  // the inclusive prefix of the candidate counts.
-  uint32_t incl = w.n;
+  // The warp's candidates, segment after segment, are numbered 0..total-1.
+  uint32_t incl = count;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
     const uint32_t v = __shfl_up_sync(FULLW, incl, o);
     if (lane >= o) incl += v;
   }
   const uint32_t total = __shfl_sync(FULLW, incl, 31);
+  const uint32_t first = incl - count;
+  const uint32_t slots = __reduce_add_sync(FULLW, voxels);  // record slots the warp needs at most
+  if (count) s_seg[tid].n1.w = __uint_as_float(first);
   // record slots: one atomic per block for all its candidates, warp shares in
-  // warp order (a fragment per warp step took 2-3 flushes of staged records
-  // per warp on one global counter, which contended)
-  __shared__ uint32_t s_wtot[8];
-  __shared__ unsigned long long s_rbase;
-  const int wid = threadIdx.x >> 5;
-  if (lane == 0) s_wtot[wid] = total;
+  // warp order (one atomic per warp on the single counter kept pass 1 waiting
+  // on sets of many short segments: ABC at 1/8 of its lines 0.56 -> 0.75 ms);
+  // the first window's table is filled while it is under way
+  if (lane == 0) s_wtot[wid] = slots;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     uint32_t sum = 0;
-    for (int k = 0; k < (int)(blockDim.x >> 5); ++k) {
-      const uint32_t t = s_wtot[k];
-      s_wtot[k] = sum;
+    for (int q = 0; q < kPass1Warps; ++q) {
+      const uint32_t t = s_wtot[q];
+      s_wtot[q] = sum;
       sum += t;
     }
     s_rbase = sum ? atomicAdd(&g.st->rec_cnt, (unsigned long long)sum) : 0ull;
   }
+  const bool tabled = __all_sync(FULLW, short_walk || !count);
+  // owner and slab of the candidates of window [w0, w1)
+  auto fill = [&](uint32_t w0, uint32_t w1) {
+    if (!tabled || !count) return;
+    uint32_t s0 = first;
+    for (int q = 0; q < kTableSlabs && s0 < incl; ++q) {
+      const uint32_t s1 = slab_end(s_seg[tid], q, first, incl);
+      for (uint32_t c = max(s0, w0); c < min(s1, w1); ++c) s_own[wid][c - w0] = (uint8_t)(lane | q << 5);
+      s0 = s1;
+    }
+  };
+  fill(0u, min(total, kWindow));
   __syncthreads();
+  // Past the capacity, `room` slots of the warp's share exist.
   const unsigned long long rbase = s_rbase + s_wtot[wid];
-  if (w.n) {
-    if (order) s_seg[tid] = (uint32_t)i;
-    s_w[tid] = pack_walk(w, en, incl - w.n);
-    s_n[0][tid] = make_float4(n0.x, n0.y, n0.z, 0.0f);
-    s_n[1][tid] = make_float4(n1.x, n1.y, n1.z, 0.0f);
-  }
-  __syncwarp();
-  // Candidates the first filter stage leaves undecided (a few percent) wait in
-  // a per-warp queue and get the Newton stage 32 at a time, so the warp does
-  // not run it for one or two lanes per step.
-  __shared__ uint2 s_uq[8][64];  // (owner lane, packed voxel)
-  uint2* uq = s_uq[threadIdx.x >> 5];
-  uint32_t un = 0;  // queued (uniform)
+  const uint32_t room = rbase < g.rec_cap ? (uint32_t)min((unsigned long long)slots, g.rec_cap - rbase) : 0u;
+  unsigned long long* rec = g.rec + min(rbase, (unsigned long long)g.rec_cap);
+  uint16_t* rank = g.rank + min(rbase, (unsigned long long)g.rec_cap);
+  const Seg* segs = s_seg + (tid & ~31);
+  const uint32_t* ids = s_id + (tid & ~31);
+  unsigned long long sq = 0;
+  uint32_t sq32 = 0, ex = 0;  // a window's codes: at most 32 steps (and stage 2's) of 16 bits
+  const unsigned lt = (1u << lane) - 1u;
+  uint2* uq = s_uq[wid];
+  uint32_t un = 0;      // queued (uniform)
+  uint32_t wcount = 0;  // records this warp has written (uniform)
   // A fragment's rank is stored one emit later, so the latency of the
   // returning atomic that gives it overlaps a step of work: pend_r is the
   // record slot still waiting for its rank, the count field of the word
   // pend_old that the lane's atomic returned.
-  unsigned long long pend_r = ~0ull;
-  uint32_t pend_old = 0;
+  uint32_t pend_r = ~0u, pend_old = 0;
   auto flush_rank = [&]() {  // all lanes call
-    if (pend_r < g.rec_cap) g.rank[pend_r] = (uint16_t)pend_old;  // low 16 bits: count
-    pend_r = ~0ull;
+    if (pend_r != ~0u) rank[pend_r] = (uint16_t)pend_old;  // low 16 bits: count
+    pend_r = ~0u;
   };
-  // a kept fragment: occupancy into the packed word, record written (all lanes call)
-  auto emit = [&](bool keep, int j, const PackedWalk& p, int x, int y, int z) {
-    uint32_t idx = 0;
+  // a kept fragment: occupancy into the packed word, record written (all lanes
+  // call). w: the voxel's centre seen from v0, e2: its squared distance to the axis.
+  auto emit = [&](bool keep, int j, const float4& n0, float3 w, float e2, int x, int y, int z) {
     flush_rank();
     const unsigned am = __ballot_sync(FULLW, keep);
     if (keep) {
-      idx = brick_index(x, y, z, g.log2nb);
-      const uint32_t clip = __float_as_uint(p.w3.z) >> 27;
-      const uint32_t inc = fragment_word(g, f3(p.w0), f3(p.w1), f3(s_n[0][wb + j]),
-                                         f3(s_n[1][wb + j]), clip & 1u, clip & 2u, x, y, z, F, sq);
-      pend_old = atomicAdd(&g.word[idx], inc);
-    }
-    if (keep) {
-      const unsigned long long r = rbase + wcount + __popc(am & lt);
-      if (r < g.rec_cap) {
-        g.rec[r] = ((unsigned long long)idx << 32) | seg_of(j);
+      const Seg& S = segs[j];
+      const float3 pb = w - f3(S.d);
+      const uint32_t clip = __float_as_uint(n0.w) >> 12;
+      const uint32_t q = occupancy_code(g, w, pb, e2, f3(n0), f3(S.n1), clip & 1u, clip & 2u);
+      sq32 += q;
+      const uint32_t idx = brick_index(x, y, z, g.log2nb);
+      pend_old = atomicAdd(&g.word[idx], (q << 16) | 1u);
+      const uint32_t r = wcount + __popc(am & lt);
+      if (r < room) {
+        rec[r] = ((unsigned long long)idx << 32) | ids[j];
         pend_r = r;
-      } else {
-        set_err(g.st, kErrOverflow);
       }
     }
     wcount += __popc(am);
   };
+  // the voxel's centre seen from v0, and its squared distance to the axis at the
+  // nearest point t of the segment
+  auto offset = [&](const Seg& S, int x, int y, int z, float3& w, float& t, float3& e) {
+    w = make_float3((float)x + 0.5f - S.a.x, (float)y + 0.5f - S.a.y, (float)z + 0.5f - S.a.z);
+    t = fminf(1.0f, fmaxf(0.0f, dot3(w, f3(S.d)) * S.a.w));
+    e = w - t * f3(S.d);
+    return dot3(e, e);
+  };
   // stage 2 for queued entries below cnt (all lanes call)
   auto stage2 = [&](uint32_t cnt) {
     int dec = 0, j = 0, x = 0, y = 0, z = 0;
-    PackedWalk p;
+    float3 w = make_float3(0.f, 0.f, 0.f), e;
+    float t, e2 = 0.0f;
+    float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f);
     if ((uint32_t)lane < cnt) {
       const uint2 it = uq[lane];
       j = (int)it.x;
       unpack_voxel(it.y, x, y, z);
-      p = s_w[wb + j];
-      dec = g.force_exact ? -1 : seg_stage2_at(f3(p.w0), f3(p.w1), x, y, z, g.rl);
+      const Seg& S = segs[j];
+      n0 = S.n0;
+      e2 = offset(S, x, y, z, w, t, e);
+      const float3 la = make_float3(S.a.x - (float)x, S.a.y - (float)y, S.a.z - (float)z);
+      dec = g.force_exact ? -1 : seg_box_stage2(la, f3(S.d), g.rl);
       if (dec < 0) ++ex;
     }
-    queue_exact(g, dec < 0, (uint32_t)lane < cnt ? seg_of(j) : 0u, x, y, z, lane);
-    emit(dec > 0, j, p, x, y, z);
+    queue_exact(g, dec < 0, ids[j], x, y, z, lane);
+    emit(dec > 0, j, n0, w, e2, x, y, z);
   };
-  for (uint32_t t0 = 0; t0 < total; t0 += 32) {
-    const uint32_t gq = t0 + lane;
-    int j = 0;
+  const float rl2x2 = 2.0f * g.rl * g.rl;
+  for (uint32_t w0 = 0; w0 < total; w0 += kWindow) {
+    const uint32_t w1 = min(total, w0 + kWindow);
+    if (w0) {
+      __syncwarp();
+      fill(w0, w1);
+      __syncwarp();
+    }
+    for (uint32_t t0 = w0; t0 < w1; t0 += 32) {
+      const uint32_t gq = t0 + lane;
+      int j = 0, x = 0, y = 0, z = 0, dec = 0;
+      bool have = gq < w1;
+      float3 w = make_float3(0.f, 0.f, 0.f);
+      float e2 = 0.0f;
+      float4 n0 = make_float4(0.f, 0.f, 0.f, 0.f);
+      if (tabled) {
+        if (have) {
+          const uint32_t own = s_own[wid][gq - w0];
+          j = (int)(own & 31u);
+          const Seg& S = segs[j];
+          n0 = S.n0;
+          const uint32_t b = __float_as_uint(n0.w);
+          const uint2 bx = S.box[own >> 5];
+          const uint32_t rem = gq - __float_as_uint(S.n1.w) - (bx.y & 0xffffu);
+          // rem < 256 and a width below 16: exact (rem * (magic * width - 4096) < 4096)
+          const uint32_t dj = (rem * (bx.y >> 16)) >> 12;
+          place(b & 3u, (int)(((b >> 2) & 1023u) + (own >> 5)), (int)((bx.x & 1023u) + dj),
+                (int)(((bx.x >> 10) & 1023u) + rem - dj * (bx.x >> 20)), x, y, z);
+        }
+      } else {
+        // a warp with a long segment: the owner by a binary search over the
+        // inclusive prefix of the candidate counts
 #pragma unroll
-    for (int st = 16; st > 0; st >>= 1)
-      if (__shfl_sync(FULLW, incl, j + st - 1) <= gq) j += st;
-    j = min(j, 31);
-    int x = 0, y = 0, z = 0, dec = 0;
-    PackedWalk p;
-    if (gq < total) {
-      p = s_w[wb + j];
-      // with the force_exact test option every pair goes on to the exact path
-      if (decode_candidate(p, g.n, gq - __float_as_uint(p.w3.w), x, y, z))
-        dec = g.force_exact ? -1 : seg_stage1_at(f3(p.w0), f3(p.w1), x, y, z, g.rl);
+        for (int st = 16; st > 0; st >>= 1)
+          if (__shfl_sync(FULLW, incl, j + st - 1) <= gq) j += st;
+        j = min(j, 31);
+        if (have) {
+          const Seg& S = segs[j];
+          n0 = S.n0;
+          const uint32_t b = __float_as_uint(n0.w), q = gq - __float_as_uint(S.n1.w);
+          if (b & (1u << 14)) {
+            uint32_t sl = 0;
+            while (sl + 1 < (uint32_t)kBoxSlabs && slab_end(S, (int)sl, 0u, 0xffffu) <= q) ++sl;
+            const uint2 bx = S.box[sl];
+            const uint32_t rem = q - (bx.y & 0xffffu), dj = (rem * (bx.y >> 16)) >> 12;
+            place(b & 3u, (int)(((b >> 2) & 1023u) + sl), (int)((bx.x & 1023u) + dj),
+                  (int)(((bx.x >> 10) & 1023u) + rem - dj * (bx.x >> 20)), x, y, z);
+          } else {
+            have = decode_long(S, b, g.n, q, x, y, z);
+          }
+        }
+      }
+      if (have) {
+        // Stage 1. The axis point p = v0 + t d nearest the voxel's centre lies e
+        // from it: the box is within rl of p, so of the segment (accept), or it
+        // lies, along e, beyond |e| - |e|_1 / (2 |e|) = u / |e| of p and so, p being
+        // the nearest point, of the whole segment (reject when that squared
+        // exceeds rl^2 by the allowance), or the pair is undecided.
+        const Seg& S = segs[j];
+        float t;
+        float3 e;
+        e2 = offset(S, x, y, z, w, t, e);
+        const float fx = fabsf(e.x), fy = fabsf(e.y), fz = fabsf(e.z);
+        const float ex_ = fmaxf(fx - 0.5f, 0.0f), ey = fmaxf(fy - 0.5f, 0.0f), ez = fmaxf(fz - 0.5f, 0.0f);
+        const float up2 = ex_ * ex_ + ey * ey + ez * ez;
+        const float u = fmaf(-0.5f, fx + fy + fz, e2);
+        dec = up2 <= S.d.w ? 1 : (u > 0.0f && u * u > (rl2x2 - S.d.w) * e2 ? 0 : -1);
+        if (g.force_exact) dec = -1;  // with the test option every pair goes on to the exact path
+      }
+      const unsigned um = __ballot_sync(FULLW, dec < 0);
+      if (dec < 0) uq[un + __popc(um & lt)] = make_uint2((uint32_t)j, pack_voxel(x, y, z));
+      un += __popc(um);
+      emit(dec > 0, j, n0, w, e2, x, y, z);
+      if (un >= 32) {
+        __syncwarp();
+        stage2(32);
+        __syncwarp();
+        // entries past the first 32 move to the front (reads 32.., writes ..31)
+        if ((uint32_t)lane < un - 32) uq[lane] = uq[32 + lane];
+        __syncwarp();
+        un -= 32;
+      }
     }
-    const unsigned um = __ballot_sync(FULLW, dec < 0);
-    if (dec < 0) uq[un + __popc(um & lt)] = make_uint2((uint32_t)j, pack_voxel(x, y, z));
-    un += __popc(um);
-    emit(dec > 0, j, p, x, y, z);
-    if (un >= 32) {
-      __syncwarp();
-      stage2(32);
-      __syncwarp();
-      // entries past the first 32 move to the front (reads 32.., writes ..31)
-      if ((uint32_t)lane < un - 32) uq[lane] = uq[32 + lane];
-      __syncwarp();
-      un -= 32;
-    }
+    sq += sq32;
+    sq32 = 0;
+    __syncwarp();
   }
   __syncwarp();
-  stage2(un);
+  if (un) stage2(un);
+  sq += sq32;
   flush_rank();
-  for (uint32_t k = wcount + lane; k < total; k += 32) {  // slots of candidates not kept
-    const unsigned long long r = rbase + k;
-    if (r < g.rec_cap) g.rec[r] = kNoRecord;
-  }
-  flush_counters_block(g.st, F, sq, ex);
+  if (lane == 0 && wcount > room) set_err(g.st, kErrOverflow);
+  for (uint32_t q = wcount + lane; q < room; q += 32) rec[q] = kNoRecord;  // candidates not kept
+  flush_counters_block(g.st, lane == 0 ? (unsigned long long)wcount : 0ull, sq, ex);
 }
 
 // Exact decisions of pass 1's undecided pairs.
@@ -661,7 +722,9 @@ int launch_pass1(const float4* pos, const float4* nrm, const uint32_t* order, lo
   // measured slower at 256^3 (bundles pass 1 2.3 -> 3.5 ms) and, since pass 1's
   // atomics return the rank, at 512^3 too (ABC pathlines 4.70 -> 6.83 ms; it
   // paid there while they returned nothing, 7.8 -> 7.4 ms).
-  k_pass1<<<(unsigned)((V + T - 1) / T), T, 0, s>>>(pos, nrm, order, V, g);
+  const int spw = pass1_segments_per_warp(V);
+  const long long per_block = (long long)spw * kPass1Warps;
+  k_pass1<<<(unsigned)((V + per_block - 1) / per_block), kPass1Threads, 0, s>>>(pos, nrm, order, V, spw, g);
   k_exact1<<<152 * 4, T, 0, s>>>(pos, nrm, g);
   return 2;
 }

@@ -131,52 +131,19 @@ __device__ __forceinline__ float dot3(float3 a, float3 b) { return fmaf(a.x, b.x
 __device__ __forceinline__ float cmp3(float3 a, int k) { return k == 0 ? a.x : (k == 1 ? a.y : a.z); }
 
 // ------------------------------------------------- list membership predicate
-// Decides dist(segment [a, a + d], unit box [0,1]^3) <= rl, with a and d in
-// voxel units relative to the box's lower corner (exact fp32 multiples of
-// 2^-14). Returns 1 (within), 0 (not within) or -1 (too close to call in fp32).
-//
-// Stage 1 takes a point p = a + t d of the segment near the box centre c (t
-// from the projection of c, clamped to [0, 1]), e = c - p:
-//   dist(p, box) <= rl -> within (p is on the segment)
-//   |e| - (|e_x| + |e_y| + |e_z|) / (2 |e|) - reach > rl -> not within: along
-//     the unit normal e / |e| the box lies at least |e| - (half its 1-norm)
-//     beyond p, and the segment reaches at most
-//     reach = max(0, -t d.e, (1 - t) d.e) / |e| beyond p (its endpoints are
-//     p - t d and p + (1 - t) d). This holds for any t, so the projection
-//     needs no exact division.
-// Stage 2 runs Newton steps on the convex, C^1, piecewise-quadratic squared
-// box distance f(t) and brackets its minimum: f(t) is an upper bound, and
-// convexity gives f(t) - |f'(t)| * (t or 1 - t) as a lower bound, again for
-// any t.
-// Both stages add a rounding allowance proportional to the squared magnitude
-// of the local coordinates.
-// Rounding allowance of both stages for local coordinates a, a + d.
+// dist(segment [a, a + d], unit box [0,1]^3) <= rl, with a and d in voxel units
+// relative to the box's lower corner (exact fp32 multiples of 2^-14), is decided
+// in stages, each with a rounding allowance proportional to the squared magnitude
+// of the local coordinates. Stage 1 (pass 1, voxelize.cu) tests the point of the
+// segment nearest the box's centre. Stage 2 runs Newton steps on the convex, C^1,
+// piecewise-quadratic squared box distance f(t) and brackets its minimum: f(t) is
+// an upper bound, and convexity gives f(t) - |f'(t)| * (t or 1 - t) as a lower
+// bound, for any t. What is still too close to call goes to the exact decision.
+// Rounding allowance of stage 2 for local coordinates a, a + d.
 __device__ __forceinline__ float seg_box_tol(float3 a, float3 d) {
   const float M = fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fabsf(a.z)),
                         fmaxf(fmaxf(fabsf(a.x + d.x), fabsf(a.y + d.y)), fabsf(a.z + d.z)));
   return 4.8e-7f * (M + 2.0f) * (M + 2.0f);
-}
-
-// Stage 1: 1 within, 0 not within, -1 undecided.
-__device__ __forceinline__ int seg_box_stage1(float3 a, float3 d, float rl) {
-  const float tol = seg_box_tol(a, d);
-  const float dd = dot3(d, d);
-  const float3 w = make_float3(0.5f - a.x, 0.5f - a.y, 0.5f - a.z);
-  const float t = dd > 0.0f ? fminf(1.0f, fmaxf(0.0f, __fdividef(dot3(w, d), dd))) : 0.0f;
-  const float3 e = w - t * d;  // c - p
-  const float ex = fmaxf(fabsf(e.x) - 0.5f, 0.0f), ey = fmaxf(fabsf(e.y) - 0.5f, 0.0f),
-              ez = fmaxf(fabsf(e.z) - 0.5f, 0.0f);
-  const float up2 = ex * ex + ey * ey + ez * ez;  // dist(p, box)^2
-  if (up2 + tol <= rl * rl) return 1;
-  const float e2 = dot3(e, e);
-  if (e2 > 0.0f) {
-    const float len = sqrtf(e2);
-    const float de = dot3(d, e);
-    const float reach = fmaxf(0.0f, fmaxf(-t * de, (1.0f - t) * de));
-    const float lb = len - __fdividef(0.5f * (fabsf(e.x) + fabsf(e.y) + fabsf(e.z)) + reach, len);
-    if (lb > rl && lb * lb - tol > rl * rl) return 0;
-  }
-  return -1;
 }
 
 // Stage 2: 1 within, 0 not within, -1 undecided (left to the exact decision).
@@ -307,17 +274,6 @@ static __device__ __noinline__ bool seg_box_exact(const long long* A, const long
     if (seg_near_point<3>(W, D, r, R2)) return true;
   }
   return false;
-}
-
-// Filter stages for voxel (x, y, z): 1 within, 0 not, -1 undecided. a, b are
-// the snapped global endpoints (local coordinates are exact in fp32).
-__device__ __forceinline__ int seg_stage1_at(float3 a, float3 b, int x, int y, int z, float rl) {
-  const float3 la = make_float3(a.x - (float)x, a.y - (float)y, a.z - (float)z);
-  return seg_box_stage1(la, b - a, rl);
-}
-__device__ __forceinline__ int seg_stage2_at(float3 a, float3 b, int x, int y, int z, float rl) {
-  const float3 la = make_float3(a.x - (float)x, a.y - (float)y, a.z - (float)z);
-  return seg_box_stage2(la, b - a, rl);
 }
 
 // Exact decision for voxel (x, y, z) on the 2^-14 lattice.
