@@ -274,17 +274,6 @@ __device__ __forceinline__ uint32_t add_fragment(const GridDev& g, float3 a, flo
 // A record slot pass 1 took for a candidate it did not keep.
 constexpr unsigned long long kNoRecord = ~0ull;
 
-__device__ __forceinline__ void append_record(const GridDev& g, uint32_t idx, uint32_t seg,
-                                              uint32_t rank) {
-  const unsigned long long r = atomicAdd(&g.st->rec_cnt, 1ull);
-  if (r < g.rec_cap) {
-    g.rec[r] = ((unsigned long long)idx << 32) | seg;
-    g.rank[r] = (uint16_t)rank;
-  } else {
-    set_err(g.st, kErrOverflow);
-  }
-}
-
 constexpr int kWarpRecords = 256;  // pass 2: culled records a warp stages per append
 constexpr uint32_t kNoCopy = 0xffffffffu;  // cq_cnt: pass 2 copied no culled records
 
@@ -555,21 +544,50 @@ __global__ void __launch_bounds__(kPass1Threads, kPass1Blocks) k_pass1(const flo
   flush_counters_block(g.st, lane == 0 ? (unsigned long long)wcount : 0ull, sq, ex);
 }
 
-// Exact decisions of pass 1's undecided pairs.
-__global__ void __launch_bounds__(256) k_exact1(const float4* __restrict__ pos,
+// Decisions of pass 1's undecided pairs (a few in 100k): in pairs of floats, and
+// what those leave (ties, or every pair with the force_exact test option) in
+// 128-bit integers. The kept ones take their record slots with one atomic per
+// warp. Few and long, so latency bound: a small grid starts soonest.
+constexpr int kExactThreads = 128;
+__global__ void __launch_bounds__(kExactThreads) k_exact1(const float4* __restrict__ pos,
                                                 const float4* __restrict__ nrm, GridDev g) {
   const uint32_t cnt = min(g.st->xq_cnt, g.xq_cap);
+  const int lane = threadIdx.x & 31;
   unsigned long long F = 0, sq = 0;
-  for (uint32_t e = blockIdx.x * blockDim.x + threadIdx.x; e < cnt; e += gridDim.x * blockDim.x) {
-    const uint2 it = g.xq[e];
-    int x, y, z;
-    unpack_voxel(it.y, x, y, z);
-    const float4 p0 = pos[it.x], p1 = pos[it.x + 1];
-    if (!seg_exact_at(f3(p0), f3(p1), x, y, z, g.RL)) continue;
-    const uint32_t rank =
-        add_fragment(g, f3(p0), f3(p1), f3(nrm[it.x]), f3(nrm[it.x + 1]),
-                     __float_as_uint(p0.w) & kClipOn, __float_as_uint(p1.w) & kClipOn, x, y, z, F, sq);
-    append_record(g, brick_index(x, y, z, g.log2nb), it.x, rank);
+  const unsigned long long step = gridDim.x * blockDim.x;
+  for (unsigned long long e0 = (blockIdx.x * blockDim.x + threadIdx.x) & ~31u; e0 < cnt; e0 += step) {
+    const unsigned long long e = e0 + lane;
+    bool keep = false;
+    uint32_t seg = 0, idx = 0, rank = 0;
+    if (e < cnt) {
+      const uint2 it = g.xq[e];
+      seg = it.x;
+      int x, y, z;
+      unpack_voxel(it.y, x, y, z);
+      const float4 p0 = pos[seg], p1 = pos[seg + 1];
+      const float3 la = make_float3(p0.x - (float)x, p0.y - (float)y, p0.z - (float)z);
+      const int dec = g.force_exact ? -1 : seg_box_stage3(la, f3(p1) - f3(p0), g.rl);
+      keep = dec < 0 ? seg_exact_at(f3(p0), f3(p1), x, y, z, g.RL) : dec > 0;
+      if (keep) {
+        idx = brick_index(x, y, z, g.log2nb);
+        rank = add_fragment(g, f3(p0), f3(p1), f3(nrm[seg]), f3(nrm[seg + 1]),
+                            __float_as_uint(p0.w) & kClipOn, __float_as_uint(p1.w) & kClipOn, x, y, z,
+                            F, sq);
+      }
+    }
+    const unsigned km = __ballot_sync(FULLW, keep);
+    if (!km) continue;
+    unsigned long long r = 0;
+    if (lane == 0) r = atomicAdd(&g.st->rec_cnt, (unsigned long long)__popc(km));
+    r = __shfl_sync(FULLW, r, 0) + __popc(km & ((1u << lane) - 1u));
+    if (keep) {
+      if (r < g.rec_cap) {
+        g.rec[r] = ((unsigned long long)idx << 32) | seg;
+        g.rank[r] = (uint16_t)rank;
+      } else {
+        set_err(g.st, kErrOverflow);
+      }
+    }
   }
   unsigned long long z0 = 0;
   flush_counters(g.st, F, sq, z0);
@@ -716,7 +734,6 @@ __global__ void __launch_bounds__(256) k_scatter_culled(GridDev g) {
 int launch_pass1(const float4* pos, const float4* nrm, const uint32_t* order, long long V,
                  const GridDev& g, cudaStream_t s) {
   if (V < 2) return 0;
-  const int T = 256;
   // One atomic per fragment at every grid side: summing the increments of the
   // lanes of a warp step that share a voxel first (a match on the voxel index)
   // measured slower at 256^3 (bundles pass 1 2.3 -> 3.5 ms) and, since pass 1's
@@ -725,7 +742,7 @@ int launch_pass1(const float4* pos, const float4* nrm, const uint32_t* order, lo
   const int spw = pass1_segments_per_warp(V);
   const long long per_block = (long long)spw * kPass1Warps;
   k_pass1<<<(unsigned)((V + per_block - 1) / per_block), kPass1Threads, 0, s>>>(pos, nrm, order, V, spw, g);
-  k_exact1<<<152 * 4, T, 0, s>>>(pos, nrm, g);
+  k_exact1<<<152 * 2, kExactThreads, 0, s>>>(pos, nrm, g);
   return 2;
 }
 

@@ -146,34 +146,114 @@ __device__ __forceinline__ float seg_box_tol(float3 a, float3 d) {
   return 4.8e-7f * (M + 2.0f) * (M + 2.0f);
 }
 
+// Newton's step from t on the piecewise linear, increasing derivative of f (half
+// of it g, its slope gp), kept inside the bracket [lo, hi] of the minimiser, which
+// it narrows first; a step onto an end that has been tried goes to the middle
+// instead (the plain step can go back and forth across a face for ever).
+struct Bracket {
+  float lo = 0.0f, hi = 1.0f;
+  bool tried_lo = false, tried_hi = false;
+  __device__ __forceinline__ float next(float t, float g, float gp) {
+    if (g > 0.0f) { hi = t; tried_hi = true; }
+    else { lo = t; tried_lo = true; }
+    const float u = fminf(hi, fmaxf(lo, t - __fdividef(g, gp)));
+    return (u == lo && tried_lo) || (u == hi && tried_hi) ? 0.5f * (lo + hi) : u;
+  }
+};
+constexpr int kNewtonSteps = 8;
+
 // Stage 2: 1 within, 0 not within, -1 undecided (left to the exact decision).
 __device__ __forceinline__ int seg_box_stage2(float3 a, float3 d, float rl) {
   const float tol = seg_box_tol(a, d);
   const float dd = dot3(d, d);
   const float3 w = make_float3(0.5f - a.x, 0.5f - a.y, 0.5f - a.z);
+  const float rl2 = rl * rl;
   float t = dd > 0.0f ? fminf(1.0f, fmaxf(0.0f, __fdividef(dot3(w, d), dd))) : 0.0f;
-  float f = 0.0f, g = 0.0f;
-#pragma unroll
-  for (int it = 0; it < 4; ++it) {
-    float gg = 0.0f, gp = 0.0f, ff = 0.0f;
+  Bracket br;
+  for (int it = 0; it < kNewtonSteps; ++it) {
+    float g = 0.0f, gp = 0.0f, f = 0.0f;
 #pragma unroll
     for (int k = 0; k < 3; ++k) {
       const float ak = cmp3(a, k), dk = cmp3(d, k);
       const float x = fmaf(t, dk, ak);
       const float e = x < 0.0f ? x : (x > 1.0f ? x - 1.0f : 0.0f);
-      gg = fmaf(dk, e, gg);
-      ff = fmaf(e, e, ff);
+      g = fmaf(dk, e, g);
+      f = fmaf(e, e, f);
       if (e != 0.0f) gp = fmaf(dk, dk, gp);
     }
-    f = ff;
-    g = gg;
-    if (it == 3 || gp == 0.0f) break;
-    t = fminf(1.0f, fmaxf(0.0f, t - __fdividef(gg, gp)));
+    if (f + tol <= rl2) return 1;
+    const float lb = f - 2.0f * fabsf(g) * (g > 0.0f ? t - br.lo : br.hi - t);
+    if (lb - tol > rl2) return 0;
+    if (gp == 0.0f) break;
+    t = br.next(t, g, gp);
   }
-  const float rl2 = rl * rl;
-  if (f + tol <= rl2) return 1;
-  const float lb = f - 2.0f * fabsf(g) * (g > 0.0f ? t : 1.0f - t);
-  if (lb - tol > rl2) return 0;
+  return -1;
+}
+
+// Stage 3: stage 2's bracket in pairs of floats (about 46 bits, by error-free sums
+// and products), which decides all but true ties and pairs within 1e-12 (M + 2)^2
+// of one, M the largest local coordinate: the pair arithmetic below errs by at
+// most a few units of 2^-44 M^2. 1 within, 0 not within, -1 undecided.
+__device__ __forceinline__ void two_sum(float a, float b, float& s, float& e) {
+  s = __fadd_rn(a, b);
+  const float v = __fsub_rn(s, a);
+  e = __fadd_rn(__fsub_rn(a, __fsub_rn(s, v)), __fsub_rn(b, v));
+}
+__device__ __forceinline__ int seg_box_stage3(float3 a, float3 d, float rl) {
+  const float dd = dot3(d, d);
+  const float3 w = make_float3(0.5f - a.x, 0.5f - a.y, 0.5f - a.z);
+  const float M = fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fabsf(a.z)),
+                        fmaxf(fmaxf(fabsf(a.x + d.x), fabsf(a.y + d.y)), fabsf(a.z + d.z)));
+  const float tol = 1e-12f * (M + 2.0f) * (M + 2.0f);
+  const float rh = __fmul_rn(rl, rl), re = fmaf(rl, rl, -rh);
+  float t = dd > 0.0f ? fminf(1.0f, fmaxf(0.0f, __fdividef(dot3(w, d), dd))) : 0.0f;
+  Bracket br;
+  float tl = 0.0f;  // the parameter is t + tl
+  for (int it = 0; it < kNewtonSteps + 4; ++it) {
+    float fh = 0.0f, fl = 0.0f, gh = 0.0f, gl = 0.0f, gp = 0.0f;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+      const float ak = cmp3(a, k), dk = cmp3(d, k);
+      // x = a + (t + tl) d
+      const float p = __fmul_rn(t, dk), pe = fmaf(t, dk, -p);
+      float s, e, xh, xl;
+      two_sum(ak, p, s, e);
+      two_sum(s, __fadd_rn(e, fmaf(tl, dk, pe)), xh, xl);
+      // its offset from [0, 1]
+      if (xh > 1.0f || (xh == 1.0f && xl > 0.0f)) {
+        two_sum(xh, -1.0f, xh, e);
+        xl = __fadd_rn(xl, e);
+      } else if (!(xh < 0.0f || (xh == 0.0f && xl < 0.0f))) {
+        continue;
+      }
+      const float q = __fmul_rn(xh, xh), qe = fmaf(2.0f * xh, xl, fmaf(xh, xh, -q));
+      two_sum(fh, q, fh, e);
+      fl = __fadd_rn(fl, __fadd_rn(e, qe));
+      const float r = __fmul_rn(dk, xh), rl_ = fmaf(dk, xl, fmaf(dk, xh, -r));
+      two_sum(gh, r, gh, e);
+      gl = __fadd_rn(gl, __fadd_rn(e, rl_));
+      gp = fmaf(dk, dk, gp);
+    }
+    float vh, ve;
+    two_sum(fh, -rh, vh, ve);
+    const float v = __fadd_rn(vh, __fadd_rn(ve, __fsub_rn(fl, re)));  // squared distance - rl^2
+    if (v + tol <= 0.0f) return 1;
+    const float g = __fadd_rn(gh, gl);
+    // convexity over the whole segment: the minimum is at most this far below
+    const float gap = 2.0f * fabsf(g) * (g > 0.0f ? t : 1.0f - t) * 1.000001f;
+    if (v - gap - tol > 0.0f) return 0;
+    if (gp == 0.0f || (g > 0.0f && t == 0.0f) || (g < 0.0f && t == 1.0f)) break;
+    // near the minimiser the step refines the pair; before that, as in stage 2
+    const float step = __fdividef(g, gp);
+    if (fabsf(step) < 1e-5f) {
+      two_sum(t, __fsub_rn(tl, step), t, tl);
+      if (t < 0.0f || (t == 0.0f && tl < 0.0f)) t = tl = 0.0f;
+      if (t > 1.0f || (t == 1.0f && tl > 0.0f)) { t = 1.0f; tl = 0.0f; }
+    } else {
+      t = br.next(t, g, gp);
+      tl = 0.0f;
+    }
+  }
   return -1;
 }
 
