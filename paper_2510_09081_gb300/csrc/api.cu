@@ -697,9 +697,8 @@ vrt_status vrt_cull(vrt_grid g, const vrt_camera* cam, const vrt_render_params* 
   }
   // reset the list-build counters (scan tile counter .. end)
   const size_t off = offsetof(DevStatus, sum_count_field);
-  VRT_CUDA(g, cudaMemsetAsync((char*)g->st + off, 0, sizeof(DevStatus) - off, g->stream));
-  VRT_CUDA(g, cudaMemsetAsync((char*)g->st + offsetof(DevStatus, occupied_voxels), 0, sizeof(unsigned int), g->stream));
-  VRT_CUDA(g, cudaMemsetAsync(g->tile_state, 0, (size_t)g->n_tiles * 8, g->stream));
+  g->launches += launch_reset((uint32_t*)((char*)g->st + off), (uint32_t)((sizeof(DevStatus) - off) / 4),
+                              (uint32_t*)g->tile_state, 2 * g->n_tiles, g->stream);
   stage_mark(g, ST_CULL, 0);
   if (cull) {
     if (!g->eroded) VRT_CUDA(g, dalloc(g, &g->eroded, nv));
@@ -717,7 +716,6 @@ vrt_status vrt_cull(vrt_grid g, const vrt_camera* cam, const vrt_render_params* 
   stage_mark(g, ST_SCAN, 0);
   g->launches += launch_scan(d, cull ? 0 : 1, g->tile_state, g->n_tiles, g->scan_stall,
                              g->scan_stall >= 0 ? kSpinLimitTest : 0, g->stream);
-  g->launches += launch_finalize(d, g->stream);
   stage_mark(g, ST_SCAN, 1);
   stage_mark(g, ST_PASS2, 0);
   g->launches += launch_scatter(d, cull ? 1 : 0, nullptr, nullptr, g->stream);
@@ -824,9 +822,7 @@ vrt_status vrt_trace(vrt_grid g, const vrt_camera* cam, const vrt_render_params*
   // round queues without limit, so the last round always completes.
   a.max_queue = kMaxRepairRounds >= 2 ? kRayQueueLimit : 0xffffffffu;
   VRT_CUDA(g, cudaMemsetAsync((char*)g->st + offsetof(DevStatus, vq_cnt), 0,
-                              4 * sizeof(unsigned int), g->stream));
-  VRT_CUDA(g, cudaMemsetAsync((char*)g->st + offsetof(DevStatus, tr_next), 0,
-                              sizeof(unsigned int) * (kMaxRepairRounds + 1), g->stream));
+                              sizeof(unsigned int) * (4 + kMaxRepairRounds + 1), g->stream));
   a.work_next = &g->st->tr_next[0];
   a.short_list = g->short_list;
   a.ray_keys = g->ray_keys;

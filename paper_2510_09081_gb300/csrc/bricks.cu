@@ -16,7 +16,7 @@ namespace vrt {
 // 512 contiguous bytes) and the brick's 16 threads combine their four bits.
 __global__ void __launch_bounds__(256) k_brick_occ(GridDev g, uint8_t* __restrict__ out,
                                                    uint2* __restrict__ mask) {
-  const uint32_t row = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t row = blockIdx.x * blockDim.x + threadIdx.x + dependency_wait();
   const int lane = threadIdx.x & 31;
   const uint4 v = __ldg(reinterpret_cast<const uint4*>(g.word) + row);  // n^3 / 4 rows: whole blocks
   const uint32_t m = ((v.x & 0xffffu) ? 1u : 0u) | ((v.y & 0xffffu) ? 2u : 0u) |
@@ -37,7 +37,7 @@ __global__ void __launch_bounds__(256) k_brick_occ(GridDev g, uint8_t* __restric
 __global__ void __launch_bounds__(256) k_brick_dist(int log2nb, int axis,
                                                     const uint8_t* __restrict__ in,
                                                     uint8_t* __restrict__ out) {
-  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t b = blockIdx.x * blockDim.x + threadIdx.x + dependency_wait();
   const uint32_t nb = 1u << (3 * log2nb);
   if (b >= nb) return;
   const int side = 1 << log2nb;
@@ -52,19 +52,32 @@ __global__ void __launch_bounds__(256) k_brick_dist(int log2nb, int axis,
   out[b] = (uint8_t)d;
 }
 
+__global__ void __launch_bounds__(256) k_reset(uint32_t* a, uint32_t na, uint32_t* b, uint32_t nb) {
+  dependency_wait();
+  for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < na + nb; i += gridDim.x * blockDim.x)
+    if (i < na) a[i] = 0u;
+    else b[i - na] = 0u;
+}
+
+int launch_reset(uint32_t* a, uint32_t na, uint32_t* b, uint32_t nb, cudaStream_t s) {
+  const unsigned blocks = (na + nb + 1023) / 1024;
+  launch_chained(k_reset, blocks < 152u ? blocks : 152u, 256, s, a, na, b, nb);
+  return 1;
+}
+
 int launch_brick_dist_passes(int log2nb, uint8_t* tmp, uint8_t* dist, cudaStream_t s) {
   const uint32_t nb = 1u << (3 * log2nb);
   const int T = 256;
   const unsigned blocks = (nb + T - 1) / T;
-  k_brick_dist<<<blocks, T, 0, s>>>(log2nb, 0, tmp, dist);
-  k_brick_dist<<<blocks, T, 0, s>>>(log2nb, 1, dist, tmp);
-  k_brick_dist<<<blocks, T, 0, s>>>(log2nb, 2, tmp, dist);
+  launch_chained(k_brick_dist, blocks, T, s, log2nb, 0, tmp, dist);
+  launch_chained(k_brick_dist, blocks, T, s, log2nb, 1, dist, tmp);
+  launch_chained(k_brick_dist, blocks, T, s, log2nb, 2, tmp, dist);
   return 3;
 }
 
 int launch_brick_dist(const GridDev& g, uint8_t* tmp, uint8_t* dist, uint2* mask, cudaStream_t s) {
   const int T = 256;
-  k_brick_occ<<<(1u << (3 * g.log2nb + 4)) / T, T, 0, s>>>(g, tmp, mask);
+  launch_chained(k_brick_occ, (1u << (3 * g.log2nb + 4)) / T, T, s, g, tmp, mask);
   return 1 + launch_brick_dist_passes(g.log2nb, tmp, dist, s);
 }
 

@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(256) k_erode(GridDev g, uint8_t* __restrict__ 
                                                float* __restrict__ emean,
                                                uint32_t* __restrict__ occq,
                                                unsigned long long occq_cap) {
-  const uint32_t row = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t row = blockIdx.x * blockDim.x + threadIdx.x + dependency_wait();
   const uint32_t nrow = ((uint32_t)g.n * g.n * g.n) >> 2;  // a multiple of 32 (n >= 16)
   const int lane = threadIdx.x & 31;
   if (row >= nrow) return;  // whole warps
@@ -244,7 +244,7 @@ __global__ void __launch_bounds__(256) k_visible(GridDev g, CullCam cc,
                                                  const uint8_t* __restrict__ eroded,
                                                  const uint8_t* __restrict__ cdist,
                                                  const float* __restrict__ emean) {
-  const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x;
+  const uint32_t idx = blockIdx.x * blockDim.x + threadIdx.x + dependency_wait();
   const uint32_t nvox = (uint32_t)g.n * g.n * g.n;
   const bool visible = idx < nvox && (__ldg(&g.word[idx]) & 0xffffu) &&
                        voxel_visible(g, cc, eroded, cdist, emean, idx);
@@ -261,8 +261,9 @@ __global__ void __launch_bounds__(256) k_visible_queued(GridDev g, CullCam cc,
                                                         const float* __restrict__ emean,
                                                         const uint32_t* __restrict__ occq,
                                                         unsigned long long occq_cap) {
+  const uint32_t first = blockIdx.x * blockDim.x + threadIdx.x + dependency_wait();
   const unsigned long long cnt = min((unsigned long long)g.st->occq_cnt, occq_cap);
-  for (unsigned long long q = (unsigned long long)blockIdx.x * blockDim.x + threadIdx.x; q < cnt;
+  for (unsigned long long q = first; q < cnt;
        q += (unsigned long long)gridDim.x * blockDim.x) {
     const uint32_t idx = __ldg(&occq[q]);
     if (voxel_visible(g, cc, eroded, cdist, emean, idx)) atomicOr(&g.vis[idx >> 5], 1u << (idx & 31));
@@ -316,11 +317,11 @@ int launch_cull(const GridDev& g, const HostCamera& cam, float alpha, uint8_t* e
   // the queue holds every voxel at most once, so it never overflows when it
   // has room for the whole grid; otherwise each voxel's thread tests its own
   const bool queued = occq && occq_cap >= nvox;
-  k_erode<<<(nvox / 4 + T - 1) / T, T, 0, s>>>(g, eroded, btmp, emean, queued ? occq : nullptr,
-                                               occq_cap);
+  launch_chained(k_erode, (nvox / 4 + T - 1) / T, T, s, g, eroded, btmp, emean,
+                 queued ? occq : nullptr, occq_cap);
   const int passes = launch_brick_dist_passes(g.log2nb, btmp, cdist, s);
-  if (queued) k_visible_queued<<<152 * 8, T, 0, s>>>(g, cc, eroded, cdist, emean, occq, occq_cap);
-  else k_visible<<<(nvox + T - 1) / T, T, 0, s>>>(g, cc, eroded, cdist, emean);
+  if (queued) launch_chained(k_visible_queued, 152 * 8, T, s, g, cc, eroded, cdist, emean, occq, occq_cap);
+  else launch_chained(k_visible, (nvox + T - 1) / T, T, s, g, cc, eroded, cdist, emean);
   return 2 + passes;
 }
 

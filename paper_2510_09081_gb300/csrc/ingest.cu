@@ -20,7 +20,7 @@ __global__ void __launch_bounds__(256) k_ingest(const float* __restrict__ raw,
                                                 const uint8_t* __restrict__ flags, long long lo,
                                                 long long hi, float4* __restrict__ pos,
                                                 float4* __restrict__ nrm, DevStatus* st) {
-  const long long i = lo + (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long i = lo + (long long)blockIdx.x * blockDim.x + threadIdx.x + dependency_wait();
   if (i >= hi) return;
   bool bad = false;
   const float x = snap(raw[3 * i], bad), y = snap(raw[3 * i + 1], bad), z = snap(raw[3 * i + 2], bad);
@@ -47,7 +47,7 @@ int launch_ingest(const float* raw, const uint8_t* flags, long long lo, long lon
                   float4* nrm, DevStatus* st, cudaStream_t s) {
   if (hi <= lo) return 0;
   const int T = 256;
-  k_ingest<<<(unsigned)((hi - lo + T - 1) / T), T, 0, s>>>(raw, flags, lo, hi, pos, nrm, st);
+  launch_chained(k_ingest, (unsigned)((hi - lo + T - 1) / T), T, s, raw, flags, lo, hi, pos, nrm, st);
   return 1;
 }
 

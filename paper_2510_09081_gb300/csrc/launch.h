@@ -9,6 +9,26 @@
 
 namespace vrt {
 
+// Launches `kernel` so that it may start while the kernel before it on the stream
+// drains: its blocks are resident, waiting in dependency_wait(), when that one
+// completes, which saves most of a launch's latency (a frame of a small set is a
+// chain of 11 to 33 kernels of a few microseconds). Every kernel launched this
+// way calls dependency_wait() before it touches memory. After a copy, a memset or
+// an event the stream orders it as usual.
+template <class... P, class... A>
+void launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, cudaStream_t s, A... args) {
+  cudaLaunchConfig_t c = {};
+  c.gridDim = grid;
+  c.blockDim = dim3(threads);
+  c.stream = s;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // Camera as given through the C ABI, widened to fp64 on the host.
 struct HostCamera {
   int width, height, ortho;
@@ -81,6 +101,8 @@ struct ShadeArgs {
 };
 // Every voxel next to a listed one (one block per brick); rewrites the mask.
 int launch_shade(const ShadeArgs& a, cudaStream_t s);
+// Zeroes up to two ranges of 32-bit words.
+int launch_reset(uint32_t* a, uint32_t na, uint32_t* b, uint32_t nb, cudaStream_t s);
 // Voxels next to the voxels a repair round listed, not yet shaded this frame.
 int launch_shade_repair(const ShadeArgs& a, cudaStream_t s);
 
@@ -122,7 +144,6 @@ int launch_scatter(const GridDev& g, int mode, const uint32_t* need, const uint3
 // so the tiles after it give up their waits after spin_limit polls.
 int launch_scan(const GridDev& g, int all_visible, unsigned long long* tile_state, uint32_t n_tiles,
                 int stall_tile, int spin_limit, cudaStream_t s);
-int launch_finalize(const GridDev& g, cudaStream_t s);
 int launch_mips(const GridDev& g, void* mips, int fmt, const long long* lev_off, int n_levels,
                 cudaStream_t s);
 // Cull marks; btmp, cdist: one byte per brick (scratch; distance to a brick

@@ -26,7 +26,7 @@ __device__ __forceinline__ float load_texel(const __nv_bfloat16* p) { return __b
 template <class T>
 __global__ void __launch_bounds__(256) k_mip01(GridDev g, T* __restrict__ l0, T* __restrict__ l1) {
   const int m = g.n >> 1;
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x + dependency_wait();
   if (t >= (long long)m * m * m) return;
   const int x = (int)(t % m), y = (int)((t / m) % m), z = (int)(t / ((long long)m * m));
   const float inv = 1.0f / g.occ_scale;
@@ -48,7 +48,7 @@ __global__ void __launch_bounds__(256) k_mip01(GridDev g, T* __restrict__ l0, T*
 
 template <class T>
 __global__ void __launch_bounds__(256) k_mip_down(const T* __restrict__ src, T* __restrict__ dst, int m) {
-  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  const long long t = (long long)blockIdx.x * blockDim.x + threadIdx.x + dependency_wait();
   if (t >= (long long)m * m * m) return;
   const int x = (int)(t % m), y = (int)((t / m) % m), z = (int)(t / ((long long)m * m));
   const int mp = 2 * m;
@@ -69,12 +69,12 @@ int launch_mips_t(const GridDev& g, T* mips, const long long* lev_off, int n_lev
   long long m = g.n >> 1;
   long long cnt = m * m * m;
   int launches = 1;
-  k_mip01<T><<<(unsigned)((cnt + T_ - 1) / T_), T_, 0, s>>>(g, mips + lev_off[0], mips + lev_off[1]);
+  launch_chained(k_mip01<T>, (unsigned)((cnt + T_ - 1) / T_), T_, s, g, mips + lev_off[0], mips + lev_off[1]);
   for (int l = 2; l < n_levels; ++l) {
     m = g.n >> l;
     cnt = m * m * m;
-    k_mip_down<T><<<(unsigned)((cnt + T_ - 1) / T_), T_, 0, s>>>(mips + lev_off[l - 1], mips + lev_off[l],
-                                                                 (int)m);
+    launch_chained(k_mip_down<T>, (unsigned)((cnt + T_ - 1) / T_), T_, s, mips + lev_off[l - 1],
+                   mips + lev_off[l], (int)m);
     ++launches;
   }
   return launches;

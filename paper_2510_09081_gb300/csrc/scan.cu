@@ -32,6 +32,7 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(GridDev g, int all_visibl
   __shared__ uint32_t s_warp[kScanThreads / 32];
   __shared__ uint32_t s_prefix;
   __shared__ unsigned long long s_red[4][kScanThreads / 32];
+  dependency_wait();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (tid == 0) {
     s_tile = atomicAdd(&g.st->scan_tile_counter, 1u);
@@ -165,23 +166,20 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(GridDev g, int all_visibl
     if (a2 & 0xffffffffull) atomicAdd(&g.st->occupied_voxels, (uint32_t)(a2 & 0xffffffffull));
     if (a2 >> 32) atomicAdd(&g.st->visible_voxels, (uint32_t)(a2 >> 32));
     atomicMax(&g.st->max_count, (uint32_t)a3);
+    // the last tile to add its sums checks them
+    __threadfence();
+    if (atomicAdd(&g.st->scan_tiles_done, 1u) == n_tiles - 1) {
+      __threadfence();
+      const volatile DevStatus* st = g.st;
+      if (st->sum_count_field != st->F || st->sum_occ_field != st->sum_q) set_err(g.st, kErrOverflow);
+    }
   }
-}
-
-__global__ void k_finalize(GridDev g) {
-  DevStatus* st = g.st;
-  if (st->sum_count_field != st->F || st->sum_occ_field != st->sum_q) set_err(st, kErrOverflow);
 }
 
 int launch_scan(const GridDev& g, int all_visible, unsigned long long* tile_state, uint32_t n_tiles,
                 int stall_tile, int spin_limit, cudaStream_t s) {
-  k_scan<<<n_tiles, kScanThreads, 0, s>>>(g, all_visible, tile_state, n_tiles, stall_tile,
-                                          spin_limit > 0 ? spin_limit : kSpinLimit);
-  return 1;
-}
-
-int launch_finalize(const GridDev& g, cudaStream_t s) {
-  k_finalize<<<1, 1, 0, s>>>(g);
+  launch_chained(k_scan, n_tiles, kScanThreads, s, g, all_visible, tile_state, n_tiles, stall_tile,
+                 spin_limit > 0 ? spin_limit : kSpinLimit);
   return 1;
 }
 

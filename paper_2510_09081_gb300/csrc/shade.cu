@@ -90,7 +90,7 @@ __device__ float voxel_shade(const ShadeArgs& A, int x, int y, int z) {
 __global__ void __launch_bounds__(64) k_shade(ShadeArgs A) {
   const int lb = A.g.log2nb;
   const uint32_t mb = (1u << lb) - 1u;
-  const uint32_t b = blockIdx.x;
+  const uint32_t b = blockIdx.x + dependency_wait();
   const int t = threadIdx.x;
   // a brick at distance >= 2 from every occupied brick has no listed voxel
   // within one step of any of its voxels
@@ -119,6 +119,7 @@ __global__ void __launch_bounds__(64) k_shade(ShadeArgs A) {
 // Repair round: the neighbours of each newly listed voxel not shaded yet; the
 // thread that sets a voxel's mask bit computes its value.
 __global__ void k_shade_repair(ShadeArgs A) {
+  dependency_wait();
   const uint32_t nq = min(*A.vq_cnt, A.vq_cap);
   const int n = A.g.n;
   const unsigned long long tot = (unsigned long long)nq * 27ull;
@@ -143,12 +144,12 @@ __global__ void k_shade_repair(ShadeArgs A) {
 
 int launch_shade(const ShadeArgs& a, cudaStream_t s) {
   const unsigned n_bricks = 1u << (3 * a.g.log2nb);
-  k_shade<<<n_bricks, 64, 0, s>>>(a);
+  launch_chained(k_shade, n_bricks, 64, s, a);
   return 1;
 }
 
 int launch_shade_repair(const ShadeArgs& a, cudaStream_t s) {
-  k_shade_repair<<<152, 256, 0, s>>>(a);
+  launch_chained(k_shade_repair, 152, 256, s, a);
   return 1;
 }
 

@@ -1080,9 +1080,10 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks<OPAQUE, COUNT, AO>) 
   const int tw = A.tile_w, th = A.tile_n / tw;
   const uint32_t quads_x = (uint32_t)(A.cam.width + 2 * tw - 1) / (uint32_t)(2 * tw);
   const uint32_t quads_y = (uint32_t)(A.cam.height + 2 * th - 1) / (uint32_t)(2 * th);
+  const uint32_t block = blockIdx.x + dependency_wait();
   Work W;
   for (bool more = true; more; more = !OPAQUE) {
-    uint32_t tile = blockIdx.x * (kTraceThreads / 32) + (threadIdx.x >> 5);
+    uint32_t tile = block * (kTraceThreads / 32) + (threadIdx.x >> 5);
     if (!OPAQUE) {
       if (lane == 0) tile = atomicAdd(A.work_next, 1u);
       tile = __shfl_sync(FULL, tile, 0);
@@ -1109,6 +1110,7 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks<OPAQUE, COUNT, AO>) 
   __shared__ WarpMem<OPAQUE, KEY16> s_mem[kTraceThreads / 32];
   const int lane = threadIdx.x & 31;
   WarpMem<OPAQUE, KEY16>& S = s_mem[threadIdx.x >> 5];
+  dependency_wait();
   const uint32_t total = min(*A.pix_count, A.pq_cap);
   const uint32_t n_warps = gridDim.x * (blockDim.x >> 5);
   const uint32_t share = min(32u, (total + n_warps - 1) / n_warps);
@@ -1134,7 +1136,7 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks<OPAQUE, COUNT, AO>) 
 template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
 void launch_one(const TraceArgs& a, cudaStream_t s) {
   if (a.pix_list) {
-    k_trace_list<OPAQUE, COUNT, KEY16, AO><<<152 * 4, kTraceThreads, 0, s>>>(a);
+    launch_chained(k_trace_list<OPAQUE, COUNT, KEY16, AO>, 152 * 4, kTraceThreads, s, a);
     return;
   }
   const int tw = a.tile_w, th = a.tile_n / tw;
@@ -1142,7 +1144,7 @@ void launch_one(const TraceArgs& a, cudaStream_t s) {
   // compiled to keep resident
   const unsigned blocks = OPAQUE ? ((a.cam.width + 2 * tw - 1) / (2 * tw)) * ((a.cam.height + 2 * th - 1) / (2 * th))
                                  : 152 * (COUNT ? 4 : kMinBlocks<OPAQUE, COUNT, AO>);
-  k_trace_tile<OPAQUE, COUNT, KEY16, AO><<<blocks, kTraceThreads, 0, s>>>(a);
+  launch_chained(k_trace_tile<OPAQUE, COUNT, KEY16, AO>, blocks, kTraceThreads, s, a);
 }
 
 template <bool COUNT, bool KEY16>
@@ -1183,7 +1185,7 @@ int launch_trace(const TraceArgs& args, int K, cudaStream_t s) {
 // and neighbours share texels.
 __global__ void __launch_bounds__(kTraceThreads) k_shade_hits(TraceArgs A) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int px = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7);
+  const int px = blockIdx.x * 16 + (warp & 1) * 8 + (lane & 7) + (int)dependency_wait();
   const int py = blockIdx.y * 8 + (warp >> 1) * 4 + (lane >> 3);
   if (px >= A.cam.width || py >= A.cam.height) return;
   float4* out = &A.rgba[(size_t)py * A.cam.width + px];
@@ -1201,12 +1203,13 @@ __global__ void __launch_bounds__(kTraceThreads) k_shade_hits(TraceArgs A) {
 
 int launch_shade_hits(const TraceArgs& a, cudaStream_t s) {
   const dim3 grid((a.cam.width + 15) / 16, (a.cam.height + 7) / 8);
-  k_shade_hits<<<grid, kTraceThreads, 0, s>>>(a);
+  launch_chained(k_shade_hits, grid, kTraceThreads, s, a);
   return 1;
 }
 
 // --------------------------------------------------- instrumented trace
 __global__ void k_touch_count(const uint32_t* bits, size_t words, unsigned long long* out) {
+  dependency_wait();
   unsigned long long c = 0;
   for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < words;
        i += (size_t)gridDim.x * blockDim.x)
@@ -1219,15 +1222,16 @@ __global__ void k_touch_count(const uint32_t* bits, size_t words, unsigned long 
 int launch_touch_count(const uint32_t* list_bits, size_t list_words, const uint32_t* vert_bits,
                        size_t vert_words, const uint32_t* vox_bits, size_t vox_words,
                        DevStatus* st, cudaStream_t s) {
-  k_touch_count<<<152 * 4, 256, 0, s>>>(list_bits, list_words, &st->tr_u_entries);
-  k_touch_count<<<152 * 4, 256, 0, s>>>(vert_bits, vert_words, &st->tr_u_vertices);
-  k_touch_count<<<152 * 4, 256, 0, s>>>(vox_bits, vox_words, &st->tr_u_voxels);
+  launch_chained(k_touch_count, 152 * 4, 256, s, list_bits, list_words, &st->tr_u_entries);
+  launch_chained(k_touch_count, 152 * 4, 256, s, vert_bits, vert_words, &st->tr_u_vertices);
+  launch_chained(k_touch_count, 152 * 4, 256, s, vox_bits, vox_words, &st->tr_u_voxels);
   return 3;
 }
 
 // ----------------------------------------------------------------- repair
 __global__ void k_repair_alloc(GridDev g, const uint32_t* vq, const uint32_t* vq_cnt,
                                const uint32_t* pq_cnt, uint32_t vq_cap) {
+  dependency_wait();
   const uint32_t nq = min(*vq_cnt, vq_cap);
   if (blockIdx.x == 0 && threadIdx.x == 0 && nq) {
     atomicAdd(&g.st->repair_rounds, 1u);
@@ -1246,6 +1250,7 @@ __global__ void k_repair_alloc(GridDev g, const uint32_t* vq, const uint32_t* vq
 
 __global__ void k_repair_clear(GridDev g, uint32_t* need, const uint32_t* vq, const uint32_t* vq_cnt,
                                uint32_t vq_cap, int next) {
+  dependency_wait();
   const uint32_t nq = min(*vq_cnt, vq_cap);
   for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < nq; q += gridDim.x * blockDim.x) {
     const uint32_t idx = vq[q];
@@ -1259,13 +1264,13 @@ __global__ void k_repair_clear(GridDev g, uint32_t* need, const uint32_t* vq, co
 
 int launch_repair_alloc(const GridDev& g, const uint32_t* vq, const uint32_t* vq_cnt,
                         const uint32_t* pq_cnt, uint32_t vq_cap, cudaStream_t s) {
-  k_repair_alloc<<<152, 256, 0, s>>>(g, vq, vq_cnt, pq_cnt, vq_cap);
+  launch_chained(k_repair_alloc, 152, 256, s, g, vq, vq_cnt, pq_cnt, vq_cap);
   return 1;
 }
 
 int launch_repair_clear(const GridDev& g, uint32_t* need, const uint32_t* vq,
                          const uint32_t* vq_cnt, uint32_t vq_cap, int next, cudaStream_t s) {
-  k_repair_clear<<<152, 256, 0, s>>>(g, need, vq, vq_cnt, vq_cap, next);
+  launch_chained(k_repair_clear, 152, 256, s, g, need, vq, vq_cnt, vq_cap, next);
   return 1;
 }
 

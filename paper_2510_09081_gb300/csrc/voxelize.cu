@@ -320,7 +320,7 @@ __global__ void __launch_bounds__(kPass1Threads, kPass1Blocks) k_pass1(const flo
   const long long base = ((long long)blockIdx.x * kPass1Warps + wid) * segs_per_warp;
   // slots in spatial order (nearby segments in the same and neighbouring
   // warps keep the packed-word atomics within a smaller part of the grid)
-  const long long k = base + lane;
+  const long long k = base + lane + dependency_wait();
   const long long i = lane < segs_per_warp && k < V ? (order ? (long long)__ldg(&order[k]) : k) : V;
   uint32_t count = 0, bits = 0, voxels = 0;
   bool short_walk = true;
@@ -551,6 +551,7 @@ __global__ void __launch_bounds__(kPass1Threads, kPass1Blocks) k_pass1(const flo
 constexpr int kExactThreads = 128;
 __global__ void __launch_bounds__(kExactThreads) k_exact1(const float4* __restrict__ pos,
                                                 const float4* __restrict__ nrm, GridDev g) {
+  dependency_wait();
   const uint32_t cnt = min(g.st->xq_cnt, g.xq_cap);
   const int lane = threadIdx.x & 31;
   unsigned long long F = 0, sq = 0;
@@ -614,7 +615,8 @@ __device__ __forceinline__ bool bit_set(const uint32_t* bits, uint32_t i) {
 // build instead.
 __global__ void __launch_bounds__(256) k_scatter(GridDev g, int mode, const uint32_t* __restrict__ need,
                                                  const uint32_t* __restrict__ pending) {
-  if (mode == 2 && *pending == 0) return;
+  const uint32_t zero = dependency_wait();
+  if (mode == 2 && pending[zero] == 0) return;
   __shared__ unsigned long long s_rec[8][kWarpRecords];
   unsigned long long* cq = reinterpret_cast<unsigned long long*>(g.xq);
   bool copy = false;  // mode 1: copy the culled records (grid-uniform)
@@ -632,7 +634,7 @@ __global__ void __launch_bounds__(256) k_scatter(GridDev g, int mode, const uint
   unsigned long long* srec = s_rec[threadIdx.x >> 5];
   int wcount = 0;  // culled records staged by this warp (mode 1, uniform)
   unsigned long long listed = 0;
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint32_t warp = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) + zero;
   const uint32_t n_warps = (gridDim.x * blockDim.x) >> 5;
   for (unsigned long long e0 = warp * 32ull; e0 < cnt; e0 += n_warps * 32ull) {
     const unsigned long long e = e0 + lane;
@@ -693,13 +695,14 @@ __global__ void __launch_bounds__(256) k_scatter(GridDev g, int mode, const uint
 // at 512^3: pass 2 0.71 -> 0.47 ms; where most fragments are listed, four
 // rounds' scattered list stores at once measured slower: bundles 0.90 -> 1.11).
 __global__ void __launch_bounds__(256) k_scatter_culled(GridDev g) {
+  const uint32_t zero = dependency_wait();
   const unsigned long long F = g.st->F;
   if (2 * (F - g.st->list_tail) < F) return;  // k_scatter's build
   if (blockIdx.x == 0 && threadIdx.x == 0) g.st->cq_cnt = kNoCopy;
   const unsigned long long cnt = min(g.st->rec_cnt, (unsigned long long)g.rec_cap);
   constexpr int U = 4;
   const int lane = threadIdx.x & 31;
-  const uint32_t warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
+  const uint32_t warp = ((blockIdx.x * blockDim.x + threadIdx.x) >> 5) + zero;
   const uint32_t n_warps = (gridDim.x * blockDim.x) >> 5;
   unsigned long long listed = 0;
   for (unsigned long long e0 = warp * (32ull * U); e0 < cnt; e0 += n_warps * (32ull * U)) {
@@ -741,15 +744,16 @@ int launch_pass1(const float4* pos, const float4* nrm, const uint32_t* order, lo
   // paid there while they returned nothing, 7.8 -> 7.4 ms).
   const int spw = pass1_segments_per_warp(V);
   const long long per_block = (long long)spw * kPass1Warps;
-  k_pass1<<<(unsigned)((V + per_block - 1) / per_block), kPass1Threads, 0, s>>>(pos, nrm, order, V, spw, g);
-  k_exact1<<<152 * 2, kExactThreads, 0, s>>>(pos, nrm, g);
+  launch_chained(k_pass1, (unsigned)((V + per_block - 1) / per_block), kPass1Threads, s, pos, nrm, order, V,
+                 spw, g);
+  launch_chained(k_exact1, 152 * 2, kExactThreads, s, pos, nrm, g);
   return 2;
 }
 
 int launch_scatter(const GridDev& g, int mode, const uint32_t* need, const uint32_t* pending,
                    cudaStream_t s) {
-  if (mode == 1) k_scatter_culled<<<152 * 8, 256, 0, s>>>(g);
-  k_scatter<<<152 * 8, 256, 0, s>>>(g, mode, need, pending);
+  if (mode == 1) launch_chained(k_scatter_culled, 152 * 8, 256, s, g);
+  launch_chained(k_scatter, 152 * 8, 256, s, g, mode, need, pending);
   return mode == 1 ? 2 : 1;
 }
 

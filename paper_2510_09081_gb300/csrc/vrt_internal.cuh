@@ -41,7 +41,7 @@ constexpr uint32_t kCulledStart = 0xC0000000u;
 
 struct DevStatus {
   unsigned int err;
-  unsigned int occupied_voxels;
+  unsigned int pad0;
   unsigned long long F;              // fragments of pass 1
   unsigned long long sum_q;          // occupancy codes of pass 1
   unsigned long long exact_decisions;  // list decisions on the exact path
@@ -53,11 +53,16 @@ struct DevStatus {
   unsigned int xq_cnt;               // undecided (segment, voxel) pairs of pass 1
   unsigned int cq_cnt;               // records of unlisted voxels pass 2 copied to xq
   unsigned int list_tail;            // next free list entry (scan total + repairs)
+  unsigned int occupied_voxels;
   unsigned int visible_voxels;
   unsigned int max_count;
   unsigned int scan_tile_counter;
+  unsigned int scan_tiles_done;
+  // --- reset by every trace
   unsigned int vq_cnt[2];            // culled voxels a ray needed (ping-pong per round)
   unsigned int pq_cnt[2];            // pixels to trace again (ping-pong per round)
+  unsigned int tr_next[kMaxRepairRounds + 1];  // work items handed out per trace launch
+  // ---
   unsigned int repaired_voxels;
   unsigned int repair_rounds;
   unsigned int retraced_pixels;
@@ -67,8 +72,6 @@ struct DevStatus {
   unsigned long long tr_capsule;     // entries past the line-distance test
   unsigned long long tr_voxels;      // voxel lists processed
   unsigned long long tr_steps;       // DDA steps (voxels and empty bricks)
-  unsigned int tr_next[kMaxRepairRounds + 1];  // work items handed out per trace launch
-  unsigned int tr_pad;
   unsigned long long tr_ww_voxels;   // voxel lists taken by the whole-warp path
   unsigned long long tr_ww_entries;  // entries it examined (rescans included)
   unsigned long long tr_hits;        // accepted hits (keys a ray received)
@@ -119,6 +122,18 @@ struct GridDev {
   uint32_t rec_cap;
   DevStatus* st;
 };
+
+// Waits for the kernels before this one on the stream and their writes, then lets
+// the next one's blocks take the places this one's leave. Returns 0: read-only
+// loads, which a memory clobber need not hold back, take their index through it.
+__device__ __forceinline__ uint32_t dependency_wait() {
+  uint32_t zero;
+  asm volatile("griddepcontrol.wait;\n\tgriddepcontrol.launch_dependents;\n\tmov.u32 %0, 0;"
+               : "=r"(zero)
+               :
+               : "memory");
+  return zero;
+}
 
 __device__ __forceinline__ void set_err(DevStatus* st, uint32_t bit) { atomicOr(&st->err, bit); }
 
