@@ -6,10 +6,9 @@
 // published prefix. Every wait is bounded; a wait that gives up sets the
 // timeout bit and the tile carries on with the sum it has.
 //
-// The same pass checks the packed words: the sums of the count and occupancy
-// fields over all voxels must equal the fragment and occupancy totals that
-// pass 1 accumulated separately, otherwise a 16-bit field overflowed. It also
-// marks bricks that hold an occupied voxel (for empty-space skipping).
+// The same pass sums the count and occupancy fields over all voxels, which pass 2
+// compares with the fragment and occupancy totals that pass 1 accumulated
+// separately: a difference means that a 16-bit field overflowed.
 #include "launch.h"
 
 namespace vrt {
@@ -166,13 +165,6 @@ __global__ void __launch_bounds__(kScanThreads) k_scan(GridDev g, int all_visibl
     if (a2 & 0xffffffffull) atomicAdd(&g.st->occupied_voxels, (uint32_t)(a2 & 0xffffffffull));
     if (a2 >> 32) atomicAdd(&g.st->visible_voxels, (uint32_t)(a2 >> 32));
     atomicMax(&g.st->max_count, (uint32_t)a3);
-    // the last tile to add its sums checks them
-    __threadfence();
-    if (atomicAdd(&g.st->scan_tiles_done, 1u) == n_tiles - 1) {
-      __threadfence();
-      const volatile DevStatus* st = g.st;
-      if (st->sum_count_field != st->F || st->sum_occ_field != st->sum_q) set_err(g.st, kErrOverflow);
-    }
   }
 }
 

@@ -617,6 +617,12 @@ __global__ void __launch_bounds__(256) k_scatter(GridDev g, int mode, const uint
                                                  const uint32_t* __restrict__ pending) {
   const uint32_t zero = dependency_wait();
   if (mode == 2 && pending[zero] == 0) return;
+  if (mode != 2 && blockIdx.x == 0 && threadIdx.x == 0) {
+    // the packed words' field sums (the scan's) against pass 1's totals: a
+    // difference means that a 16-bit field overflowed
+    const DevStatus* st = g.st;
+    if (st->sum_count_field != st->F || st->sum_occ_field != st->sum_q) set_err(g.st, kErrOverflow);
+  }
   __shared__ unsigned long long s_rec[8][kWarpRecords];
   unsigned long long* cq = reinterpret_cast<unsigned long long*>(g.xq);
   bool copy = false;  // mode 1: copy the culled records (grid-uniform)

@@ -57,7 +57,7 @@ struct DevStatus {
   unsigned int visible_voxels;
   unsigned int max_count;
   unsigned int scan_tile_counter;
-  unsigned int scan_tiles_done;
+  unsigned int pad1;
   // --- reset by every trace
   unsigned int vq_cnt[2];            // culled voxels a ray needed (ping-pong per round)
   unsigned int pq_cnt[2];            // pixels to trace again (ping-pong per round)
