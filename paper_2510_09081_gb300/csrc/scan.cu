@@ -111,11 +111,11 @@ __global__ void __launch_bounds__(kTileThreads, 8) k_scan(GridDev g, int all_vis
       a0 += s_red[0][q]; a1 += s_red[1][q]; a2 += s_red[2][q];
       a3 = max(a3, s_red[3][q]);
     }
-    if (a0) atomicAdd(&g.st->sum_count_field, (unsigned long long)a0);
-    if (a1) atomicAdd(&g.st->sum_occ_field, (unsigned long long)a1);
-    if (a2 & 0xffffu) atomicAdd(&g.st->occupied_voxels, a2 & 0xffffu);
-    if (a2 >> 16) atomicAdd(&g.st->visible_voxels, a2 >> 16);
-    if (a3) atomicMax(&g.st->max_count, a3);
+    ScanPart& p = g.st->scan_part[tile % kScanParts];
+    if (a0) atomicAdd(&p.count_field, (unsigned long long)a0);
+    if (a1) atomicAdd(&p.occ_field, (unsigned long long)a1);
+    if (a2) atomicAdd(&p.voxels, (unsigned long long)(a2 >> 16) << 32 | (a2 & 0xffffu));
+    if (a3) atomicMax(&p.max_count, a3);
   }
 }
 

@@ -617,11 +617,28 @@ __global__ void __launch_bounds__(256) k_scatter(GridDev g, int mode, const uint
                                                  const uint32_t* __restrict__ pending) {
   const uint32_t zero = dependency_wait();
   if (mode == 2 && pending[zero] == 0) return;
-  if (mode != 2 && blockIdx.x == 0 && threadIdx.x == 0) {
-    // the packed words' field sums (the scan's) against pass 1's totals: a
-    // difference means that a 16-bit field overflowed
-    const DevStatus* st = g.st;
-    if (st->sum_count_field != st->F || st->sum_occ_field != st->sum_q) set_err(g.st, kErrOverflow);
+  if (mode != 2 && blockIdx.x == 0 && threadIdx.x < kScanParts) {
+    // the scan's counters, and its field sums of the packed words against pass 1's
+    // totals: a difference means that a 16-bit field overflowed
+    DevStatus* st = g.st;
+    const ScanPart p = st->scan_part[threadIdx.x + zero];
+    unsigned long long c = p.count_field, o = p.occ_field, v = p.voxels;
+    uint32_t mc = p.max_count;
+#pragma unroll
+    for (int k = kScanParts / 2; k > 0; k >>= 1) {
+      c += __shfl_xor_sync((1u << kScanParts) - 1u, c, k);
+      o += __shfl_xor_sync((1u << kScanParts) - 1u, o, k);
+      v += __shfl_xor_sync((1u << kScanParts) - 1u, v, k);
+      mc = max(mc, __shfl_xor_sync((1u << kScanParts) - 1u, mc, k));
+    }
+    if (threadIdx.x == 0) {
+      st->sum_count_field = c;
+      st->sum_occ_field = o;
+      st->occupied_voxels = (uint32_t)v;
+      st->visible_voxels = (uint32_t)(v >> 32);
+      st->max_count = mc;
+      if (c != st->F || o != st->sum_q) set_err(st, kErrOverflow);
+    }
   }
   __shared__ unsigned long long s_rec[8][kWarpRecords];
   unsigned long long* cq = reinterpret_cast<unsigned long long*>(g.xq);

@@ -39,6 +39,17 @@ constexpr uint32_t kErrRepair = 16u;    // repair rounds exhausted
 // capacities stay below it, so a cursor at or above it marks such a voxel.
 constexpr uint32_t kCulledStart = 0xC0000000u;
 
+// Counters of the scan's tiles, on lines of their own and summed by pass 2. On one
+// line, an atomic takes 1.4 ns whatever its address there, and the tickets that the
+// tiles wait for stood in the same queue (512^3 voxels with every tile occupied,
+// five atomics a tile: 0.297 ms; on these lines 0.199).
+constexpr int kScanParts = 16;
+struct alignas(128) ScanPart {
+  unsigned long long count_field, occ_field;
+  unsigned long long voxels;         // occupied, visible << 32
+  unsigned int max_count;
+};
+
 struct DevStatus {
   unsigned int err;
   unsigned int pad0;
@@ -47,8 +58,8 @@ struct DevStatus {
   unsigned long long exact_decisions;  // list decisions on the exact path
   unsigned long long rec_cnt;        // record slots taken by pass 1 and its exact path
   // --- reset by every list build from here on
-  unsigned long long sum_count_field;  // checked by the scan
-  unsigned long long sum_occ_field;
+  unsigned long long sum_count_field;  // these, the voxel counts and max_count: pass 2's sums
+  unsigned long long sum_occ_field;    // of scan_part[], checked against pass 1's
   unsigned long long listed;         // entries written by pass 2 and repairs
   unsigned int xq_cnt;               // undecided (segment, voxel) pairs of pass 1
   unsigned int cq_cnt;               // records of unlisted voxels pass 2 copied to xq
@@ -80,6 +91,7 @@ struct DevStatus {
   // distinct list entries, vertices and voxel words the rays of the last
   // instrumented trace read (its repair rounds included)
   unsigned long long tr_u_entries, tr_u_vertices, tr_u_voxels;
+  ScanPart scan_part[kScanParts];        // reset by every list build
 };
 
 // -------------------------------------------------------------- grid layout
