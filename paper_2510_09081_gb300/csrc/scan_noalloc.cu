@@ -17,6 +17,8 @@
 // and reported. The scratch is cleared by a kernel that this one is chained to.
 // 256^3 voxels, call after call: 43.7 us with two memsets and 16 consecutive words
 // to a thread, 31.2 now (136 MB, 4.4 TB/s).
+#include <cooperative_groups.h>
+
 #include <atomic>
 #include <mutex>
 #include <string>
@@ -29,6 +31,11 @@ namespace vrt {
 namespace {
 
 constexpr uint32_t kNaMaxTiles = 32768;          // 134,217,728 voxels (512^3)
+// Calls of up to this many tiles (a 32^3 grid) run as one cluster, the largest that
+// needs no opt-in: one launch instead of two. Call after call from the host 10.8 ->
+// 8.9 us, as nodes of a graph 3.2 -> 2.9 us (with two memsets and a kernel 11.3 and
+// 8.2 us).
+constexpr uint32_t kClusterTiles = 8;
 constexpr int kNaSpinLimit = 1 << 22;
 // status bits of status_out
 constexpr uint32_t kNaGaveUp = 1u, kNaWrapped = 2u;
@@ -40,22 +47,31 @@ struct NoAllocScratch {
 };
 static __device__ __align__(256) NoAllocScratch g_noalloc_scratch;
 
+// CLUSTER: the blocks are one cluster, which swaps its sums over distributed shared
+// memory: no scratch, so no kernel to clear it, no ticket and no look-back. Blocks
+// past the last tile (the cluster's size is a power of two) only keep the barriers.
+template <bool CLUSTER>
 __global__ void __launch_bounds__(kTileThreads, 6) k_scan_noalloc(
     NoAllocScratch* scratch, const uint32_t* __restrict__ words, const uint32_t* __restrict__ marks,
     uint32_t* __restrict__ offsets, uint32_t* total_out, uint32_t* status_out, uint32_t n_tiles,
     int stall_tile, int spin_limit) {
   __shared__ uint32_t s_tile;
-  __shared__ uint32_t s_prefix;
+  __shared__ uint32_t s_prefix, s_sum;
   __shared__ uint32_t s_warp[kTileWarps];
   dependency_wait();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-  if (tid == 0) s_tile = atomicAdd(&scratch->tile_counter, 1u);
-  __syncthreads();
-  const uint32_t tile = s_tile;
+  if (!CLUSTER) {
+    if (tid == 0) s_tile = atomicAdd(&scratch->tile_counter, 1u);
+    __syncthreads();
+  }
+  const uint32_t tile = CLUSTER ? blockIdx.x : s_tile;
+  const bool some = !CLUSTER || tile < n_tiles;
   uint2 cnt[kTileRows];
   uint32_t sum[kTileRows], excl[kTileRows];
 #pragma unroll
   for (int q = 0; q < kTileRows; ++q) {
+    cnt[q] = make_uint2(0u, 0u);
+    if (!some) continue;
     const uint32_t i = tile_word(tile, q);
     const uint32_t bits = marks ? marks[i >> 5] >> (i & 31) : 0xfu;
     cnt[q] = masked(pack_counts(*reinterpret_cast<const uint4*>(words + i)), bits);
@@ -71,10 +87,21 @@ __global__ void __launch_bounds__(kTileThreads, 6) k_scan_noalloc(
     if (q < warp) warp_off += s_warp[q];
     agg += s_warp[q];
   }
+  uint32_t cluster_before = 0;  // below 2^31
+  if (CLUSTER) {
+    auto cluster = cooperative_groups::this_cluster();
+    if (tid == 0) s_sum = agg;
+    cluster.sync();
+    if (warp == 0)
+      cluster_before = __reduce_add_sync(
+          0xffffffffu, (uint32_t)lane < tile ? *cluster.map_shared_rank(&s_sum, (unsigned)lane) : 0u);
+    cluster.sync();  // no block leaves while its sum is being read
+  }
   if (warp == 0) {
-    bool gave_up;
+    bool gave_up = false;
     const unsigned long long before =
-        look_back(scratch->state, tile, agg, (int)tile != stall_tile, spin_limit, &gave_up);
+        CLUSTER ? cluster_before
+                : look_back(scratch->state, tile, agg, (int)tile != stall_tile, spin_limit, &gave_up);
     if (lane == 0) {
       if (gave_up && status_out) atomicOr(status_out, kNaGaveUp);
       s_prefix = (uint32_t)before;
@@ -86,6 +113,7 @@ __global__ void __launch_bounds__(kTileThreads, 6) k_scan_noalloc(
     }
   }
   __syncthreads();
+  if (!some) return;
   // offsets are the low 32 bits of the prefix sums (they wrap past 2^32 - 1)
   const uint32_t run = s_prefix + warp_off;
 #pragma unroll
@@ -148,13 +176,32 @@ extern "C" vrt_status vrt_scan_counts_noalloc(const uint32_t* words, const uint3
   }
   const uint32_t n_tiles = (uint32_t)(n_voxels / kTileWords);
   cudaStream_t s = (cudaStream_t)cuda_stream;
-  // the states of the tiles this call uses and the tile counter start at zero
   NoAllocScratch* sc = (NoAllocScratch*)scratch;
-  launch_reset(reinterpret_cast<uint32_t*>(sc->state), 2 * n_tiles, &sc->tile_counter, 1, s);
   const long long stall = g_stall_tile.load();
-  launch_chained(k_scan_noalloc, n_tiles, kTileThreads, s, sc, words, marks, offsets, total_out,
-                 status_out, n_tiles, stall >= 0 ? (int)stall : -1,
-                 stall >= 0 ? kSpinLimitTest : kNaSpinLimit);
+  if (n_tiles <= kClusterTiles && stall < 0) {
+    unsigned size = 1;
+    while (size < n_tiles) size *= 2;
+    cudaLaunchConfig_t c = {};
+    c.gridDim = dim3(size);
+    c.blockDim = dim3(kTileThreads);
+    c.stream = s;
+    cudaLaunchAttribute at[2] = {};
+    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[0].val.programmaticStreamSerializationAllowed = 1;
+    at[1].id = cudaLaunchAttributeClusterDimension;
+    at[1].val.clusterDim.x = size;
+    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    c.attrs = at;
+    c.numAttrs = 2;
+    cudaLaunchKernelEx(&c, k_scan_noalloc<true>, sc, words, marks, offsets, total_out, status_out,
+                       n_tiles, -1, 0);
+  } else {
+    // the states of the tiles this call uses and the tile counter start at zero
+    launch_reset(reinterpret_cast<uint32_t*>(sc->state), 2 * n_tiles, &sc->tile_counter, 1, s);
+    launch_chained(k_scan_noalloc<false>, n_tiles, kTileThreads, s, sc, words, marks, offsets,
+                   total_out, status_out, n_tiles, stall >= 0 ? (int)stall : -1,
+                   stall >= 0 ? kSpinLimitTest : kNaSpinLimit);
+  }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(VRT_ERR_CUDA, cudaGetErrorString(e));
   return VRT_OK;

@@ -1,6 +1,6 @@
 """The list-offset scan's tiles: every position in a tile, marks in every nibble,
-full 16-bit counts beside non-zero upper halves, and more tiles than one
-look-back window or one set of resident blocks."""
+full 16-bit counts beside non-zero upper halves, the sizes at and beside a full
+cluster, and more tiles than one look-back window or one set of resident blocks."""
 import numpy as np
 import pytest
 
@@ -11,7 +11,7 @@ pytestmark = pytest.mark.gpu
 torch = pytest.importorskip("torch")
 
 
-@pytest.mark.parametrize("n_tiles", [1, 2, 33, 1301])
+@pytest.mark.parametrize("n_tiles", [1, 2, 3, 8, 9, 33, 1301])
 @pytest.mark.parametrize("marked", ["all", "random", "one per tile", "none"])
 def test_offsets_equal_the_prefix_sum(n_tiles, marked):
     n = 4096 * n_tiles
