@@ -397,11 +397,12 @@ vrt_status vrt_get_stage_ms(vrt_grid g, float* ms, int32_t n);
  * orders voxels in 4^3 bricks (brick index x-fastest, then 16 z + 4 y + x
  * inside the brick); pass words in that order to reproduce its offsets.
  * The call issues two kernels on `cuda_stream` (one clears its scratch, one
- * scans; up to 32768 voxels one kernel that needs no scratch); it calls no cudaMalloc, cudaFree or allocating library
- * routine. Every call shares the scratch array and leaves its contents
- * behind; calls that overlap on the GPU (two streams, two threads) race and
- * give wrong results. The first call on a device looks up the array's device
- * address (cudaGetSymbolAddress) with that device current; make that first
+ * scans; up to 32768 voxels one kernel that needs no scratch); it calls no
+ * cudaMalloc, cudaFree or allocating library routine. Every call shares the
+ * scratch array and leaves its contents behind; calls that overlap on the GPU
+ * (two streams, two threads) race and give wrong results. The first call on a
+ * device looks up the array's device address (cudaGetSymbolAddress) with that
+ * device current; make that first
  * call before any stream capture. Errors: VRT_ERR_INVALID_ARG, VRT_ERR_CUDA;
  * vrt_last_error(NULL) gives the message. */
 vrt_status vrt_scan_counts_noalloc(const uint32_t* words, const uint32_t* marks, uint32_t* offsets,
