@@ -7,6 +7,8 @@
 #include <cstddef>
 #include <cstdio>
 #include <cstring>
+#include <map>
+#include <mutex>
 #include <new>
 #include <string>
 #include <unordered_map>
@@ -24,6 +26,7 @@ struct vrt_grid_s {
   int occ_scale = 32;
   uint64_t max_frag_desc = 0;
   cudaStream_t stream = nullptr;
+  cudaStream_t entered = nullptr;  // the stream counted for this grid (stream_enter)
   // vertices
   long long V = 0, P = 0, V_alloc = 0;
   // vertices uploaded or updated since the last ingest, with their polyline
@@ -110,6 +113,27 @@ struct vrt_grid_s {
 // host thread, so failing calls on different threads do not race on it.
 thread_local std::string g_create_error;
 
+namespace vrt {
+namespace {
+std::mutex g_streams_mu;
+std::map<cudaStream_t, long long> g_streams;  // grids on each stream
+}  // namespace
+
+void stream_enter(cudaStream_t s) {
+  std::lock_guard<std::mutex> lk(g_streams_mu);
+  ++g_streams[s];
+}
+void stream_leave(cudaStream_t s) {
+  std::lock_guard<std::mutex> lk(g_streams_mu);
+  const auto it = g_streams.find(s);
+  if (it != g_streams.end() && --it->second == 0) g_streams.erase(it);
+}
+bool stream_alone(cudaStream_t s) {
+  std::lock_guard<std::mutex> lk(g_streams_mu);
+  return g_streams.empty() || (g_streams.size() == 1 && g_streams.begin()->first == s);
+}
+}  // namespace vrt
+
 namespace {
 
 vrt_status fail(vrt_grid g, vrt_status s, const std::string& msg) {
@@ -127,6 +151,8 @@ vrt_status cuda_fail(vrt_grid g, cudaError_t e, const char* what) {
     cudaError_t e_ = (call);                           \
     if (e_ != cudaSuccess) return cuda_fail(g, e_, #call); \
   } while (0)
+
+Queue queue(vrt_grid g) { return {g->stream, stream_alone(g->entered)}; }
 
 // Device allocations of a grid, counted in g->dev_bytes.
 template <class T>
@@ -495,6 +521,8 @@ vrt_status vrt_create_grid(const vrt_grid_desc* desc, void* cuda_stream, vrt_gri
     delete g;
     return s;
   }
+  g->entered = g->stream;
+  stream_enter(g->entered);
   // pyramid offsets
   long long off = 0, m = n;
   g->n_levels = 0;
@@ -651,12 +679,12 @@ vrt_status vrt_voxelize(vrt_grid g) {
   stage_mark(g, ST_INGEST, 0);
   // the vertices that changed since the last ingest (all of them after an upload)
   g->launches += launch_ingest(g->raw, g->flags, g->dirty_lo, g->dirty_hi, g->pos, g->nrm, g->st,
-                               g->stream);
+                               queue(g));
   g->dirty_lo = g->dirty_hi = 0;
   stage_mark(g, ST_INGEST, 1);
   stage_mark(g, ST_PASS1, 0);
-  g->launches += launch_pass1(g->pos, g->nrm, g->order, g->V, gdev(g), g->stream);
-  g->launches += launch_brick_dist(gdev(g), g->btmp, g->bdist, g->bmask, g->stream);
+  g->launches += launch_pass1(g->pos, g->nrm, g->order, g->V, gdev(g), queue(g));
+  g->launches += launch_brick_dist(gdev(g), g->btmp, g->bdist, g->bmask, queue(g));
   stage_mark(g, ST_PASS1, 1);
   VRT_CUDA(g, cudaGetLastError());
   g->stage = 2;
@@ -669,7 +697,7 @@ vrt_status vrt_build_mips(vrt_grid g) {
   if (g->stage < 2) return fail(g, VRT_ERR_STATE, "vrt_voxelize first");
   if (!g->mips) VRT_CUDA(g, dalloc(g, (float**)&g->mips, (size_t)(g->lev_off[g->n_levels - 1] + 1)));
   stage_mark(g, ST_MIPS, 0);
-  g->launches += launch_mips(gdev(g), g->mips, g->mips_fmt, g->lev_off, g->n_levels, g->stream);
+  g->launches += launch_mips(gdev(g), g->mips, g->mips_fmt, g->lev_off, g->n_levels, queue(g));
   ++g->mips_id;
   stage_mark(g, ST_MIPS, 1);
   VRT_CUDA(g, cudaGetLastError());
@@ -698,7 +726,7 @@ vrt_status vrt_cull(vrt_grid g, const vrt_camera* cam, const vrt_render_params* 
   // reset the list-build counters (scan tile counter .. end)
   const size_t off = offsetof(DevStatus, sum_count_field);
   g->launches += launch_reset((uint32_t*)((char*)g->st + off), (uint32_t)((sizeof(DevStatus) - off) / 4),
-                              (uint32_t*)g->tile_state, 2 * g->n_tiles, g->stream);
+                              (uint32_t*)g->tile_state, 2 * g->n_tiles, queue(g));
   stage_mark(g, ST_CULL, 0);
   if (cull) {
     if (!g->eroded) VRT_CUDA(g, dalloc(g, &g->eroded, nv));
@@ -708,17 +736,17 @@ vrt_status vrt_cull(vrt_grid g, const vrt_camera* cam, const vrt_render_params* 
     // the cull keeps its queue of occupied voxels there
     g->launches += launch_cull(d, host_cam(cam), p->alpha, g->eroded, g->btmp, g->cdist, g->emean,
                                g->cull_depth, reinterpret_cast<uint32_t*>(g->xq),
-                               2ull * g->xq_cap, g->stream);
+                               2ull * g->xq_cap, queue(g));
   } else {
     VRT_CUDA(g, cudaMemsetAsync(g->vis, 0xff, nv / 8, g->stream));
   }
   stage_mark(g, ST_CULL, 1);
   stage_mark(g, ST_SCAN, 0);
   g->launches += launch_scan(d, cull ? 0 : 1, g->tile_state, g->n_tiles, g->scan_stall,
-                             g->scan_stall >= 0 ? kSpinLimitTest : 0, g->stream);
+                             g->scan_stall >= 0 ? kSpinLimitTest : 0, queue(g));
   stage_mark(g, ST_SCAN, 1);
   stage_mark(g, ST_PASS2, 0);
-  g->launches += launch_scatter(d, cull ? 1 : 0, nullptr, nullptr, g->stream);
+  g->launches += launch_scatter(d, cull ? 1 : 0, nullptr, nullptr, queue(g));
   stage_mark(g, ST_PASS2, 1);
   VRT_CUDA(g, cudaGetLastError());
   g->culled = cull ? 1 : 0;
@@ -789,7 +817,7 @@ vrt_status vrt_trace(vrt_grid g, const vrt_camera* cam, const vrt_render_params*
                              ((uint64_t)lb[2] << 32) | (uint64_t)sa.ao};
     if (std::memcmp(key, g->shade_key, sizeof(key)) != 0) {
       stage_mark(g, ST_SHADE, 0);
-      g->launches += launch_shade(sa, g->stream);
+      g->launches += launch_shade(sa, queue(g));
       stage_mark(g, ST_SHADE, 1);
       std::memcpy(g->shade_key, key, sizeof(key));
     }
@@ -838,7 +866,7 @@ vrt_status vrt_trace(vrt_grid g, const vrt_camera* cam, const vrt_render_params*
     a.touch_vox = g->touch_vox;
   }
   stage_mark(g, ST_TRACE, 0);
-  g->launches += launch_trace(a, K, g->stream);
+  g->launches += launch_trace(a, K, queue(g));
   stage_mark(g, ST_TRACE, 1);
   if (g->culled) {
     stage_mark(g, ST_REPAIR, 0);
@@ -846,16 +874,16 @@ vrt_status vrt_trace(vrt_grid g, const vrt_camera* cam, const vrt_render_params*
     for (int r = 0; r < kMaxRepairRounds; ++r) {
       const int ci = r & 1, nx = ci ^ 1;
       g->launches += launch_repair_alloc(d, g->vq[ci], &g->st->vq_cnt[ci], &g->st->pq_cnt[ci],
-                                         g->vq_cap, g->stream);
+                                         g->vq_cap, queue(g));
       if (p->voxel_shading) {
         ShadeArgs sr = sa;
         sr.vq = g->vq[ci];
         sr.vq_cnt = &g->st->vq_cnt[ci];
         sr.vq_cap = g->vq_cap;
-        g->launches += launch_shade_repair(sr, g->stream);
+        g->launches += launch_shade_repair(sr, queue(g));
       }
-      g->launches += launch_scatter(d, 2, g->need, &g->st->vq_cnt[ci], g->stream);
-      g->launches += launch_repair_clear(d, g->need, g->vq[ci], &g->st->vq_cnt[ci], g->vq_cap, nx, g->stream);
+      g->launches += launch_scatter(d, 2, g->need, &g->st->vq_cnt[ci], queue(g));
+      g->launches += launch_repair_clear(d, g->need, g->vq[ci], &g->st->vq_cnt[ci], g->vq_cap, nx, queue(g));
       TraceArgs b = a;
       b.pix_list = g->pq[ci];
       b.pix_count = &g->st->pq_cnt[ci];
@@ -863,20 +891,20 @@ vrt_status vrt_trace(vrt_grid g, const vrt_camera* cam, const vrt_render_params*
       b.pq = g->pq[nx]; b.pq_cnt = &g->st->pq_cnt[nx];
       b.max_queue = (r + 2 >= kMaxRepairRounds) ? 0xffffffffu : kRayQueueLimit;
       b.work_next = &g->st->tr_next[r + 1];
-      g->launches += launch_trace(b, K, g->stream);
+      g->launches += launch_trace(b, K, queue(g));
     }
     stage_mark(g, ST_REPAIR, 1);
   }
   if (K == 1 && a.ao == 1) {
     stage_mark(g, ST_SHADE, 0);
-    g->launches += launch_shade_hits(a, g->stream);
+    g->launches += launch_shade_hits(a, queue(g));
     stage_mark(g, ST_SHADE, 1);
   }
   if (g->trace_counters) {
     VRT_CUDA(g, cudaMemsetAsync((char*)g->st + offsetof(DevStatus, tr_u_entries), 0,
                                 3 * sizeof(unsigned long long), g->stream));
     g->launches += launch_touch_count(g->touch_list, g->touch_list_words, g->touch_vert,
-                                      g->touch_vert_words, g->touch_vox, nv / 32, g->st, g->stream);
+                                      g->touch_vert_words, g->touch_vox, nv / 32, g->st, queue(g));
   }
   VRT_CUDA(g, cudaGetLastError());
   return VRT_OK;
@@ -1215,6 +1243,11 @@ vrt_status vrt_grid_device_bytes(vrt_grid g, uint64_t* bytes) {
 vrt_status vrt_set_stream(vrt_grid g, void* cuda_stream) {
   if (!g) return fail(nullptr, VRT_ERR_INVALID_ARG, "grid is NULL");
   g->stream = (cudaStream_t)cuda_stream;
+  if (g->stream != g->entered) {
+    stream_enter(g->stream);
+    stream_leave(g->entered);
+    g->entered = g->stream;
+  }
   return VRT_OK;
 }
 
@@ -1302,6 +1335,7 @@ vrt_status vrt_destroy(vrt_grid g) {
   if (!g) return VRT_OK;
   cudaStreamSynchronize(g->stream);
   free_all(g);
+  stream_leave(g->entered);
   delete g;
   return VRT_OK;
 }

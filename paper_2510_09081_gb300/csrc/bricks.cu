@@ -59,26 +59,26 @@ __global__ void __launch_bounds__(256) k_reset(uint32_t* a, uint32_t na, uint32_
     else b[i - na] = 0u;
 }
 
-int launch_reset(uint32_t* a, uint32_t na, uint32_t* b, uint32_t nb, cudaStream_t s) {
+int launch_reset(uint32_t* a, uint32_t na, uint32_t* b, uint32_t nb, const Queue& q) {
   const unsigned blocks = (na + nb + 1023) / 1024;
-  launch_chained(k_reset, blocks < 152u ? blocks : 152u, 256, s, a, na, b, nb);
+  launch(k_reset, blocks < 152u ? blocks : 152u, 256, q, a, na, b, nb);
   return 1;
 }
 
-int launch_brick_dist_passes(int log2nb, uint8_t* tmp, uint8_t* dist, cudaStream_t s) {
+int launch_brick_dist_passes(int log2nb, uint8_t* tmp, uint8_t* dist, const Queue& q) {
   const uint32_t nb = 1u << (3 * log2nb);
   const int T = 256;
   const unsigned blocks = (nb + T - 1) / T;
-  launch_chained(k_brick_dist, blocks, T, s, log2nb, 0, tmp, dist);
-  launch_chained(k_brick_dist, blocks, T, s, log2nb, 1, dist, tmp);
-  launch_chained(k_brick_dist, blocks, T, s, log2nb, 2, tmp, dist);
+  launch(k_brick_dist, blocks, T, q, log2nb, 0, tmp, dist);
+  launch(k_brick_dist, blocks, T, q, log2nb, 1, dist, tmp);
+  launch(k_brick_dist, blocks, T, q, log2nb, 2, tmp, dist);
   return 3;
 }
 
-int launch_brick_dist(const GridDev& g, uint8_t* tmp, uint8_t* dist, uint2* mask, cudaStream_t s) {
+int launch_brick_dist(const GridDev& g, uint8_t* tmp, uint8_t* dist, uint2* mask, const Queue& q) {
   const int T = 256;
-  launch_chained(k_brick_occ, (1u << (3 * g.log2nb + 4)) / T, T, s, g, tmp, mask);
-  return 1 + launch_brick_dist_passes(g.log2nb, tmp, dist, s);
+  launch(k_brick_occ, (1u << (3 * g.log2nb + 4)) / T, T, q, g, tmp, mask);
+  return 1 + launch_brick_dist_passes(g.log2nb, tmp, dist, q);
 }
 
 }  // namespace vrt

@@ -365,7 +365,7 @@ float3 tof(D3 a) { return make_float3((float)a.x, (float)a.y, (float)a.z); }
 
 int launch_cull(const GridDev& g, const HostCamera& cam, float alpha, uint8_t* eroded,
                 uint8_t* btmp, uint8_t* cdist, float* emean, float depth_max, uint32_t* occq,
-                unsigned long long occq_cap, cudaStream_t s) {
+                unsigned long long occq_cap, const Queue& q) {
   const D3 eye = {cam.eye[0], cam.eye[1], cam.eye[2]};
   const D3 tgt = {cam.target[0], cam.target[1], cam.target[2]};
   const D3 upw = {cam.up[0], cam.up[1], cam.up[2]};
@@ -402,11 +402,11 @@ int launch_cull(const GridDev& g, const HostCamera& cam, float alpha, uint8_t* e
   // enough bricks per warp that rejecting one costs little, but warps enough to
   // fill the GPU
   const int per_warp = g.n >= 512 ? 32 : (g.n >= 256 ? 8 : 2);
-  launch_chained(k_erode, (nvox / 64 / per_warp * 32 + T - 1) / T, T, s, g, cc, per_warp, eroded, btmp, emean,
+  launch(k_erode, (nvox / 64 / per_warp * 32 + T - 1) / T, T, q, g, cc, per_warp, eroded, btmp, emean,
                  queued ? occq : nullptr, occq_cap);
-  const int passes = launch_brick_dist_passes(g.log2nb, btmp, cdist, s);
-  if (queued) launch_chained(k_visible_queued, 152 * 8, T, s, g, cc, eroded, cdist, emean, occq, occq_cap);
-  else launch_chained(k_visible, (nvox + T - 1) / T, T, s, g, cc, eroded, cdist, emean);
+  const int passes = launch_brick_dist_passes(g.log2nb, btmp, cdist, q);
+  if (queued) launch(k_visible_queued, 152 * 8, T, q, g, cc, eroded, cdist, emean, occq, occq_cap);
+  else launch(k_visible, (nvox + T - 1) / T, T, q, g, cc, eroded, cdist, emean);
   return 2 + passes;
 }
 

@@ -44,10 +44,10 @@ __global__ void __launch_bounds__(256) k_ingest(const float* __restrict__ raw,
 }
 
 int launch_ingest(const float* raw, const uint8_t* flags, long long lo, long long hi, float4* pos,
-                  float4* nrm, DevStatus* st, cudaStream_t s) {
+                  float4* nrm, DevStatus* st, const Queue& q) {
   if (hi <= lo) return 0;
   const int T = 256;
-  launch_chained(k_ingest, (unsigned)((hi - lo + T - 1) / T), T, s, raw, flags, lo, hi, pos, nrm, st);
+  launch(k_ingest, (unsigned)((hi - lo + T - 1) / T), T, q, raw, flags, lo, hi, pos, nrm, st);
   return 1;
 }
 

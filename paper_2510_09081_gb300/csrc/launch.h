@@ -9,23 +9,41 @@
 
 namespace vrt {
 
-// Launches `kernel` so that it may start while the kernel before it on the stream
-// drains: its blocks are resident, waiting in dependency_wait(), when that one
-// completes, which saves most of a launch's latency (a frame of a small set is a
-// chain of 11 to 33 kernels of a few microseconds). Every kernel launched this
-// way calls dependency_wait() before it touches memory. After a copy, a memset or
+// Where kernels are launched: a stream, and whether each may start while the one
+// before it drains (launch).
+struct Queue {
+  cudaStream_t s;
+  bool chained;
+};
+
+// The streams of the process's grids and servers. Launches are chained only while
+// there is one: with frames of 128^3 to 512^3 sets on four streams at once, all
+// chained, a run of the serving workload was seen to stop with the GPU busy, and
+// reading showed no reason in the kernels (their waits and loops end), so chained
+// launches and several streams do not meet. A grid enters the stream it takes and
+// leaves it for the next; a server enters all of its streams while it lives.
+void stream_enter(cudaStream_t s);
+void stream_leave(cudaStream_t s);
+// Whether no other stream than s is entered.
+bool stream_alone(cudaStream_t s);
+
+// Launches `kernel`; chained, so that it may start while the kernel before it on
+// the stream drains: its blocks are resident, waiting in dependency_wait(), when that
+// one completes, which saves most of a launch's latency (a frame of a small set is a
+// chain of 11 to 33 kernels of a few microseconds). Every kernel launched here
+// calls dependency_wait() before it touches memory. After a copy, a memset or
 // an event the stream orders it as usual.
 template <class... P, class... A>
-void launch_chained(void (*kernel)(P...), dim3 grid, unsigned threads, cudaStream_t s, A... args) {
+void launch(void (*kernel)(P...), dim3 grid, unsigned threads, const Queue& q, A... args) {
   cudaLaunchConfig_t c = {};
   c.gridDim = grid;
   c.blockDim = dim3(threads);
-  c.stream = s;
+  c.stream = q.s;
   cudaLaunchAttribute at = {};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
   at.val.programmaticStreamSerializationAllowed = 1;
   c.attrs = &at;
-  c.numAttrs = 1;
+  c.numAttrs = q.chained ? 1 : 0;
   cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
@@ -100,15 +118,15 @@ struct ShadeArgs {
   uint32_t vq_cap;
 };
 // Every voxel next to a listed one (one block per brick); rewrites the mask.
-int launch_shade(const ShadeArgs& a, cudaStream_t s);
+int launch_shade(const ShadeArgs& a, const Queue& q);
 // Zeroes up to two ranges of 32-bit words.
-int launch_reset(uint32_t* a, uint32_t na, uint32_t* b, uint32_t nb, cudaStream_t s);
+int launch_reset(uint32_t* a, uint32_t na, uint32_t* b, uint32_t nb, const Queue& q);
 // Voxels next to the voxels a repair round listed, not yet shaded this frame.
-int launch_shade_repair(const ShadeArgs& a, cudaStream_t s);
+int launch_shade_repair(const ShadeArgs& a, const Queue& q);
 
 // Ingest of vertices [lo, hi) (nothing when hi <= lo).
 int launch_ingest(const float* raw, const uint8_t* flags, long long lo, long long hi, float4* pos,
-                  float4* nrm, DevStatus* st, cudaStream_t s);
+                  float4* nrm, DevStatus* st, const Queue& q);
 constexpr int kPass1Threads = 128;
 constexpr int kPass1Blocks = 9;  // resident per SM: 56 registers, 24 KB of shared memory
 // Segments a warp of pass 1 takes, of a set of V vertices. They are a serial chain
@@ -125,27 +143,27 @@ inline int pass1_segments_per_warp(long long V) {
 // polyline's vertices consecutive; a polyline's last vertex starts no
 // segment), or in index order when `order` is null.
 int launch_pass1(const float4* pos, const float4* nrm, const uint32_t* order, long long V,
-                 const GridDev& g, cudaStream_t s);
+                 const GridDev& g, const Queue& q);
 // 12-bit spatial keys (Morton code of the 16^3 cell) of the vertices mid[0..P).
 int launch_poly_keys(const float* raw, const uint32_t* mid, uint32_t P, int n, uint16_t* key,
                      cudaStream_t s);
 // Occupancy masks and empty-brick distance field from the counts of pass 1
 // (tmp: one byte per brick).
-int launch_brick_dist(const GridDev& g, uint8_t* tmp, uint8_t* dist, uint2* mask, cudaStream_t s);
+int launch_brick_dist(const GridDev& g, uint8_t* tmp, uint8_t* dist, uint2* mask, const Queue& q);
 // The three distance passes from per-brick bytes in tmp (0 = occupied, else
 // kBrickDistMax); tmp is overwritten.
-int launch_brick_dist_passes(int log2nb, uint8_t* tmp, uint8_t* dist, cudaStream_t s);
+int launch_brick_dist_passes(int log2nb, uint8_t* tmp, uint8_t* dist, const Queue& q);
 // Pass 2 over the fragment records. mode 0: every occupied voxel has a list;
 // 1: voxels marked by the cull; 2: repair, only voxels whose `need` bit is set
 // (skipped when *pending is 0).
 int launch_scatter(const GridDev& g, int mode, const uint32_t* need, const uint32_t* pending,
-                   cudaStream_t s);
+                   const Queue& q);
 // stall_tile >= 0 (testing): that tile never publishes its look-back state,
 // so the tiles after it give up their waits after spin_limit polls.
 int launch_scan(const GridDev& g, int all_visible, unsigned long long* tile_state, uint32_t n_tiles,
-                int stall_tile, int spin_limit, cudaStream_t s);
+                int stall_tile, int spin_limit, const Queue& q);
 int launch_mips(const GridDev& g, void* mips, int fmt, const long long* lev_off, int n_levels,
-                cudaStream_t s);
+                const Queue& q);
 // Cull marks; btmp, cdist: one byte per brick (scratch; distance to a brick
 // with eroded occupancy); emean: one float per brick (mean eroded occupancy);
 // depth_max: estimated optical depth past which a voxel is culled (<= 0: the
@@ -153,22 +171,22 @@ int launch_mips(const GridDev& g, void* mips, int fmt, const long long* lev_off,
 // (occq_cap entries; when fewer than n^3, every voxel's thread tests its own).
 int launch_cull(const GridDev& g, const HostCamera& cam, float alpha, uint8_t* eroded,
                 uint8_t* btmp, uint8_t* cdist, float* emean, float depth_max, uint32_t* occq,
-                unsigned long long occq_cap, cudaStream_t s);
-int launch_trace(const TraceArgs& a, int K, cudaStream_t s);
+                unsigned long long occq_cap, const Queue& q);
+int launch_trace(const TraceArgs& a, int K, const Queue& q);
 // Cone AO of the hits an opaque trace (K = 1, a.ao = 1) and its repair rounds
 // left in a.rgba.
-int launch_shade_hits(const TraceArgs& a, cudaStream_t s);
+int launch_shade_hits(const TraceArgs& a, const Queue& q);
 // Instrumented trace: the set bits of the three touch bitmaps into
 // st->tr_u_entries, tr_u_vertices, tr_u_voxels (which the caller cleared).
 int launch_touch_count(const uint32_t* list_bits, size_t list_words, const uint32_t* vert_bits,
                        size_t vert_words, const uint32_t* vox_bits, size_t vox_words,
-                       DevStatus* st, cudaStream_t s);
+                       DevStatus* st, const Queue& q);
 // Repair round: list the voxels of vq (count *vq_cnt), pass 2 restricted to
 // them, then clear their `need` bits and the next round's queue counters.
 int launch_repair_alloc(const GridDev& g, const uint32_t* vq, const uint32_t* vq_cnt,
-                        const uint32_t* pq_cnt, uint32_t vq_cap, cudaStream_t s);
+                        const uint32_t* pq_cnt, uint32_t vq_cap, const Queue& q);
 int launch_repair_clear(const GridDev& g, uint32_t* need, const uint32_t* vq,
-                         const uint32_t* vq_cnt, uint32_t vq_cap, int next, cudaStream_t s);
+                         const uint32_t* vq_cnt, uint32_t vq_cap, int next, const Queue& q);
 
 // Host-side checks shared by the C ABI and the serving loop: nullptr when the
 // camera and render parameters are acceptable to vrt_cull and vrt_trace, else

@@ -80,16 +80,16 @@ __global__ void __launch_bounds__(256) k_mip_down(const T* __restrict__ src, T* 
 }
 
 template <class T>
-int launch_mips_t(const GridDev& g, T* mips, const long long* lev_off, int n_levels, cudaStream_t s) {
+int launch_mips_t(const GridDev& g, T* mips, const long long* lev_off, int n_levels, const Queue& q) {
   const int T_ = 256;
   long long m = g.n >> 1;
   long long cnt = m * m * m / 2;  // threads: 16 voxels each
   int launches = 1;
-  launch_chained(k_mip01<T>, (unsigned)((cnt + T_ - 1) / T_), T_, s, g, mips + lev_off[0], mips + lev_off[1]);
+  launch(k_mip01<T>, (unsigned)((cnt + T_ - 1) / T_), T_, q, g, mips + lev_off[0], mips + lev_off[1]);
   for (int l = 2; l < n_levels; ++l) {
     m = g.n >> l;
     cnt = m * m * m;
-    launch_chained(k_mip_down<T>, (unsigned)((cnt + T_ - 1) / T_), T_, s, mips + lev_off[l - 1],
+    launch(k_mip_down<T>, (unsigned)((cnt + T_ - 1) / T_), T_, q, mips + lev_off[l - 1],
                    mips + lev_off[l], (int)m);
     ++launches;
   }
@@ -97,10 +97,10 @@ int launch_mips_t(const GridDev& g, T* mips, const long long* lev_off, int n_lev
 }
 
 int launch_mips(const GridDev& g, void* mips, int fmt, const long long* lev_off, int n_levels,
-                cudaStream_t s) {
-  if (fmt == kMipsF16) return launch_mips_t(g, (__half*)mips, lev_off, n_levels, s);
-  if (fmt == kMipsBF16) return launch_mips_t(g, (__nv_bfloat16*)mips, lev_off, n_levels, s);
-  return launch_mips_t(g, (float*)mips, lev_off, n_levels, s);
+                const Queue& q) {
+  if (fmt == kMipsF16) return launch_mips_t(g, (__half*)mips, lev_off, n_levels, q);
+  if (fmt == kMipsBF16) return launch_mips_t(g, (__nv_bfloat16*)mips, lev_off, n_levels, q);
+  return launch_mips_t(g, (float*)mips, lev_off, n_levels, q);
 }
 
 }  // namespace vrt

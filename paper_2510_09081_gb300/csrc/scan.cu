@@ -120,8 +120,8 @@ __global__ void __launch_bounds__(kTileThreads, 8) k_scan(GridDev g, int all_vis
 }
 
 int launch_scan(const GridDev& g, int all_visible, unsigned long long* tile_state, uint32_t n_tiles,
-                int stall_tile, int spin_limit, cudaStream_t s) {
-  launch_chained(k_scan, n_tiles, kTileThreads, s, g, all_visible, tile_state, n_tiles, stall_tile,
+                int stall_tile, int spin_limit, const Queue& q) {
+  launch(k_scan, n_tiles, kTileThreads, q, g, all_visible, tile_state, n_tiles, stall_tile,
                  spin_limit > 0 ? spin_limit : kSpinLimit);
   return 1;
 }

@@ -175,7 +175,7 @@ extern "C" vrt_status vrt_scan_counts_noalloc(const uint32_t* words, const uint3
     scratch = g_scratch_addr[dev];
   }
   const uint32_t n_tiles = (uint32_t)(n_voxels / kTileWords);
-  cudaStream_t s = (cudaStream_t)cuda_stream;
+  const Queue q = {(cudaStream_t)cuda_stream, stream_alone((cudaStream_t)cuda_stream)};
   NoAllocScratch* sc = (NoAllocScratch*)scratch;
   const long long stall = g_stall_tile.load();
   if (n_tiles <= kClusterTiles && stall < 0) {
@@ -184,23 +184,22 @@ extern "C" vrt_status vrt_scan_counts_noalloc(const uint32_t* words, const uint3
     cudaLaunchConfig_t c = {};
     c.gridDim = dim3(size);
     c.blockDim = dim3(kTileThreads);
-    c.stream = s;
+    c.stream = q.s;
     cudaLaunchAttribute at[2] = {};
-    at[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at[0].val.programmaticStreamSerializationAllowed = 1;
-    at[1].id = cudaLaunchAttributeClusterDimension;
-    at[1].val.clusterDim.x = size;
-    at[1].val.clusterDim.y = at[1].val.clusterDim.z = 1;
+    at[0].id = cudaLaunchAttributeClusterDimension;
+    at[0].val.clusterDim.x = size;
+    at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     c.attrs = at;
-    c.numAttrs = 2;
+    c.numAttrs = q.chained ? 2 : 1;
     cudaLaunchKernelEx(&c, k_scan_noalloc<true>, sc, words, marks, offsets, total_out, status_out,
                        n_tiles, -1, 0);
   } else {
     // the states of the tiles this call uses and the tile counter start at zero
-    launch_reset(reinterpret_cast<uint32_t*>(sc->state), 2 * n_tiles, &sc->tile_counter, 1, s);
-    launch_chained(k_scan_noalloc<false>, n_tiles, kTileThreads, s, sc, words, marks, offsets,
-                   total_out, status_out, n_tiles, stall >= 0 ? (int)stall : -1,
-                   stall >= 0 ? kSpinLimitTest : kNaSpinLimit);
+    launch_reset(reinterpret_cast<uint32_t*>(sc->state), 2 * n_tiles, &sc->tile_counter, 1, q);
+    launch(k_scan_noalloc<false>, n_tiles, kTileThreads, q, sc, words, marks, offsets, total_out,
+           status_out, n_tiles, stall >= 0 ? (int)stall : -1, stall >= 0 ? kSpinLimitTest : kNaSpinLimit);
   }
   const cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return fail(VRT_ERR_CUDA, cudaGetErrorString(e));

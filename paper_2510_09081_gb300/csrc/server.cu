@@ -553,6 +553,7 @@ vrt_status vrt_server_create(const vrt_server_desc* desc, vrt_server* out) {
     }
     s->slots.push_back(std::move(sl));
   }
+  for (auto& o : s->slots) vrt::stream_enter(o->stream);  // frames overlap: no chained launches
   cudaSetDevice(prev);
   s->th = std::thread(scheduler, s);
   *out = s;
@@ -695,6 +696,7 @@ vrt_status vrt_server_destroy(vrt_server s) {
   for (auto& st : s->sets)
     if (st->grid) vrt_destroy(st->grid);
   for (auto& sl : s->slots) {
+    vrt::stream_leave(sl->stream);
     cudaStreamDestroy(sl->stream);
     for (cudaStream_t b : sl->branch) cudaStreamDestroy(b);
     for (cudaEvent_t e : sl->join) cudaEventDestroy(e);

@@ -142,14 +142,14 @@ __global__ void k_shade_repair(ShadeArgs A) {
 
 }  // namespace
 
-int launch_shade(const ShadeArgs& a, cudaStream_t s) {
+int launch_shade(const ShadeArgs& a, const Queue& q) {
   const unsigned n_bricks = 1u << (3 * a.g.log2nb);
-  launch_chained(k_shade, n_bricks, 64, s, a);
+  launch(k_shade, n_bricks, 64, q, a);
   return 1;
 }
 
-int launch_shade_repair(const ShadeArgs& a, cudaStream_t s) {
-  launch_chained(k_shade_repair, 152, 256, s, a);
+int launch_shade_repair(const ShadeArgs& a, const Queue& q) {
+  launch(k_shade_repair, 152, 256, q, a);
   return 1;
 }
 

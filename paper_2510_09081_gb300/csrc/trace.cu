@@ -1134,9 +1134,9 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks<OPAQUE, COUNT, AO>) 
 }
 
 template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
-void launch_one(const TraceArgs& a, cudaStream_t s) {
+void launch_one(const TraceArgs& a, const Queue& q) {
   if (a.pix_list) {
-    launch_chained(k_trace_list<OPAQUE, COUNT, KEY16, AO>, 152 * 4, kTraceThreads, s, a);
+    launch(k_trace_list<OPAQUE, COUNT, KEY16, AO>, 152 * 4, kTraceThreads, q, a);
     return;
   }
   const int tw = a.tile_w, th = a.tile_n / tw;
@@ -1144,17 +1144,17 @@ void launch_one(const TraceArgs& a, cudaStream_t s) {
   // compiled to keep resident
   const unsigned blocks = OPAQUE ? ((a.cam.width + 2 * tw - 1) / (2 * tw)) * ((a.cam.height + 2 * th - 1) / (2 * th))
                                  : 152 * (COUNT ? 4 : kMinBlocks<OPAQUE, COUNT, AO>);
-  launch_chained(k_trace_tile<OPAQUE, COUNT, KEY16, AO>, blocks, kTraceThreads, s, a);
+  launch(k_trace_tile<OPAQUE, COUNT, KEY16, AO>, blocks, kTraceThreads, q, a);
 }
 
 template <bool COUNT, bool KEY16>
-void launch_mode(const TraceArgs& a, int K, cudaStream_t s) {
-  if (K == 1) launch_one<true, COUNT, KEY16, false>(a, s);  // AO: k_shade_hits
-  else if (a.ao == 1) launch_one<false, COUNT, KEY16, true>(a, s);
-  else launch_one<false, COUNT, KEY16, false>(a, s);
+void launch_mode(const TraceArgs& a, int K, const Queue& q) {
+  if (K == 1) launch_one<true, COUNT, KEY16, false>(a, q);  // AO: k_shade_hits
+  else if (a.ao == 1) launch_one<false, COUNT, KEY16, true>(a, q);
+  else launch_one<false, COUNT, KEY16, false>(a, q);
 }
 
-int launch_trace(const TraceArgs& args, int K, cudaStream_t s) {
+int launch_trace(const TraceArgs& args, int K, const Queue& q) {
   TraceArgs a = args;
   a.tile_n = 32;
   if (K > 1) {
@@ -1168,11 +1168,11 @@ int launch_trace(const TraceArgs& args, int K, cudaStream_t s) {
     if (a.tile_n < 32) a.tile_w = a.tile_n == 16 ? 4 : 2;
   }
   if (a.count) {
-    if (a.key16) launch_mode<true, true>(a, K, s);
-    else launch_mode<true, false>(a, K, s);
+    if (a.key16) launch_mode<true, true>(a, K, q);
+    else launch_mode<true, false>(a, K, q);
   } else {
-    if (a.key16) launch_mode<false, true>(a, K, s);
-    else launch_mode<false, false>(a, K, s);
+    if (a.key16) launch_mode<false, true>(a, K, q);
+    else launch_mode<false, false>(a, K, q);
   }
   return 1;
 }
@@ -1201,9 +1201,9 @@ __global__ void __launch_bounds__(kTraceThreads) k_shade_hits(TraceArgs A) {
   *out = make_float4(A.alpha * c.x, A.alpha * c.y, A.alpha * c.z, v.w);
 }
 
-int launch_shade_hits(const TraceArgs& a, cudaStream_t s) {
+int launch_shade_hits(const TraceArgs& a, const Queue& q) {
   const dim3 grid((a.cam.width + 15) / 16, (a.cam.height + 7) / 8);
-  launch_chained(k_shade_hits, grid, kTraceThreads, s, a);
+  launch(k_shade_hits, grid, kTraceThreads, q, a);
   return 1;
 }
 
@@ -1221,10 +1221,10 @@ __global__ void k_touch_count(const uint32_t* bits, size_t words, unsigned long 
 
 int launch_touch_count(const uint32_t* list_bits, size_t list_words, const uint32_t* vert_bits,
                        size_t vert_words, const uint32_t* vox_bits, size_t vox_words,
-                       DevStatus* st, cudaStream_t s) {
-  launch_chained(k_touch_count, 152 * 4, 256, s, list_bits, list_words, &st->tr_u_entries);
-  launch_chained(k_touch_count, 152 * 4, 256, s, vert_bits, vert_words, &st->tr_u_vertices);
-  launch_chained(k_touch_count, 152 * 4, 256, s, vox_bits, vox_words, &st->tr_u_voxels);
+                       DevStatus* st, const Queue& q) {
+  launch(k_touch_count, 152 * 4, 256, q, list_bits, list_words, &st->tr_u_entries);
+  launch(k_touch_count, 152 * 4, 256, q, vert_bits, vert_words, &st->tr_u_vertices);
+  launch(k_touch_count, 152 * 4, 256, q, vox_bits, vox_words, &st->tr_u_voxels);
   return 3;
 }
 
@@ -1263,14 +1263,14 @@ __global__ void k_repair_clear(GridDev g, uint32_t* need, const uint32_t* vq, co
 }
 
 int launch_repair_alloc(const GridDev& g, const uint32_t* vq, const uint32_t* vq_cnt,
-                        const uint32_t* pq_cnt, uint32_t vq_cap, cudaStream_t s) {
-  launch_chained(k_repair_alloc, 152, 256, s, g, vq, vq_cnt, pq_cnt, vq_cap);
+                        const uint32_t* pq_cnt, uint32_t vq_cap, const Queue& q) {
+  launch(k_repair_alloc, 152, 256, q, g, vq, vq_cnt, pq_cnt, vq_cap);
   return 1;
 }
 
 int launch_repair_clear(const GridDev& g, uint32_t* need, const uint32_t* vq,
-                         const uint32_t* vq_cnt, uint32_t vq_cap, int next, cudaStream_t s) {
-  launch_chained(k_repair_clear, 152, 256, s, g, need, vq, vq_cnt, vq_cap, next);
+                         const uint32_t* vq_cnt, uint32_t vq_cap, int next, const Queue& q) {
+  launch(k_repair_clear, 152, 256, q, g, need, vq, vq_cnt, vq_cap, next);
   return 1;
 }
 

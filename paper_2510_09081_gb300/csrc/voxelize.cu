@@ -758,7 +758,7 @@ __global__ void __launch_bounds__(256) k_scatter_culled(GridDev g) {
 }
 
 int launch_pass1(const float4* pos, const float4* nrm, const uint32_t* order, long long V,
-                 const GridDev& g, cudaStream_t s) {
+                 const GridDev& g, const Queue& q) {
   if (V < 2) return 0;
   // One atomic per fragment at every grid side: summing the increments of the
   // lanes of a warp step that share a voxel first (a match on the voxel index)
@@ -767,16 +767,16 @@ int launch_pass1(const float4* pos, const float4* nrm, const uint32_t* order, lo
   // paid there while they returned nothing, 7.8 -> 7.4 ms).
   const int spw = pass1_segments_per_warp(V);
   const long long per_block = (long long)spw * kPass1Warps;
-  launch_chained(k_pass1, (unsigned)((V + per_block - 1) / per_block), kPass1Threads, s, pos, nrm, order, V,
+  launch(k_pass1, (unsigned)((V + per_block - 1) / per_block), kPass1Threads, q, pos, nrm, order, V,
                  spw, g);
-  launch_chained(k_exact1, 152 * 2, kExactThreads, s, pos, nrm, g);
+  launch(k_exact1, 152 * 2, kExactThreads, q, pos, nrm, g);
   return 2;
 }
 
 int launch_scatter(const GridDev& g, int mode, const uint32_t* need, const uint32_t* pending,
-                   cudaStream_t s) {
-  if (mode == 1) launch_chained(k_scatter_culled, 152 * 8, 256, s, g);
-  launch_chained(k_scatter, 152 * 8, 256, s, g, mode, need, pending);
+                   const Queue& q) {
+  if (mode == 1) launch(k_scatter_culled, 152 * 8, 256, q, g);
+  launch(k_scatter, 152 * 8, 256, q, g, mode, need, pending);
   return mode == 1 ? 2 : 1;
 }
 
