@@ -294,7 +294,12 @@ vrt_status vrt_read_shading(vrt_grid g, float* values_host, uint8_t* valid_host)
  * same voxel share each list entry's loads, so the best shape depends on the
  * scene and camera (vrt_tune_shapes measures it). The image does not depend on
  * it. Transparent images too small for such tiles to fill the GPU use tiles of
- * 16, 8 or 4 pixels of a fixed shape. */
+ * 16, 8 or 4 pixels of a fixed shape.
+ * VRT_OPT_TEST_TRACE_CALLS (12), for testing the limits of the trace's loops:
+ * value v in [1, 2^20) makes the trace give up a ray once it has walked through v
+ * bricks, cubes of empty bricks and occupied voxels, instead of after more than a
+ * ray can meet: vrt_sync then returns VRT_ERR_TIMEOUT, and the pixels given up
+ * hold what their rays had found. 0 restores the limit. */
 #define VRT_OPT_FORCE_EXACT 1
 #define VRT_OPT_STAGE_TIMING 2
 #define VRT_OPT_TRACE_COUNTERS 3
@@ -306,6 +311,7 @@ vrt_status vrt_read_shading(vrt_grid g, float* values_host, uint8_t* valid_host)
 #define VRT_OPT_TRACE_RAY_KEYS 9
 #define VRT_OPT_HIT_KEY 10
 #define VRT_OPT_TRACE_TILE 11
+#define VRT_OPT_TEST_TRACE_CALLS 12
 #define VRT_HIT_KEY_DEPTH_ID 0
 #define VRT_HIT_KEY_16_16 1
 #define VRT_MIPS_F32 0

@@ -99,6 +99,7 @@ struct vrt_grid_s {
   uint32_t ray_keys = 0xffffu;    // VRT_OPT_TRACE_RAY_KEYS (default: no limit of its own)
   int key16 = 0;                     // VRT_OPT_HIT_KEY
   int tile_w = 4;                    // VRT_OPT_TRACE_TILE
+  uint32_t trace_calls = 0;         // VRT_OPT_TEST_TRACE_CALLS (0: the trace's own limit)
   bool use_graph = false;
   cudaGraphExec_t graph_exec = nullptr;
   cudaStream_t cap_stream = nullptr;
@@ -856,6 +857,7 @@ vrt_status vrt_trace(vrt_grid g, const vrt_camera* cam, const vrt_render_params*
   a.ray_keys = g->ray_keys;
   a.key16 = g->key16;
   a.tile_w = g->tile_w;
+  a.max_calls = g->trace_calls;
   if (g->trace_counters) {  // touch bitmaps, cleared for this trace
     if (const vrt_status ts = size_touch_bitmaps(g)) return ts;
     VRT_CUDA(g, cudaMemsetAsync(g->touch_list, 0, g->touch_list_words * 4, g->stream));
@@ -924,6 +926,9 @@ vrt_status vrt_sync(vrt_grid g) {
   uint32_t e = hs.err;
   if (g->culled && hs.vq_cnt[kMaxRepairRounds & 1] != 0) e |= kErrRepair;
   if (hs.err) VRT_CUDA(g, cudaMemset(g->st, 0, sizeof(unsigned int)));
+  // a trace that ended before its repair did leaves voxels marked as queued
+  if (e & (kErrTimeout | kErrRepair))
+    VRT_CUDA(g, cudaMemsetAsync(g->need, 0, (size_t)g->n * g->n * g->n / 8, g->stream));
   if (e & kErrRange) return fail(g, VRT_ERR_INVALID_ARG, "device coordinates out of range or not finite");
   if (e & kErrOverflow) return fail(g, VRT_ERR_OVERFLOW, "a 16-bit voxel field or the list capacity overflowed");
   if (e & kErrTimeout) return fail(g, VRT_ERR_TIMEOUT, "a bounded device wait gave up");
@@ -1272,6 +1277,11 @@ vrt_status vrt_set_option(vrt_grid g, int32_t option, int64_t value) {
     if (value != 2 && value != 4 && value != 8 && value != 16)
       return fail(g, VRT_ERR_INVALID_ARG, "trace tile width must be 2, 4, 8 or 16");
     g->tile_w = (int)value;
+    return VRT_OK;
+  }
+  if (option == VRT_OPT_TEST_TRACE_CALLS) {
+    if (value < 0 || value >= (1ll << 20)) return fail(g, VRT_ERR_INVALID_ARG, "trace calls must be in [0, 2^20)");
+    g->trace_calls = (uint32_t)value;
     return VRT_OK;
   }
   if (option == VRT_OPT_HIT_KEY) {
