@@ -58,13 +58,14 @@ __global__ void __launch_bounds__(kTileThreads, 6) k_scan_noalloc(
   __shared__ uint32_t s_tile;
   __shared__ uint32_t s_prefix, s_sum;
   __shared__ uint32_t s_warp[kTileWarps];
-  dependency_wait();
+  const uint32_t zero = dependency_wait();
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   if (!CLUSTER) {
     if (tid == 0) s_tile = atomicAdd(&scratch->tile_counter, 1u);
     __syncthreads();
   }
-  const uint32_t tile = CLUSTER ? blockIdx.x : s_tile;
+  // the loads of words and marks, which may be read-only ones, wait through `zero`
+  const uint32_t tile = (CLUSTER ? blockIdx.x : s_tile) + zero;
   const bool some = !CLUSTER || tile < n_tiles;
   uint2 cnt[kTileRows];
   uint32_t sum[kTileRows], excl[kTileRows];
