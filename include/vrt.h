@@ -274,11 +274,11 @@ vrt_status vrt_read_shading(vrt_grid g, float* values_host, uint8_t* valid_host)
  * wrong (every list access stays bounded). -1 restores the normal scan. With
  * g == NULL it applies, process-wide, to vrt_scan_counts_noalloc (status bit
  * 0). No wait is left unbounded in either case.
- * VRT_OPT_TRACE_SHORT_LIST (8): value in [0, 1024] (not set: no limit): voxel
+ * VRT_OPT_TRACE_SHORT_LIST (8): value in [0, 1024], or -1 (default): no limit: voxel
  * lists up to this length share the warp entry by entry in the trace; longer ones
  * take the whole-warp path (one list at a time). The image does not depend on
  * it; for testing that path.
- * VRT_OPT_TRACE_RAY_KEYS (9): value in [1, 32] (not set: no limit): a transparent
+ * VRT_OPT_TRACE_RAY_KEYS (9): value in [1, 32], or -1 (default): no limit: a transparent
  * ray with more hits in one voxel takes the whole-warp path for it. The image
  * does not depend on it; for testing.
  * VRT_OPT_HIT_KEY (10): the order of the hits a ray composites within one

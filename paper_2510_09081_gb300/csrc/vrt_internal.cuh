@@ -22,6 +22,7 @@ constexpr int kMaxRepairRounds = 4;
 constexpr uint32_t kRayQueueLimit = 8;          // culled voxels one ray queues per round
 constexpr uint32_t kShortList = 1024;           // trace: largest limit of the shared-entry path's list length
 constexpr int kRayKeys = 32;                    // trace: largest limit of a ray's hits on that path
+constexpr uint32_t kNoLimit = 0xffffffu;        // neither: above any list's length and hits (16-bit counts)
 constexpr int kBrickDistMax = 15;               // cap of the empty-brick distance field
 constexpr int kMipsF32 = 0, kMipsF16 = 1, kMipsBF16 = 2;  // occupancy pyramid storage
 
