@@ -274,7 +274,7 @@ vrt_status vrt_read_shading(vrt_grid g, float* values_host, uint8_t* valid_host)
  * wrong (every list access stays bounded). -1 restores the normal scan. With
  * g == NULL it applies, process-wide, to vrt_scan_counts_noalloc (status bit
  * 0). No wait is left unbounded in either case.
- * VRT_OPT_TRACE_SHORT_LIST (8): value in [0, 1024], or -1 (default): no limit: voxel
+ * VRT_OPT_TRACE_SHORT_LIST (8): value in [0, 1024] (default 1024): voxel
  * lists up to this length share the warp entry by entry in the trace; longer ones
  * take the whole-warp path (one list at a time). The image does not depend on
  * it; for testing that path.
@@ -296,7 +296,7 @@ vrt_status vrt_read_shading(vrt_grid g, float* values_host, uint8_t* valid_host)
  * it. Transparent images too small for such tiles to fill the GPU use tiles of
  * 16, 8 or 4 pixels of a fixed shape.
  * VRT_OPT_TEST_TRACE_CALLS (12), for testing the limits of the trace's loops:
- * value v in [1, 2^20) makes the trace give up a ray once it has walked through v
+ * value v in [1, 2^13) makes the trace give up a ray once it has walked through v
  * bricks, cubes of empty bricks and occupied voxels, instead of after more than a
  * ray can meet: vrt_sync then returns VRT_ERR_TIMEOUT, and the pixels given up
  * hold what their rays had found. 0 restores the limit. */

@@ -95,8 +95,8 @@ struct vrt_grid_s {
   // frame is captured on (the legacy default stream cannot be captured)
   float cull_depth = 0.0f;  // VRT_OPT_CULL_DEPTH (0: the default threshold)
   int scan_stall = -1;      // VRT_OPT_TEST_SCAN_STALL (-1: off)
-  uint32_t short_list = kNoLimit;  // VRT_OPT_TRACE_SHORT_LIST
-  uint32_t ray_keys = kNoLimit;    // VRT_OPT_TRACE_RAY_KEYS
+  uint32_t short_list = kShortList;  // VRT_OPT_TRACE_SHORT_LIST
+  uint32_t ray_keys = kNoRayLimit;   // VRT_OPT_TRACE_RAY_KEYS
   int key16 = 0;                     // VRT_OPT_HIT_KEY
   int tile_w = 4;                    // VRT_OPT_TRACE_TILE
   uint32_t trace_calls = 0;         // VRT_OPT_TEST_TRACE_CALLS (0: the trace's own limit)
@@ -1268,9 +1268,9 @@ vrt_status vrt_set_option(vrt_grid g, int32_t option, int64_t value) {
   }
   if (!g) return fail(nullptr, VRT_ERR_INVALID_ARG, "grid is NULL");
   if (option == VRT_OPT_TRACE_SHORT_LIST) {
-    if (value < -1 || value > (int64_t)kShortList)
-      return fail(g, VRT_ERR_INVALID_ARG, "short-list limit must be in [0, 1024], or -1");
-    g->short_list = value < 0 ? kNoLimit : (uint32_t)value;
+    if (value < 0 || value > (int64_t)kShortList)
+      return fail(g, VRT_ERR_INVALID_ARG, "short-list limit must be in [0, 1024]");
+    g->short_list = (uint32_t)value;
     return VRT_OK;
   }
   if (option == VRT_OPT_TRACE_TILE) {
@@ -1280,7 +1280,7 @@ vrt_status vrt_set_option(vrt_grid g, int32_t option, int64_t value) {
     return VRT_OK;
   }
   if (option == VRT_OPT_TEST_TRACE_CALLS) {
-    if (value < 0 || value >= (1ll << 20)) return fail(g, VRT_ERR_INVALID_ARG, "trace calls must be in [0, 2^20)");
+    if (value < 0 || value >= (1ll << 13)) return fail(g, VRT_ERR_INVALID_ARG, "trace calls must be in [0, 2^13)");
     g->trace_calls = (uint32_t)value;
     return VRT_OK;
   }
@@ -1293,7 +1293,7 @@ vrt_status vrt_set_option(vrt_grid g, int32_t option, int64_t value) {
   if (option == VRT_OPT_TRACE_RAY_KEYS) {
     if (value != -1 && (value < 1 || value > kRayKeys))
       return fail(g, VRT_ERR_INVALID_ARG, "ray key slots must be in [1, 32], or -1");
-    g->ray_keys = value < 0 ? kNoLimit : (uint32_t)value;
+    g->ray_keys = value < 0 ? kNoRayLimit : (uint32_t)value;
     return VRT_OK;
   }
   if (option == VRT_OPT_FORCE_EXACT) {

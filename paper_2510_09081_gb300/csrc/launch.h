@@ -92,7 +92,7 @@ struct TraceArgs {
   int key16;                 // order hits by the paper's 16+16-bit per-voxel key
   int tile_w;                // warp tile width (2, 4, 8 or 16 pixels)
   int tile_n;                // rays a warp of the main trace owns (launch_trace sets it)
-  uint32_t max_calls;        // walk calls and parts after which a ray is given up (0: the
+  uint32_t max_calls;        // walk calls after which a ray is given up (0: the
                              // grid's limit; launch_trace shifts it to Ray::calls' place)
   int count;                 // accumulate trace work counters
   uint32_t* touch_list;      // instrumented trace: bit per list entry read

@@ -8,7 +8,7 @@
 // it. The warp then numbers the entries of its lanes' pending lists one after
 // another and takes them 64 at a time, so no lane idles on another lane's longer
 // list; rays waiting in the same voxel share an entry's loads. A list longer than
-// the test options allow, or (with the 16+16 key) more hits in a round than its
+// kShortList, or a voxel in which one ray has more hits than the warp's
 // shared-memory slots hold, goes to a whole-warp path that processes one voxel
 // at a time (lane l takes entries l, l+32, ...).
 //
@@ -69,19 +69,13 @@ constexpr int kTraceThreads = 128;
 constexpr uint32_t kPool = 192;
 constexpr uint32_t kRoundPairs = 1536;
 constexpr uint32_t kLost = 1u << 31;  // WarpMem::cnt: a hit of the ray found the pool full
-// Shortest part (voxels) of a voxel's interval that a ray whose hits found the pool
-// full takes by itself: below it, many hits at one depth (segments that share a
-// point) would be approached in ever smaller steps, and the whole-warp path takes
-// the rest at once.
-constexpr float kMinPart = 1.0f / 64.0f;
-// Limits of the trace's loops, so that none can run for ever whatever the data. A
-// ray counts its walk calls and its tries of parts in the upper 20 bits of
-// Ray::calls (the lower 12 count the voxels it queued, at most 3 n): past kMaxParts
-// it makes no more parts, and past TraceArgs::max_calls, more than any walk takes,
-// it is given up and vrt_sync reports the timeout. (With a register of its own for
-// the rounds of a warp sparse walks at 4K took 2.6% longer, so 0.8%.)
-constexpr uint32_t kCall = 1u << 12;
-constexpr uint32_t kMaxParts = 1u << 19;
+// Ray::calls: the culled voxels the ray queued (bits 0-10, at most 3 n); its hits
+// in the pending voxel, once counted (11-18); its walk calls (19-31). Past
+// TraceArgs::max_calls, more than any walk takes, a ray is given up and vrt_sync
+// reports the timeout, so that no loop of the trace can run for ever whatever the
+// data. (With a register of its own for the rounds of a warp sparse walks at 4K took
+// 2.6% longer, so 0.8%.)
+constexpr uint32_t kQueued = 2047u, kHits = 255u << 11, kCall = 1u << 19;
 // Rays that share an entry's loads. Lists are short (4 entries on average for
 // sparse walks, 24 for the bundles), so larger groups leave lanes without an
 // entry: groups of 32 take 0.55 ms where 4 take 0.43 on the opaque 1080p ABC
@@ -248,7 +242,7 @@ struct Ray {
   float tcur, t1, T;
   uint32_t pix, vox;   // pixel; pending voxel's word index
   uint32_t beg, len;   // pending voxel's list
-  uint32_t calls;      // walk calls and tries of parts, << 12; culled voxels queued
+  uint32_t calls;      // walk calls, hits in the pending voxel, culled voxels queued
   bool active, pending, missed;
 };
 
@@ -483,7 +477,7 @@ __device__ __forceinline__ void resolve_list(const TraceArgs& A, M& S, Ray& R) {
   if (COUNT) touch(A.touch_vox, idx);
   if (end0 >= kCulledStart) {
     // at the first culled voxel, keep the ray's state for the re-trace to resume from
-    if (R.calls % kCall == 0 && A.resume) {
+    if ((R.calls & kQueued) == 0 && A.resume) {
       const float4 c = S.acc[lane];
       A.resume[2 * R.pix] = make_float4(c.x, c.y, c.z, R.T);
       A.resume[2 * R.pix + 1] = make_float4(S.inv[lane].w, c.w, __uint_as_float(idx), S.o[lane].w);
@@ -497,7 +491,7 @@ __device__ __forceinline__ void resolve_list(const TraceArgs& A, M& S, Ray& R) {
     }
     R.missed = true;
     R.pending = false;
-    if (++R.calls % kCall >= A.max_queue || R.t1 < 0.0f) R.active = false;
+    if ((++R.calls & kQueued) >= A.max_queue || R.t1 < 0.0f) R.active = false;
     return;
   }
   if (end0 < cnt) {
@@ -662,11 +656,18 @@ __device__ __noinline__ float voxel_composite(const TraceArgs& A, WarpMem<false,
 // which gets the capsule test 32 at a time. A hit is shaded by the lane that
 // found it. An opaque ray keeps its nearest key; a transparent ray's hits go to
 // the warp's pool, where they are ranked by key for the ray's own lane to
-// composite. Rays join a round only while their lists sum to kRoundPairs pairs;
-// a ray with a hit that found the pool full takes its voxel again in parts of its
-// interval. `wait` is set for lanes whose voxel the next round takes; a lane left
-// pending without it (more than A.ray_keys hits, or the pool full with 16+16 keys)
-// goes to the whole-warp path, which starts its voxel again from scratch.
+// composite. Rays join a round only while their lists sum to kRoundPairs pairs. A
+// ray with a hit that found the pool full keeps the number of its hits, and the
+// next rounds take such rays only, as many as the pool holds the hits of: so each
+// takes its voxel once more. `wait` is set for lanes whose voxel a later round takes; a
+// lane left pending without it (a list past A.short_list, more hits than the pool or
+// A.ray_keys) goes to the whole-warp path, which starts its voxel again from
+// scratch.
+//
+// Where many rays have many hits in one voxel, what a full pool costs decides: 40,
+// 200, 1500 and 3000 tubes through one column of voxels, and 3000 at one place,
+// 640x480 pixels, alpha 0.3, took 0.31, 2.3, 24, 65 and 1329 ms with the voxel taken in
+// parts of its interval whenever the pool was full; 0.20, 0.66, 3.4, 4.6 and 5.5 so.
 template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
 __device__ __forceinline__ void process_flat(const TraceArgs& A, WarpMem<OPAQUE, KEY16>& S, Ray& R, Work& W,
                                              bool& wait) {
@@ -674,16 +675,21 @@ __device__ __forceinline__ void process_flat(const TraceArgs& A, WarpMem<OPAQUE,
   const unsigned lt = (1u << lane) - 1u;
   bool take = R.pending && R.len <= A.short_list;
   wait = false;
-  if (!OPAQUE && __reduce_add_sync(FULL, take ? R.len : 0u) > kRoundPairs) {
-    uint32_t sum = take ? R.len : 0u;
+  if (!OPAQUE) {
+    const bool again = __any_sync(FULL, (R.calls & kHits) != 0u);
+    const uint32_t need = !take ? 0u : (again ? (R.calls & kHits) >> 11 : R.len);
+    const uint32_t room = again ? kPool : kRoundPairs;
+    if (again || __reduce_add_sync(FULL, need) > room) {
+      uint32_t sum = need;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      const uint32_t v = __shfl_up_sync(FULL, sum, o);
-      if (lane >= o) sum += v;
-    }
-    if (take && sum - R.len >= kRoundPairs) {  // the next round's
-      take = false;
-      wait = true;
+      for (int o = 1; o < 32; o <<= 1) {
+        const uint32_t v = __shfl_up_sync(FULL, sum, o);
+        if (lane >= o) sum += v;
+      }
+      // a later round's: rays whose hits are not counted yet while others' are, and
+      // those past the room (the pool must hold all hits; the pairs may exceed theirs)
+      wait = take && (again ? need == 0u || sum > room : sum - need >= room);
+      take = take && !wait;
     }
   }
   // Lanes waiting in the same voxel (same list start) form groups of at most
@@ -881,16 +887,9 @@ __device__ __forceinline__ void process_flat(const TraceArgs& A, WarpMem<OPAQUE,
     const uint32_t raw = S.cnt[lane];
     redo = (raw & ~kLost) > A.ray_keys || (raw & kLost);
     if (take && redo) {
-      // Hits past the pool: the ray takes the voxel again up to a depth before
-      // which the pool should hold every ray's hits, and then the rest. (The
-      // 16+16 key quantizes depths over the whole interval, and a limit on a
-      // ray's hits asks for the whole-warp path.)
-      const float a = S.o[lane].w, b = S.d[lane].w;
-      const float m = fmaf(b - a, 0.4f * (float)kPool / (float)pn, a);
-      wait = !KEY16 && (raw & ~kLost) <= A.ray_keys && m - a >= kMinPart && m < b &&
-             R.calls < kMaxParts * kCall;
-      if (wait) R.calls += kCall;
-      S.d[lane].w = wait ? m : R.tcur;
+      const uint32_t mine = raw & ~kLost;
+      wait = mine <= min(A.ray_keys, kPool);
+      if (wait) R.calls |= mine << 11;
     }
     const uint32_t nk = redo ? 0u : raw;
     const uint32_t hits = min(pn, kPool);
@@ -949,16 +948,11 @@ __device__ __forceinline__ void process_flat(const TraceArgs& A, WarpMem<OPAQUE,
     }
   }
   if (!take || redo) return;
-  if (!KEY16 && R.T >= kTStop && S.d[lane].w < R.tcur) {  // the rest of the voxel's interval
-    S.o[lane].w = S.d[lane].w;
-    S.d[lane].w = R.tcur;
-    wait = true;
-    return;
-  }
   if (COUNT) {
     ++W.vox;
     W.entries += R.len;
   }
+  R.calls &= ~kHits;
   R.pending = false;
   if (R.T < kTStop || R.t1 < 0.0f) R.active = false;
 }
@@ -974,8 +968,8 @@ __device__ __forceinline__ void lap(unsigned long long& c, long long& t) {
 }
 
 // Trace the rays of the warp's lanes to their ends. Every round walks at least one
-// ray on or takes at least one ray's voxel to its end or the end of a part, so the
-// rays' limits bound the rounds.
+// ray on, and of the rounds over the warp's pending lists every one takes at least
+// one ray's list: to its end, to the count of its hits, or to the whole-warp path.
 template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
 __device__ __forceinline__ void trace_warp(const TraceArgs& A, WarpMem<OPAQUE, KEY16>& S, Ray& R, Work& W) {
   const int lane = threadIdx.x & 31;
@@ -1180,9 +1174,8 @@ int launch_trace(const TraceArgs& args, int K, const Queue& q) {
   TraceArgs a = args;
   a.tile_n = 32;
   // A ray's walk calls: one a brick and one an occupied voxel on its way, at most
-  // 3 n / 4 and 3 n, doubled for the voxel that a clamped crossing may step back;
-  // and its parts.
-  if (a.max_calls == 0) a.max_calls = kMaxParts + 8u * (uint32_t)a.g.n + 64u;
+  // 3 n / 4 and 3 n, doubled for the voxel that a clamped crossing may step back.
+  if (a.max_calls == 0) a.max_calls = 8u * (uint32_t)a.g.n + 64u;
   a.max_calls *= kCall;
   if (K > 1) {
     // A small image's tiles shrink until there are warps enough to fill the GPU:

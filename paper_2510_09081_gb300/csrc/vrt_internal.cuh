@@ -20,9 +20,10 @@ constexpr float kCoordMax = 768.0f;
 constexpr float kTStop = 1e-4f;                // transmittance where a ray stops
 constexpr int kMaxRepairRounds = 4;
 constexpr uint32_t kRayQueueLimit = 8;          // culled voxels one ray queues per round
-constexpr uint32_t kShortList = 1024;           // trace: largest limit of the shared-entry path's list length
+constexpr uint32_t kShortList = 1024;           // trace: longer lists go to the whole-warp path, which stops
+                                                // at the hits a ray needs (20000 tubes at one place 112 -> 35 ms)
 constexpr int kRayKeys = 32;                    // trace: largest limit of a ray's hits on that path
-constexpr uint32_t kNoLimit = 0xffffffu;        // neither: above any list's length and hits (16-bit counts)
+constexpr uint32_t kNoRayLimit = 0xffffu;       // no such limit (counts are 16 bits)
 constexpr int kBrickDistMax = 15;               // cap of the empty-brick distance field
 constexpr int kMipsF32 = 0, kMipsF16 = 1, kMipsBF16 = 2;  // occupancy pyramid storage
 

@@ -1,7 +1,6 @@
 """The limits of the trace's loops: a trace whose rays use up their walk calls ends and says so,
-and the next one is whole again; hits that share one depth, more than the warp's
-pool holds, leave the shared path for the whole-warp path after a bounded number
-of parts."""
+and the next one is whole again; hits that share one depth, as many as the warp's pool holds, more, and lists past
+the shared path's longest."""
 import numpy as np
 import pytest
 
@@ -39,7 +38,7 @@ def test_rays_that_are_given_up_are_reported(alpha, ao, cull, w, h):
         assert np.array_equal(a, b)
 
 
-@pytest.mark.parametrize("copies", [190, 200, 2000, 20000])
+@pytest.mark.parametrize("copies", [30, 190, 200, 1000, 1030, 2000, 20000])
 @pytest.mark.parametrize("alpha", [0.3, 0.02])
 def test_hits_at_one_depth(copies, alpha):
     # one tube along x, `copies` times: a ray down z hits all of them at one depth

@@ -1,5 +1,5 @@
 """The trace's testing limits (longest list and most hits on the shared path) can be
-set and taken back to the default, no limit."""
+set and taken back to the default."""
 import numpy as np
 import pytest
 
@@ -11,10 +11,10 @@ pytestmark = pytest.mark.gpu
 
 # tubes along x through the same voxels: opaque, lists longer than the limit; transparent,
 # more hits a ray than the limit, but fewer for the 4 rays of a tile than the pool holds
-@pytest.mark.parametrize("option,limit,refused,tubes,alpha", [
-    (vrt.OPT_TRACE_SHORT_LIST, 1024, (-2, 1025), 6000, 1.0),
-    (vrt.OPT_TRACE_RAY_KEYS, 8, (-2, 0, 33), 40, 0.02)])
-def test_limits_return_to_the_default(option, limit, refused, tubes, alpha):
+@pytest.mark.parametrize("option,limit,default_value,refused,tubes,alpha", [
+    (vrt.OPT_TRACE_SHORT_LIST, 5, 1024, (-1, 1025), 40, 1.0),
+    (vrt.OPT_TRACE_RAY_KEYS, 8, -1, (-2, 0, 33), 40, 0.02)])
+def test_limits_return_to_the_default(option, limit, default_value, refused, tubes, alpha):
     rng = np.random.default_rng(3)
     off = 16.5 + rng.uniform(-0.3, 0.3, (tubes, 1, 2))
     xyz = np.concatenate([np.tile([[[4.0], [28.0]]], (tubes, 1, 1)), np.tile(off, (1, 2, 1))], 2)
@@ -33,7 +33,7 @@ def test_limits_return_to_the_default(option, limit, refused, tubes, alpha):
     default = lists_taken_by_whole_warps()
     vrt.set_option(r.h, option, limit)
     limited = lists_taken_by_whole_warps()
-    vrt.set_option(r.h, option, -1)
+    vrt.set_option(r.h, option, default_value)
     again = lists_taken_by_whole_warps()
     for value in refused:
         with pytest.raises(vrt.VrtError) as e:
