@@ -351,7 +351,10 @@ vrt_status vrt_tune_grid_side(const vrt_grid_desc* base, const float* xyz, int32
  * vrt_tune_grid_side, for every grid side in `sides` and every tile width in
  * `tiles` (VRT_OPT_TRACE_TILE: 2, 4, 8 or 16); ms_out (nullable) receives
  * n_sides * n_tiles mean frame times, side-major (+inf where that pair could
- * not render the scene); *best_side and *best_tile the fastest pair. */
+ * not render the scene); *best_side and *best_tile the fastest pair. For a
+ * transparent image so small that the trace sets the shape itself
+ * (VRT_OPT_TRACE_TILE) a side is timed once, for all widths, and the first one
+ * is returned. */
 vrt_status vrt_tune_shapes(const vrt_grid_desc* base, const float* xyz, int32_t stride,
                            int64_t n_vertices, const int64_t* polyline_offsets,
                            int64_t n_polylines, const vrt_camera* cam, const vrt_render_params* p,

@@ -1193,7 +1193,13 @@ vrt_status vrt_tune_shapes(const vrt_grid_desc* base, const float* xyz, int32_t 
     vrt_grid g = nullptr;
     vrt_status r = vrt_create_grid(&d, nullptr, &g);
     if (r == VRT_OK) r = vrt_upload_segments(g, scaled.data(), 3, n_vertices, offsets, n_polylines, 0);
+    // where the trace sets the shape itself, one measurement is all widths'
+    const bool own_shape = p->alpha < 1.0f && transparent_tile_rays((long long)npx) < 32;
     for (int32_t j = 0; j < n_tiles; ++j) {
+      if (own_shape && j > 0) {
+        if (ms_out) ms_out[(size_t)i * n_tiles + j] = ms_out[(size_t)i * n_tiles];
+        continue;
+      }
       float ms = INFINITY;
       vrt_status rj = r;
       if (rj == VRT_OK) rj = vrt_set_option(g, VRT_OPT_TRACE_TILE, tiles[j]);

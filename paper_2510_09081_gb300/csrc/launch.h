@@ -174,6 +174,19 @@ int launch_mips(const GridDev& g, void* mips, int fmt, const long long* lev_off,
 int launch_cull(const GridDev& g, const HostCamera& cam, float alpha, uint8_t* eroded,
                 uint8_t* btmp, uint8_t* cdist, float* emean, float depth_max, uint32_t* occq,
                 unsigned long long occq_cap, const Queue& q);
+constexpr int kTraceThreads = 128;
+// Rays a warp's tile of the transparent trace holds, of an image of npx pixels: 32
+// in a shape of the caller's (TraceArgs::tile_w), fewer in a fixed one. A small
+// image's tiles shrink until there are warps enough to fill the GPU (5 blocks an SM):
+// a tile is a serial chain of rounds, and its units of work are entries, not
+// rays, so few rays still fill a warp's lanes (157x93 pixels at alpha 0.1:
+// 0.75 ms with 32 rays a tile, 0.46 with 16, 0.31 with 8, 0.22 with 4;
+// where tiles of 32 fill the GPU, 16 cost a third more).
+inline int transparent_tile_rays(long long npx) {
+  int n = 32;
+  while (n > 4 && npx / n < 152ll * 5 * (kTraceThreads / 32)) n >>= 1;
+  return n;
+}
 int launch_trace(const TraceArgs& a, int K, const Queue& q);
 // Cone AO of the hits an opaque trace (K = 1, a.ao = 1) and its repair rounds
 // left in a.rgba.

@@ -61,7 +61,6 @@ namespace vrt {
 
 constexpr unsigned FULL = 0xffffffffu;
 constexpr int kLaneKeys = 4;              // transparent, shared list: keys kept per lane per scan
-constexpr int kTraceThreads = 128;
 // Transparent: hits of a round that a warp's rays share (slots are bytes), and the
 // (ray, entry) pairs a round takes rays for. About 7% of the pairs of dense sets
 // give hits; 128 and 768 send more rays back for another pass (bundles at
@@ -81,8 +80,6 @@ constexpr uint32_t kQueued = 2047u, kHits = 255u << 11, kCall = 1u << 19;
 // entry: groups of 32 take 0.55 ms where 4 take 0.43 on the opaque 1080p ABC
 // view, and 3.37 against 3.30 on the bundles; single rays 0.46 and 3.73.
 constexpr int kGroup = 4;
-// Warps the GPU holds at the transparent trace's 5 blocks per SM.
-constexpr int kResidentWarps = 152 * 5 * (kTraceThreads / 32);
 
 // Instrumented trace: mark element i of a touch bitmap.
 __device__ __forceinline__ void touch(uint32_t* bits, uint32_t i) {
@@ -1178,13 +1175,7 @@ int launch_trace(const TraceArgs& args, int K, const Queue& q) {
   if (a.max_calls == 0) a.max_calls = 8u * (uint32_t)a.g.n + 64u;
   a.max_calls *= kCall;
   if (K > 1) {
-    // A small image's tiles shrink until there are warps enough to fill the GPU:
-    // a tile is a serial chain of rounds, and its units of work are entries, not
-    // rays, so few rays still fill a warp's lanes (157x93 pixels at alpha 0.1:
-    // 0.75 ms with 32 rays a tile, 0.46 with 16, 0.31 with 8, 0.22 with 4;
-    // where tiles of 32 fill the GPU, 16 cost a third more).
-    const long long npx = (long long)a.cam.width * a.cam.height;
-    while (a.tile_n > 4 && npx / a.tile_n < kResidentWarps) a.tile_n >>= 1;
+    a.tile_n = transparent_tile_rays((long long)a.cam.width * a.cam.height);
     if (a.tile_n < 32) a.tile_w = a.tile_n == 16 ? 4 : 2;
   }
   if (a.count) {
