@@ -600,11 +600,7 @@ vrt_status vrt_upload_segments(vrt_grid g, const float* xyz, int32_t stride, int
   unsigned long long cap = g->max_frag_desc ? g->max_frag_desc
                                             : (unsigned long long)(per * (double)std::max(V, 1ll));
   cap = std::min<unsigned long long>(cap, kCulledStart - 1ull);
-  // Pass 1 takes record slots for candidates, warp by warp; a small set's warps
-  // take fewer segments, so more of the unused slots fall inside the capacity:
-  // room for them.
-  unsigned long long rec_cap = cap;
-  if (pass1_segments_per_warp(V) < 32) rec_cap += std::min<unsigned long long>(4ull * cap, 1ull << 20);
+  const unsigned long long rec_cap = record_capacity(cap, V);
   if (cap != g->list_cap || rec_cap != g->rec_cap || !g->lists) {
     VRT_CUDA(g, cudaStreamSynchronize(g->stream));
     dfree(g, g->lists);

@@ -4,6 +4,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <algorithm>
+
 #include "vrt.h"
 #include "vrt_internal.cuh"
 
@@ -141,6 +143,12 @@ inline int pass1_segments_per_warp(long long V) {
   while (n > 4 && V / n < 152ll * kPass1Blocks) n >>= 1;
   return n;
 }
+// Fragment records held for a list capacity of `cap` entries. Pass 1 takes record
+// slots for candidates, warp by warp; a small set's warps take fewer segments, so
+// more of the unused slots fall inside the capacity: room for them.
+inline unsigned long long record_capacity(unsigned long long cap, long long V) {
+  return cap + (pass1_segments_per_warp(V) < 32 ? std::min<unsigned long long>(4ull * cap, 1ull << 20) : 0ull);
+}
 // Pass 1 over the segments in the order `order` (V vertex indices, each
 // polyline's vertices consecutive; a polyline's last vertex starts no
 // segment), or in index order when `order` is null.
@@ -212,6 +220,9 @@ const char* frame_args_error(const vrt_camera* cam, const vrt_render_params* p);
 // that the frame's calls allocate nothing and can be captured into a CUDA
 // graph (may synchronize the grid's stream).
 vrt_status prepare_frame(vrt_grid g, const vrt_camera* cam, const vrt_render_params* p);
+// Estimated device bytes of a grid of this side with n_vertices vertices, segments of
+// mean length mean_len, and every buffer its frames can need.
+uint64_t set_bytes(int side, float radius, uint64_t max_fragments, int64_t n_vertices, double mean_len);
 
 // Testing hook of vrt_scan_counts_noalloc (vrt_set_option(NULL,
 // VRT_OPT_TEST_SCAN_STALL, tile)): tile >= 0 makes that look-back tile skip

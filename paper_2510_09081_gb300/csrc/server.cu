@@ -106,6 +106,22 @@ struct vrt_server_s {
   uint64_t batches = 0, batched_frames = 0;
 };
 
+// Footprint estimate of a set before it has been resident (its measured size
+// replaces it afterwards), its frames culled, shaded and of 1080p: a set that needs
+// more than was reserved for it would take the resident ones past the budget.
+uint64_t vrt::set_bytes(int side, float radius, uint64_t max_fragments, int64_t n_vertices, double mean_len) {
+  const uint64_t n = (uint64_t)side, nv = n * n * n, V = (uint64_t)std::max<int64_t>(n_vertices, 1);
+  const double rl = radius + 1.0 / 512.0;
+  const double per = std::max(16.0, 0.9 * (mean_len + 2 * rl + 2) * (2 * rl + 2) * (2 * rl + 2));
+  const uint64_t cap = max_fragments ? max_fragments : (uint64_t)(per * V);
+  const uint64_t xq = std::max<uint64_t>(4 * V, 1ull << 22);
+  // words, cursors, marks, fields, brick masks, pyramid; vertices and their order;
+  // lists; records and ranks; exact queue; cull scratch; voxel-space shading field and
+  // mask; pixel queues at 1080p; the status and the arrays' ends
+  return nv * 17 + nv / 4 + nv / 8 + V * (45 + 4) + cap * 4 + vrt::record_capacity(cap, n_vertices) * 10 + xq * 8 +
+         nv * 5 + nv * 4 + nv / 8 + 2073600ull * 40 + (64u << 10);
+}
+
 namespace {
 
 // Failures of server calls report through vrt_last_error(NULL), whose message
@@ -115,32 +131,20 @@ vrt_status sfail(vrt_server, vrt_status st, const std::string& m) {
   return st;
 }
 
-// Footprint estimate of a set before it has been resident (its measured size
-// replaces it afterwards): the grid's voxel arrays, vertex buffers, list and
-// record capacity, exact queue, pyramid, cull and repair scratch at 1080p.
 uint64_t estimate_bytes(const ServerSet& st) {
-  const uint64_t n = (uint64_t)st.desc.n, nv = n * n * n, V = (uint64_t)std::max<int64_t>(st.V, 1);
-  const double rl = st.desc.radius + 1.0 / 512.0;
   double mean_len = 1.0;
-  {
-    double sum = 0;
-    int64_t cnt = 0;
-    for (int64_t p = 0; p < st.P; ++p)
-      for (int64_t i = st.offsets[p]; i + 1 < st.offsets[p + 1]; i += 64) {
-        const float* a = &st.xyz[3 * i];
-        const float* b = &st.xyz[3 * (i + 1)];
-        sum += std::sqrt((double)(b[0] - a[0]) * (b[0] - a[0]) + (double)(b[1] - a[1]) * (b[1] - a[1]) +
-                         (double)(b[2] - a[2]) * (b[2] - a[2]));
-        ++cnt;
-      }
-    if (cnt) mean_len = sum / cnt;
-  }
-  const double per = std::max(16.0, 0.9 * (mean_len + 2 * rl + 2) * (2 * rl + 2) * (2 * rl + 2));
-  const uint64_t cap = st.desc.max_fragments ? st.desc.max_fragments : (uint64_t)(per * V);
-  const uint64_t xq = std::max<uint64_t>(4 * V, 1ull << 22);
-  // words, cursors, marks, fields, pyramid; vertices; lists, records and ranks;
-  // exact queue; cull scratch; voxel-space shading field and mask; pixel queues at 1080p
-  return nv * 17 + nv / 4 + V * 45 + cap * 14 + xq * 8 + nv * 5 + nv * 4 + nv / 8 + 2073600ull * 40;
+  double sum = 0;
+  int64_t cnt = 0;
+  for (int64_t p = 0; p < st.P; ++p)
+    for (int64_t i = st.offsets[p]; i + 1 < st.offsets[p + 1]; i += 64) {
+      const float* a = &st.xyz[3 * i];
+      const float* b = &st.xyz[3 * (i + 1)];
+      sum += std::sqrt((double)(b[0] - a[0]) * (b[0] - a[0]) + (double)(b[1] - a[1]) * (b[1] - a[1]) +
+                       (double)(b[2] - a[2]) * (b[2] - a[2]));
+      ++cnt;
+    }
+  if (cnt) mean_len = sum / cnt;
+  return vrt::set_bytes(st.desc.n, st.desc.radius, st.desc.max_fragments, st.V, mean_len);
 }
 
 void CUDART_CB on_frame_done(void* arg) {
