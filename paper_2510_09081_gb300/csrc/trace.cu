@@ -503,14 +503,15 @@ __device__ __forceinline__ void resolve_list(const TraceArgs& A, M& S, Ray& R) {
 }
 
 // An opaque ray ends at its nearest hit. With cone AO its pixel carries the hit
-// (segment id and depth) to k_shade_hits, which writes the colour; otherwise it
-// is shaded here.
+// (segment id and depth, kHitTag) to k_shade_hits, which writes the colour; otherwise
+// it is shaded here.
+constexpr uint32_t kHitTag = 0x7fc0a05cu;  // a NaN: no colour holds it
 template <class M>
 __device__ __forceinline__ void opaque_hit(const TraceArgs& A, M& S, Ray& R, uint32_t id, float t) {
   const int lane = threadIdx.x & 31;
   float3 c;
   if (A.ao == 1) {
-    c = make_float3(__uint_as_float(id), t, 0.0f);
+    c = make_float3(__uint_as_float(id), t, __uint_as_float(kHitTag));
   } else {
     c = tangent_colour(f3(__ldg(&A.pos[id])), f3(__ldg(&A.pos[id + 1])));
     if (A.ao) c = field_shade(A, f3(S.o[lane]) + t * f3(S.d[lane])) * c;
@@ -1201,9 +1202,10 @@ __global__ void __launch_bounds__(kTraceThreads) k_shade_hits(TraceArgs A) {
   if (px >= A.cam.width || py >= A.cam.height) return;
   float4* out = &A.rgba[(size_t)py * A.cam.width + px];
   const float4 v = *out;
-  if (v.w == 0.0f) return;  // no hit: transparent black
+  // no hit (transparent black), or a pixel that the repair left unfinished (vrt_sync
+  // reports it): it holds what the caller's image held
+  if (__float_as_uint(v.z) != kHitTag) return;
   const uint32_t id = __float_as_uint(v.x);
-  // a pixel the repair left unfinished (vrt_sync reports it) holds no hit
   if (id >= A.n_vert || id + 1 >= A.n_vert) return;
   float3 o, d;
   pixel_ray(A.cam, px, py, o, d);
