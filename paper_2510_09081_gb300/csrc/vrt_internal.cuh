@@ -167,7 +167,10 @@ __device__ __forceinline__ float cmp3(float3 a, int k) { return k == 0 ? a.x : (
 // segment nearest the box's centre. Stage 2 runs Newton steps on the convex, C^1,
 // piecewise-quadratic squared box distance f(t) and brackets its minimum: f(t) is
 // an upper bound, and convexity gives f(t) - |f'(t)| * (t or 1 - t) as a lower
-// bound, for any t. What is still too close to call goes to the exact decision.
+// bound, for any t. (The distance to the steps' bracket instead of t or 1 - t would
+// rest on the rounded signs of earlier derivatives, and decides no more: 24.418
+// against 24.427% of 26M pairs near the list radius are left.) What is still too
+// close to call goes to the exact decision.
 // Rounding allowance of stage 2 for local coordinates a, a + d.
 __device__ __forceinline__ float seg_box_tol(float3 a, float3 d) {
   const float M = fmaxf(fmaxf(fmaxf(fabsf(a.x), fabsf(a.y)), fabsf(a.z)),
@@ -211,7 +214,7 @@ __device__ __forceinline__ int seg_box_stage2(float3 a, float3 d, float rl) {
       if (e != 0.0f) gp = fmaf(dk, dk, gp);
     }
     if (f + tol <= rl2) return 1;
-    const float lb = f - 2.0f * fabsf(g) * (g > 0.0f ? t - br.lo : br.hi - t);
+    const float lb = f - 2.0f * fabsf(g) * (g > 0.0f ? t : 1.0f - t);
     if (lb - tol > rl2) return 0;
     if (gp == 0.0f) break;
     t = br.next(t, g, gp);
