@@ -278,9 +278,9 @@ vrt_status vrt_read_shading(vrt_grid g, float* values_host, uint8_t* valid_host)
  * lists up to this length share the warp entry by entry in the trace; longer ones
  * take the whole-warp path (one list at a time). The image does not depend on
  * it; for testing that path.
- * VRT_OPT_TRACE_RAY_KEYS (9): value in [1, 32], or -1 (default): no limit: a transparent
- * ray with more hits in one voxel takes the whole-warp path for it. The image
- * does not depend on it; for testing.
+ * VRT_OPT_TRACE_RAY_KEYS (9): value in [1, 32], or -1 (default): a transparent ray
+ * with more hits in one voxel (-1: than the warp's 192 slots) takes the whole-warp
+ * path for it. The image does not depend on it; for testing.
  * VRT_OPT_HIT_KEY (10): the order of the hits a ray composites within one
  * voxel (Sec. 3.5). VRT_HIT_KEY_DEPTH_ID (default): by depth in fp32, equal
  * depths by segment id -- the ground-truth order, independent of how the list

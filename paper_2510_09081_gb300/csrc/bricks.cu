@@ -61,7 +61,7 @@ __global__ void __launch_bounds__(256) k_reset(uint32_t* a, uint32_t na, uint32_
 
 int launch_reset(uint32_t* a, uint32_t na, uint32_t* b, uint32_t nb, const Queue& q) {
   const unsigned blocks = (na + nb + 1023) / 1024;
-  launch(k_reset, blocks < 152u ? blocks : 152u, 256, q, a, na, b, nb);
+  launch(k_reset, blocks < kSms ? blocks : kSms, 256, q, a, na, b, nb);
   return 1;
 }
 

@@ -140,7 +140,7 @@ constexpr int kPass1Blocks = 9;  // resident per SM: 56 registers, 24 KB of shar
 // of 7 0.050, 0.046, 0.048; at 98k it no longer pays (0.044 with 32, 0.047 with 16).
 inline int pass1_segments_per_warp(long long V) {
   int n = 32;
-  while (n > 4 && V / n < 152ll * kPass1Blocks) n >>= 1;
+  while (n > 4 && V / n < (long long)kSms * kPass1Blocks) n >>= 1;
   return n;
 }
 // Fragment records held for a list capacity of `cap` entries. Pass 1 takes record
@@ -192,7 +192,7 @@ constexpr int kTraceThreads = 128;
 // where tiles of 32 fill the GPU, 16 cost a third more).
 inline int transparent_tile_rays(long long npx) {
   int n = 32;
-  while (n > 4 && npx / n < 152ll * 5 * (kTraceThreads / 32)) n >>= 1;
+  while (n > 4 && npx / n < (long long)kSms * 5 * (kTraceThreads / 32)) n >>= 1;
   return n;
 }
 int launch_trace(const TraceArgs& a, int K, const Queue& q);

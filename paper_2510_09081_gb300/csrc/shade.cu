@@ -149,7 +149,7 @@ int launch_shade(const ShadeArgs& a, const Queue& q) {
 }
 
 int launch_shade_repair(const ShadeArgs& a, const Queue& q) {
-  launch(k_shade_repair, 152, 256, q, a);
+  launch(k_shade_repair, kSms, 256, q, a);
   return 1;
 }
 

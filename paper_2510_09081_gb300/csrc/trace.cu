@@ -1073,7 +1073,8 @@ __device__ __forceinline__ void write_pixel(const TraceArgs& A, const M& S, cons
 }
 
 // Resident blocks per SM the trace kernels are compiled for: 96 registers for
-// the transparent trace (6 blocks at 80 spill: sparse walks at 4K 25.8 ms against
+// the transparent trace, which spills 28 bytes of stores and 36 of loads at that (6
+// blocks, at 80 registers, spill far more: sparse walks at 4K 25.8 ms against
 // 20.8; 4 blocks 24.6), 72 for the opaque one.
 template <bool OPAQUE, bool COUNT, bool AO>
 constexpr int kMinBlocks = COUNT ? 1 : (OPAQUE ? 6 : (AO ? 4 : 5));
@@ -1150,14 +1151,14 @@ __global__ void __launch_bounds__(kTraceThreads, kMinBlocks<OPAQUE, COUNT, AO>) 
 template <bool OPAQUE, bool COUNT, bool KEY16, bool AO>
 void launch_one(const TraceArgs& a, const Queue& q) {
   if (a.pix_list) {
-    launch(k_trace_list<OPAQUE, COUNT, KEY16, AO>, 152 * 4, kTraceThreads, q, a);
+    launch(k_trace_list<OPAQUE, COUNT, KEY16, AO>, kSms * 4, kTraceThreads, q, a);
     return;
   }
   const int tw = a.tile_w, th = a.tile_n / tw;
   // opaque: a block per 2x2 tiles; transparent: as many blocks as the kernel is
   // compiled to keep resident
   const unsigned blocks = OPAQUE ? ((a.cam.width + 2 * tw - 1) / (2 * tw)) * ((a.cam.height + 2 * th - 1) / (2 * th))
-                                 : 152 * (COUNT ? 4 : kMinBlocks<OPAQUE, COUNT, AO>);
+                                 : kSms * (COUNT ? 4 : kMinBlocks<OPAQUE, COUNT, AO>);
   launch(k_trace_tile<OPAQUE, COUNT, KEY16, AO>, blocks, kTraceThreads, q, a);
 }
 
@@ -1235,9 +1236,9 @@ __global__ void k_touch_count(const uint32_t* bits, size_t words, unsigned long 
 int launch_touch_count(const uint32_t* list_bits, size_t list_words, const uint32_t* vert_bits,
                        size_t vert_words, const uint32_t* vox_bits, size_t vox_words,
                        DevStatus* st, const Queue& q) {
-  launch(k_touch_count, 152 * 4, 256, q, list_bits, list_words, &st->tr_u_entries);
-  launch(k_touch_count, 152 * 4, 256, q, vert_bits, vert_words, &st->tr_u_vertices);
-  launch(k_touch_count, 152 * 4, 256, q, vox_bits, vox_words, &st->tr_u_voxels);
+  launch(k_touch_count, kSms * 4, 256, q, list_bits, list_words, &st->tr_u_entries);
+  launch(k_touch_count, kSms * 4, 256, q, vert_bits, vert_words, &st->tr_u_vertices);
+  launch(k_touch_count, kSms * 4, 256, q, vox_bits, vox_words, &st->tr_u_voxels);
   return 3;
 }
 
@@ -1277,13 +1278,13 @@ __global__ void k_repair_clear(GridDev g, uint32_t* need, const uint32_t* vq, co
 
 int launch_repair_alloc(const GridDev& g, const uint32_t* vq, const uint32_t* vq_cnt,
                         const uint32_t* pq_cnt, uint32_t vq_cap, const Queue& q) {
-  launch(k_repair_alloc, 152, 256, q, g, vq, vq_cnt, pq_cnt, vq_cap);
+  launch(k_repair_alloc, kSms, 256, q, g, vq, vq_cnt, pq_cnt, vq_cap);
   return 1;
 }
 
 int launch_repair_clear(const GridDev& g, uint32_t* need, const uint32_t* vq,
                          const uint32_t* vq_cnt, uint32_t vq_cap, int next, const Queue& q) {
-  launch(k_repair_clear, 152, 256, q, g, need, vq, vq_cnt, vq_cap, next);
+  launch(k_repair_clear, kSms, 256, q, g, need, vq, vq_cnt, vq_cap, next);
   return 1;
 }
 

@@ -769,14 +769,14 @@ int launch_pass1(const float4* pos, const float4* nrm, const uint32_t* order, lo
   const long long per_block = (long long)spw * kPass1Warps;
   launch(k_pass1, (unsigned)((V + per_block - 1) / per_block), kPass1Threads, q, pos, nrm, order, V,
                  spw, g);
-  launch(k_exact1, 152 * 2, kExactThreads, q, pos, nrm, g);
+  launch(k_exact1, kSms * 2, kExactThreads, q, pos, nrm, g);
   return 2;
 }
 
 int launch_scatter(const GridDev& g, int mode, const uint32_t* need, const uint32_t* pending,
                    const Queue& q) {
-  if (mode == 1) launch(k_scatter_culled, 152 * 8, 256, q, g);
-  launch(k_scatter, 152 * 8, 256, q, g, mode, need, pending);
+  if (mode == 1) launch(k_scatter_culled, kSms * 8, 256, q, g);
+  launch(k_scatter, kSms * 8, 256, q, g, mode, need, pending);
   return mode == 1 ? 2 : 1;
 }
 

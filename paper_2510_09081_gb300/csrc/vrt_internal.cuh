@@ -25,6 +25,7 @@ constexpr uint32_t kShortList = 1024;           // trace: longer lists go to the
 constexpr int kRayKeys = 32;                    // trace: largest limit of a ray's hits on that path
 constexpr uint32_t kNoRayLimit = 0xffffu;       // no such limit (counts are 16 bits)
 constexpr int kBrickDistMax = 15;               // cap of the empty-brick distance field
+constexpr unsigned kSms = 152;                  // of a GB300: sizes grids of resident blocks (no result depends on it)
 constexpr int kMipsF32 = 0, kMipsF16 = 1, kMipsBF16 = 2;  // occupancy pyramid storage
 
 // per-vertex flag bits, stored in pos[i].w as raw bits
