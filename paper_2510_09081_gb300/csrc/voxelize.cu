@@ -301,7 +301,8 @@ __device__ __forceinline__ void flush_culled(const GridDev& g, unsigned long lon
 // offset from the voxel centre and their distance serve the occupancy too (Alg. 2
 // measures the same point). Records of 128 bytes put all lanes' loads on the
 // same banks (72% of the shared-memory pipe); 144 bytes do not. Bundles (114M
-// fragments, 256^3) 2.40 -> 1.74 ms, ABC flow (195M, 512^3) 4.71 -> 3.71 ms; without
+// fragments, 256^3) 2.40 -> 1.74 ms, ABC flow (195M, 512^3) 4.71 -> 3.71 ms (1.65 and
+// 3.42 with the bracketed Newton steps and pairs of floats that came after); without
 // the atomics 10% less, so they are not what bounds it.
 __global__ void __launch_bounds__(kPass1Threads, kPass1Blocks) k_pass1(const float4* __restrict__ pos,
                                                   const float4* __restrict__ nrm,
