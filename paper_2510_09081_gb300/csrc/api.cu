@@ -116,22 +116,35 @@ thread_local std::string g_create_error;
 
 namespace vrt {
 namespace {
-std::mutex g_streams_mu;
-std::map<cudaStream_t, long long> g_streams;  // grids on each stream
+struct Streams {
+  std::mutex mu;
+  std::map<cudaStream_t, long long> users;  // grids and servers on each stream
+  bool lost = false;                        // one could not be entered (host memory): none is alone
+};
+// Never destroyed: a server's thread may still run when the process ends.
+Streams& streams() {
+  static Streams* const s = new Streams;
+  return *s;
+}
 }  // namespace
 
 void stream_enter(cudaStream_t s) {
-  std::lock_guard<std::mutex> lk(g_streams_mu);
-  ++g_streams[s];
+  std::lock_guard<std::mutex> lk(streams().mu);
+  try {
+    ++streams().users[s];
+  } catch (...) {
+    streams().lost = true;
+  }
 }
 void stream_leave(cudaStream_t s) {
-  std::lock_guard<std::mutex> lk(g_streams_mu);
-  const auto it = g_streams.find(s);
-  if (it != g_streams.end() && --it->second == 0) g_streams.erase(it);
+  std::lock_guard<std::mutex> lk(streams().mu);
+  const auto it = streams().users.find(s);
+  if (it != streams().users.end() && --it->second == 0) streams().users.erase(it);
 }
 bool stream_alone(cudaStream_t s) {
-  std::lock_guard<std::mutex> lk(g_streams_mu);
-  return g_streams.empty() || (g_streams.size() == 1 && g_streams.begin()->first == s);
+  std::lock_guard<std::mutex> lk(streams().mu);
+  const auto& u = streams().users;
+  return !streams().lost && (u.empty() || (u.size() == 1 && u.begin()->first == s));
 }
 }  // namespace vrt
 
